@@ -15,7 +15,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libeclqr.so")
 SOURCES = ["k_primal.cu", "k_lqr.cu", "k_dual.cu", "k_grad.cu", "k_refine.cu", "k_mixed.cu", "api.cu", "noalloc.cu"]
-HEADERS = ["la.cuh", "plan.cuh", "kernels.cuh", os.path.join("..", "..", "include", "eclqr.h")]
+HEADERS = ["la.cuh", "fx.cuh", "plan.cuh", "kernels.cuh", os.path.join("..", "..", "include", "eclqr.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall"]
 

@@ -86,51 +86,55 @@ namespace {
 // opt.team_warps != 0 fixes it for every kernel.  Otherwise a launch with fewer
 // tasks than SMs takes four warps, one per SM sub-partition, so that one task
 // spreads over the SM; one with at least kManyTasksPerSm tasks per SM takes the
-// kernel's entry below, and one in between the entry but at least two warps.  There the SM is filled by many tasks at once, and an FP64 warp
+// kernel's entry below; and one in between takes the entry but at least two
+// warps, or the kernel's own count for that range.  With many tasks the SM is
+// filled by many at once, and an FP64 warp
 // instruction costs its sub-partition the same time whatever its active lanes,
 // so the sequential per-problem sweeps and the small per-stage kernels run
 // fastest as one warp per task: one warp forms each reflector's scalars, each
 // reduction and each triangular solve once, where four warps would each repeat
 // them, and needs no CTA barrier.  The entries are the fastest team measured per
 // kernel and state dimension on the 4096-problem uneven batch (each (n, m) group
-// alone, about seven problems per SM).  For example the Riccati sweep takes 247
-// ms over the four groups with one warp per problem against 320 ms with four
-// (at n = 24, 86 ms with two warps against 93 with one); the affine chains take
+// alone, about seven problems per SM).  For example the affine chains take
 // 4 ms with two warps at n = 8 against 7 with eight, but 7 ms with eight at
 // n = 24 against 11 with two; the chunk up-sweeps of the long horizon (65536
 // stages in 1024 chunks) take 27 ms with two warps per chunk against 37 with one;
 // the stage elimination takes 14 ms with one warp at n = 8 against 29 ms with
 // four, but 86 ms with four at n = 24 against 120 ms with one, where its stage
-// matrices fill four warps.
+// matrices fill four warps.  The Riccati sweep's products have thousands of
+// independent integer multiply-adds per stage from n = 16 on: 48 stages of 1280
+// problems take 1.44 / 1.48 / 1.65 ms with 1 / 2 / 4 warps at n = 8, 2.56 / 2.09 /
+// 2.23 at n = 12, 3.85 / 3.40 / 3.09 at n = 16 and 8.49 / 6.00 / 5.86 at n = 24; with
+// 320 problems four warps are best at every n (0.60 against 0.71 ms with one at
+// n = 8, 2.6 against 4.7 at n = 24).
 int team_for(const eclqr_handle *h, const void *kern, int ntasks, int n) {
   if (h->opt.team_warps != 0) return h->opt.team_warps;
   if (ntasks < h->sms) return kTeamWarps;
-  // warps below n_from, and from n_from up
-  static const struct { const void *fn; int warps, n_from, warps_from; } table[] = {
-      {(const void *)k_riccati_down, 1, 24, 2},  {(const void *)k_riccati_down_f32, 1, 0, 1},
-      {(const void *)k_riccati_finish, 1, 0, 1}, {(const void *)k_elim, 1, 16, 4},
-      {(const void *)k_primal_down, 1, 24, 2},   {(const void *)k_dual_down, 1, 0, 1},
-      {(const void *)k_primal_stage, 1, 24, 2},
-      {(const void *)k_aff_down, 2, 24, 8},      {(const void *)k_dual_leaf, 1, 0, 1},
-      {(const void *)k_aff_prep, 1, 0, 1},       {(const void *)k_stage_lists, 1, 0, 1},
-      {(const void *)k_dual_stage, 2, 0, 2},     {(const void *)k_param, 1, 0, 1},
-      {(const void *)k_resid, 1, 0, 1},          {(const void *)k_pcorr, 1, 0, 1},
-      {(const void *)k_kkt, 1, 0, 1},            {(const void *)k_post_roll, 1, 0, 1},
-      {(const void *)k_recover, 1, 0, 1},        {(const void *)k_check_inputs, 1, 0, 1},
-      {(const void *)k_refine_trial, 1, 0, 1},   {(const void *)k_refine_accept, 1, 0, 1},
-      {(const void *)k_refine_prep, 1, 0, 1},    {(const void *)k_refine_gate, 1, 0, 1},
-      {(const void *)k_refine_parts, 1, 0, 1},   {(const void *)k_refine_post, 1, 0, 1},
-      {(const void *)k_rescue_prep, 1, 0, 1},    {(const void *)k_scan_check, 1, 0, 1},
-      {(const void *)k_terminal, 1, 0, 1},       {(const void *)k_dual_terminal, 1, 0, 1},
-      {(const void *)k_lqr_up, 2, 0, 2},         {(const void *)k_primal_up, 1, 0, 1},
-      {(const void *)k_dual_up, 2, 0, 2}};
+  // warps below n1, from n1 up and from n2 up; few: warps with one to four tasks per SM (0: the
+  // entry, at least two -- 256 problems of 256 stages, n = 16: 37 ms with two, 42 with one, 49 with four)
+  static const struct { const void *fn; int warps, n1, warps1, n2, warps2, few; } table[] = {
+      {(const void *)k_riccati_down, 1, 12, 2, 16, 4, 4},
+      {(const void *)k_riccati_down_f32, 1},     {(const void *)k_riccati_finish, 1},
+      {(const void *)k_elim, 1, 16, 4},          {(const void *)k_primal_down, 1, 24, 2},
+      {(const void *)k_dual_down, 1},            {(const void *)k_primal_stage, 1, 24, 2},
+      {(const void *)k_aff_down, 2, 24, 8},      {(const void *)k_dual_leaf, 1},
+      {(const void *)k_aff_prep, 1},             {(const void *)k_stage_lists, 1},
+      {(const void *)k_dual_stage, 2},           {(const void *)k_param, 1},
+      {(const void *)k_resid, 1},                {(const void *)k_pcorr, 1},
+      {(const void *)k_kkt, 1},                  {(const void *)k_post_roll, 1},
+      {(const void *)k_recover, 1},              {(const void *)k_check_inputs, 1},
+      {(const void *)k_refine_trial, 1},         {(const void *)k_refine_accept, 1},
+      {(const void *)k_refine_prep, 1},          {(const void *)k_refine_gate, 1},
+      {(const void *)k_refine_parts, 1},         {(const void *)k_refine_post, 1},
+      {(const void *)k_rescue_prep, 1},          {(const void *)k_scan_check, 1},
+      {(const void *)k_terminal, 1},             {(const void *)k_dual_terminal, 1},
+      {(const void *)k_lqr_up, 2},               {(const void *)k_primal_up, 1},
+      {(const void *)k_dual_up, 2}};
   const bool many = ntasks >= kManyTasksPerSm * h->sms;
   for (const auto &e : table)
     if (e.fn == kern) {
-      const int w = n >= e.n_from ? e.warps_from : e.warps;
-      // one to four tasks per SM: a one-warp entry takes two warps (256 problems of 256
-      // stages, n = 16: 37 ms with two, 42 with one, 49 with four)
-      return many ? w : std::max(w, 2);
+      const int w = e.n2 && n >= e.n2 ? e.warps2 : (e.n1 && n >= e.n1 ? e.warps1 : e.warps);
+      return many ? w : (e.few ? e.few : std::max(w, 2));
     }
   return kTeamWarps;
 }

@@ -10,7 +10,7 @@
 // Hessians grow without bound through stretches without control authority
 // turn into constraints instead of cancelling.  Chunks compose their own
 // stages, a log-depth scan over chunks gives V at every chunk boundary, and
-// each chunk then runs the square-root Riccati recursion inward, storing P_i,
+// each chunk then runs the Riccati recursion inward in 114-bit integers, storing P_i,
 // K_i, the Cholesky factor of Rbar + Bbar'P Bbar and Phi_i = Abar + Bbar K_i.
 //
 // Linear passes.  With those factors the remaining recursions are affine
@@ -18,6 +18,9 @@
 // z_{i+1} = Phi_i z_i + Bbar k_i + c_i forwards.  They run as chunked affine
 // scans (k_aff_*), also used for the refinement passes on the reduced KKT
 // residual and for the forward costate expansion of Sec. 7.
+#include <algorithm>
+
+#include "fx.cuh"
 #include "kernels.cuh"
 
 namespace eclqr {
@@ -30,13 +33,7 @@ __host__ int smem_lqr_level(int n) {
   const int rows = 8 * n, ldm = 3 * n + 1;
   return rows * ldm + 2 * rows + 2 * (ldm + rows) + n + 16;
 }
-// V, the stacked rows, and the reflector's two vectors; the FP32 sweep's blocks (the same
-// ones in floats, its gains and the stage data) fit in the same bytes
-__host__ int smem_riccati(int n, int m) {
-  const int rows = 2 * n + m, ld = n + m + 1;
-  return n * (n + 1) + rows * ld + rows + ld + 8;
-}
-__host__ int smem_riccati_finish(int n, int m) { return m * (n + m + 1) + n * (n + 1) + m * (n + 1) + 8; }
+__host__ int smem_riccati_finish(int n, int m) { return m * (n + m + 1) + m * (n + 1) + 8; }
 __host__ int smem_aff(int n, int m) { return 2 * (n * n + n) + n * n + 5 * n + 2 * m + 8; }
 
 // Cost-relation slot layout (ld 2n + 1): constraint rows at 0 (CI_ROWS of them),
@@ -210,15 +207,381 @@ __global__ void k_lqr_level(Group g, int src, int d, int per_task) {
   }
 }
 
-// ----------------------------------------------------------- chunk down-sweep: square-root Riccati
-// From V_b = 1/2 ||C z_b + c||^2 (the scan's value at the chunk end), each stage
-// stacks [L'_v | L'_z | l] and [C Bbar | C Abar | C cbar + c] over (v | z | 1) and
-// triangularises them by Householder QR: R_vv v + R_vz z + o_v = 0 at the
-// minimiser (K, k) and V_i = 1/2 ||R_i z + s_i||^2 with R_i upper triangular,
-// rows signed so that its diagonal is positive.  The sweep carries only V from
-// stage to stage; it stores the minimiser's rows (R_vv | R_vz | o_v) and
-// [R_i | s_i] (in the slots of P_i, p_i), and k_riccati_finish forms the
-// factors from them for every stage at once, off the sequential chain.
+// ----------------------------------------------------------- chunk down-sweep: Riccati
+// From V_b(z) = 1/2 z'P z + p'z at the chunk end (P = C'C from the scan's cost rows, or the
+// terminal cost itself), each stage forms the Hessian and gradient of cost plus value over (v, z),
+//   G = H + [Bbar Abar]' P [Bbar Abar],  g = h + [Bbar Abar]' (P cbar + p),
+// eliminates v by pivots on G's diagonal, and keeps P_i, p_i, the Schur complement on z.  The
+// pivot rows divided by the root of their pivot are the minimiser's rows (R_vv | R_vz | o_v)
+// that k_riccati_finish turns into K, k, chol(H_uu) and Phi.
+//
+// In FP64 this recursion loses the curvature that |P| |Abar|^2 cancels down to; carried as
+// square-root rows through a Householder QR it keeps it, at n + m dependent steps per stage, each a
+// reduction, a reciprocal square root and an update at 64 cycles per dependent FP64 instruction.
+// Here the recursion runs in the 114-bit integers of fx.cuh.  A condition number of P up to 2^110
+// is what a square root resolves in 55 bits, so the accuracy is that of the square-root form or
+// better, and the work is two products with independent outputs and m short pivot steps.  Column
+// exponents come from the diagonal, so entries are at most 1 in magnitude by Cauchy-Schwarz and
+// the scaling of states and controls does not matter.
+//
+// What bounds it: the integer multiply-adds (7 per 114 x 57 bit product, 4.1 cycles each per SM
+// sub-partition) where many problems share an SM, the latency of one stage's phases where few do.
+// Loops are kept rolled: with them unrolled the code outgrew the instruction cache and 1280
+// problems of 64 stages at n = 24 took 12.8 ms instead of 8.0.  Against the FP64 QR, 64 stages of
+// 1280 problems: n = 24 20.3 -> 7.8 ms, n = 16 10.2 -> 4.1, n = 8 3.38 -> 1.93; of 160 problems at
+// n = 24 7.5 -> 2.9 ms (k_riccati_finish, which no longer forms P = R'R, 2.24 -> 1.0 at 1280, n = 24).
+// The blocks are offsets into the task's shared memory (in elements of their type), so that every
+// access compiles to a shared-memory instruction with a 32-bit address.
+struct RiccatiFx {
+  int oP, oW, oG, oA, oI, ldp, ldx;
+  __host__ __device__ static int words(int n, int m) {  // 8-byte words
+    const int ldx = n + m + 1, big = n > m ? n : m;
+    return 2 * (p_size(n, m) + big * ldx + (n + m) * (n + m + 1) / 2 + n + m) + n * ldx + (3 * ldx + m + 2) / 2 + 1;
+  }
+  // the block of P, which later holds the stage Hessian's doubles
+  __host__ __device__ static int p_size(int n, int m) {
+    const int h = ((n + m) * (n + m + 1) / 2 + n + m + 1) / 2;
+    return n * (n + 1) > h ? n * (n + 1) : h;
+  }
+  __device__ RiccatiFx(int n, int m) {
+    ldp = n + 1;
+    ldx = n + m + 1;
+    oP = 0;
+    oW = p_size(n, m);
+    oG = oW + (n > m ? n : m) * ldx;
+    oA = 2 * (oG + (n + m) * (n + m + 1) / 2 + n + m);
+    oI = 2 * (oA + n * ldx);
+  }
+  __device__ int4 &P(int i) const { return ((int4 *)g_smem)[oP + i]; }  // [P | p] (ld n + 1)
+  __device__ int4 &W(int i) const { return ((int4 *)g_smem)[oW + i]; }  // P [Bbar Abar cbar]; the pivots' multipliers
+  __device__ int4 &G(int i) const { return ((int4 *)g_smem)[oG + i]; }  // G, g: packed rows, limbs or 128-bit integers
+  __device__ i128 &Gi(int i) const { return ((i128 *)g_smem)[oG + i]; }
+  __device__ int2 &A(int i) const { return ((int2 *)g_smem)[oA + i]; }  // [Bbar | Abar | cbar] (n x ldx)
+  __device__ double &Ad(int i) const { return g_smem[oA + i]; }         // the same as doubles
+  __device__ double &H(int i) const { return g_smem[2 * oP + i]; }      // [Rbar Mbar'; Mbar Qbar | rbar; qbar], packed
+  // column exponents of A (rows weighted by P's), of G, and of P (eP(nx): that of p); the pivots'
+  // shifts; a flag: a value that is not finite was met
+  __device__ int &al(int i) const { return ((int *)g_smem)[oI + i]; }
+  __device__ int &e(int i) const { return ((int *)g_smem)[oI + ldx + i]; }
+  __device__ int &eP(int i) const { return ((int *)g_smem)[oI + 2 * ldx + i]; }
+  __device__ int &hp(int i) const { return ((int *)g_smem)[oI + 3 * ldx + 1 + i]; }
+  __device__ int &bad() const { return ((int *)g_smem)[oI + 3 * ldx]; }
+};
+// the blocks of RiccatiFx, or the FP32 sweep's (V, stacked rows, two vectors, gains and stage
+// data, in floats)
+__host__ int smem_riccati(int n, int m) {
+  const int rows = 2 * n + m, ld = n + m + 1;
+  const int f32 = n * (n + 1) + rows * ld + rows + ld + m * (n + 1) + n * (n + m + 1);
+  return (std::max(RiccatiFx::words(n, m), (f32 + 1) / 2) + 9) & ~1;
+}
+
+__device__ __forceinline__ void copy_async(double *dst, const double *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
+}
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+__device__ __forceinline__ void team_sync() {
+  if (blockDim.x == 32) __syncwarp();
+  else __syncthreads();
+}
+
+// (j, k), j <= k < ld, of packed upper rows
+__device__ __forceinline__ int riccati_packed(int ld, int j, int k) { return j * ld - j * (j + 1) / 2 + k; }
+
+// P and p from raw sums: the block of G from row z0 on, nz states and the offset column, with
+// entry exponents e(z0 + a) + e(z0 + b) (p: e(z0 + a) + e(z0 + nz)).  Brings every diagonal entry to [2^112, 2^114),
+//
+// sets w.P and w.eP, and writes P and p in FP64 where they are given.
+static __device__ __noinline__ void riccati_value(const RiccatiFx w, int nz, int z0, double *Po, int ldo, double *po) {
+  const int ld = z0 + nz + 1;
+  auto raw = [&](int a, int b) { return riccati_packed(ld, z0 + a, z0 + b); };
+  const int tid = team_rank(), lane = tid & 31;
+  if (tid < 32) {
+    int pb = 0;
+    const int a = lane;
+    if (a < nz) {
+      const i128 d = w.Gi(raw(a, a));
+      // noise can leave an entry whose diagonal is not positive: its scale stays
+      const int s = d > 0 ? min((kFxP - fx_bits(d)) >> 1, 52) : 0;
+      w.eP(a) = w.e(z0 + a) - s;
+      const i128 v = w.Gi(raw(a, nz));
+      pb = v != 0 ? fx_bits(v) + s : 0;
+    }
+    pb = __reduce_max_sync(kFull, pb);
+    if (lane == 0) w.eP(nz) = w.e(z0 + nz) + (pb ? pb - kFxP : 0);
+  }
+  team_sync();
+  const bool bad = w.bad() != 0;
+  int a = 0, row = 0;  // row: linear index of (a, a); nz + 1 - a entries per row
+#pragma unroll 1
+  for (int idx = tid; idx < nz * (nz + 1) / 2 + nz; idx += TEAM) {
+    while (idx - row > nz - a) row += nz + 1 - a++;
+    const int b = a + idx - row;
+    const i128 v = w.Gi(raw(a, b));
+    const int4 l = fx_split4(fx_shift(v, w.e(z0 + a) + w.e(z0 + b) - w.eP(a) - w.eP(b)));
+    w.P(a * w.ldp + b) = l;
+    if (b < nz) w.P(b * w.ldp + a) = l;
+    if (Po) {
+      int s;
+      const long long top = fx_lead(v, s);
+      const double x = bad ? __longlong_as_double(0x7ff8000000000000ll) : fx_to(top, s + w.e(z0 + a) + w.e(z0 + b) - kFxP);
+      if (b < nz) {
+        Po[a * ldo + b] = x;
+        Po[b * ldo + a] = x;
+      } else {
+        po[a] = x;
+      }
+    }
+  }
+  team_sync();
+}
+
+// Starts the copy of a stage's [Bbar | Abar | cbar] (n1 rows) into w.Ad.
+static __device__ __forceinline__ void riccati_fetch(const Group &g, const RiccatiFx w, const double *ws, int n1, int nx,
+                                                     int mu) {
+  const int kh = nx + mu, ld = kh + 1;
+  const double *Ab = ws + g.ws.Ab, *Bb = ws + g.ws.Bb, *cb = ws + g.ws.cb;
+  const float rld = rcp_seed((float)ld);
+#pragma unroll 1
+  for (int idx = team_rank(); idx < n1 * ld; idx += TEAM) {
+    const int l = (int)(((float)idx + 0.5f) * rld), j = idx - l * ld;
+    copy_async(&w.Ad(l * w.ldx + j), j < mu ? Bb + l * g.m + j : (j < kh ? Ab + l * g.n + (j - mu) : cb + l));
+  }
+}
+
+// One stage: from w.P, w.eP (n1 states) and the fetched w.Ad to the value of the stage's nx
+// states.  Rv: the minimiser's rows (ld n + m + 1); Po, po: P_i and p_i; null where the stage is not
+// stored.  fetch() starts the copy of the next stage's w.Ad.
+template <typename Fetch>
+static __device__ __forceinline__ void riccati_stage(const Group &g, const RiccatiFx w, const double *ws, int n1, int nx,
+                                                     int mu, double *Rv, double *Po, double *po, Fetch fetch) {
+  const int n = g.n, m = g.m, tid = team_rank();
+  const int kh = nx + mu, ld = kh + 1, ldx = w.ldx, ldp = w.ldp;
+  const double *Qb = ws + g.ws.Qb, *Mb = ws + g.ws.Mb, *Rb = ws + g.ws.Rb, *qb = ws + g.ws.qb, *rb = ws + g.ws.rb;
+  auto hess = [&](int j, int k) {  // H and h in the order (v, z, 1), j <= k
+    if (k == kh) return j < mu ? rb + j : qb + (j - mu);
+    if (k < mu) return Rb + j * m + k;
+    return j < mu ? Mb + (k - mu) * m + j : Qb + (j - mu) * n + (k - mu);
+  };
+  auto packed = [&](int j, int k) { return riccati_packed(ld, j, k); };
+  // [Bbar | Abar | cbar] and its column exponents, the rows weighted by P's exponents
+#pragma unroll 1
+  for (int j = tid; j < ld; j += TEAM) w.al(j) = j == kh ? w.eP(n1) : kFxNone;
+  copy_wait();
+  team_sync();
+  const float rld = rcp_seed((float)ld);
+#pragma unroll 1
+  for (int idx = tid; idx < n1 * ld; idx += TEAM) {
+    const int l = (int)(((float)idx + 0.5f) * rld), j = idx - l * ld;
+    const double x = w.Ad(l * ldx + j);
+    const int ex = fx_expo(x);
+    if (ex != kFxNone) atomicMax(&w.al(j), ex + w.eP(l));
+    if (fx_nonfinite(x)) w.bad() = 1;
+  }
+  team_sync();
+#pragma unroll 1
+  for (int idx = tid; idx < n1 * ld; idx += TEAM) {
+    const int l = (int)(((float)idx + 0.5f) * rld), j = idx - l * ld;
+    w.A(l * ldx + j) = fx_split(fx_from(w.Ad(l * ldx + j), w.al(j) - w.eP(l)));
+  }
+  team_sync();
+  // W = P [Bbar | Abar | cbar] + [0 | 0 | p] in units of 2^-111: 2 x 2 entries per item
+  const int c2 = (ld + 1) >> 1;
+  const float rc2 = rcp_seed((float)c2);
+#pragma unroll 1
+  for (int it = tid; it < c2 * ((n1 + 1) >> 1); it += TEAM) {
+    const int rp = (int)(((float)it + 0.5f) * rc2), c = 2 * (it - rp * c2), r = 2 * rp;
+    const int r1 = min(r + 1, n1 - 1), c1 = min(c + 1, kh);
+    FxAcc acc[4];
+#pragma unroll
+    for (int q = 0; q < 4; q++) acc[q].zero();
+    int i0 = r * ldp, i1 = r1 * ldp, j0 = c, j1 = c1;
+#pragma unroll 2
+    for (int l = 0; l < n1; l++, i0++, i1++, j0 += ldx, j1 += ldx) {
+      const int4 x0 = w.P(i0), x1 = w.P(i1);
+      const int2 a0 = w.A(j0), a1 = w.A(j1);
+      acc[0].mad(x0, a0);
+      acc[1].mad(x0, a1);
+      acc[2].mad(x1, a0);
+      acc[3].mad(x1, a1);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      const int rr = q < 2 ? r : r1, cc = (q & 1) ? c1 : c;
+      i128 v = acc[q].value<60>();
+      if (cc == kh) v += fx_shift(fx_join4(w.P(rr * ldp + n1)), w.eP(n1) - w.al(kh) - 3);
+      w.W(rr * ldx + cc) = fx_split4(v);
+    }
+  }
+  team_sync();
+  // H and h, into the block of P while G is formed
+  {
+    int j = 0, row = 0;
+#pragma unroll 1
+    for (int idx = tid; idx < kh * (kh + 1) / 2 + kh; idx += TEAM) {
+      while (idx - row >= ld - j) row += ld - j++;
+      copy_async(&w.H(idx), hess(j, j + idx - row));
+    }
+  }
+  // raw G = [Bbar Abar]' W in units of 2^-114: 2 x 2 entries (j, k), j <= k, per item
+  {
+    int jt = 0, start = 0;  // row pair jt: column pairs jt .. c2 - 1
+#pragma unroll 1
+    for (int it = tid;; it += TEAM) {
+      while (2 * jt < kh && it - start >= c2 - jt) start += c2 - jt++;
+      if (2 * jt >= kh) break;
+      const int j = 2 * jt, j1 = min(j + 1, kh - 1), k = j + 2 * (it - start), k1 = min(k + 1, kh);
+      FxAcc acc[4];
+#pragma unroll
+      for (int q = 0; q < 4; q++) acc[q].zero();
+      int ia = j, ib = j1, ka = k, kb = k1;
+#pragma unroll 2
+      for (int l = 0; l < n1; l++, ia += ldx, ib += ldx, ka += ldx, kb += ldx) {
+        const int4 x0 = w.W(ka), x1 = w.W(kb);
+        const int2 a0 = w.A(ia), a1 = w.A(ib);
+        acc[0].mad(x0, a0);
+        acc[1].mad(x1, a0);
+        acc[2].mad(x0, a1);
+        acc[3].mad(x1, a1);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        const int jj = q < 2 ? j : j1, kk = (q & 1) ? k1 : k;
+        if (jj <= kk) w.Gi(packed(jj, kk)) = acc[q].value<54>();
+      }
+    }
+  }
+  copy_wait();
+  team_sync();
+  fetch();
+  // exponents of the columns of G + H from its diagonal, of the offsets from their largest entry
+#pragma unroll 1
+  for (int j = tid; j < kh; j += TEAM) {
+    const i128 d = w.Gi(packed(j, j));
+    const int t = max(d != 0 ? fx_bits(d) - kFxP + 2 * w.al(j) : kFxNone, fx_expo(w.H(packed(j, j))));
+    w.e(j) = t > kFxNone / 2 ? (t + 2) >> 1 : 0;
+  }
+  team_sync();
+  if (tid < 32) {
+    int t = kFxNone;
+#pragma unroll 1
+    for (int j = tid; j < kh; j += 32) {
+      const i128 d = w.Gi(packed(j, kh));
+      t = max(t, (d != 0 ? fx_bits(d) - kFxP + w.al(j) + w.al(kh) : kFxNone) - w.e(j));
+      t = max(t, fx_expo(w.H(packed(j, kh))) - w.e(j));
+    }
+    t = __reduce_max_sync(kFull, t);
+    if (tid == 0) w.e(kh) = t > kFxNone / 2 ? t + 1 : 0;
+  }
+  team_sync();
+  {
+    int j = 0, row = 0;
+#pragma unroll 1
+    for (int idx = tid; idx < kh * (kh + 1) / 2 + kh; idx += TEAM) {
+      while (idx - row >= ld - j) row += ld - j++;
+      const int k = j + idx - row;
+      const double h = w.H(idx);
+      if (fx_nonfinite(h)) w.bad() = 1;
+      const int ejk = w.e(j) + w.e(k);
+      const i128 v = fx_shift(w.Gi(idx), w.al(j) + w.al(k) - ejk) + fx_from4(h, ejk);
+      // the z block stays whole integers, which the last product is subtracted from
+      if (j < mu) w.G(idx) = fx_split4(v);
+      else w.Gi(idx) = v;
+    }
+  }
+  team_sync();
+  // pivots on v: y_j = G_kj 2^h, l_j = y_j / (d 2^(2h)) (units of 2^-112, in
+  // w.W), G_ij -= l_i y_j for rows i < mu
+#pragma unroll 1
+  for (int k = 0; k < mu; k++) {
+    const int gk = packed(k, 0);
+    i128 d = fx_join4(w.G(gk + k));
+    if (d <= 0) d = (i128)1 << (kFxP - 53);  // rounding noise of a singular pivot
+    const int h = (kFxP - fx_bits(d)) >> 1;
+    const i128 dp = d << (2 * h);
+    const long long g0 = fx_rcp((unsigned long long)(dp >> 50));
+    const int2 g2 = fx_split(g0);
+    FxAcc acc;
+    acc.zero();
+    acc.mad(fx_split4(dp), g2);
+    const long long r = (long long)(((i128)1 << kFxP) - acc.value<55>());
+    // the offsets' column has no bound by the diagonal: where the shift would pass 2^116, its
+    // exponent is raised first
+    const int over = fx_bits(fx_join4(w.G(gk + kh))) + h - 116;
+    if (over > 0) {
+      team_sync();
+#pragma unroll 1
+      for (int i = tid; i < kh; i += TEAM) {
+        const int x = packed(i, kh);
+        if (i < mu) w.G(x) = fx_split4(fx_shift(fx_join4(w.G(x)), -over));
+        else w.Gi(x) = fx_shift(w.Gi(x), -over);
+      }
+      if (tid == 0) w.e(kh) += over;
+      team_sync();
+    }
+    if (tid == 0) w.hp(k) = h;
+    team_sync();  // every thread has read row k before it is rewritten
+#pragma unroll 1
+    for (int j = k + tid; j < ld; j += TEAM) {
+      const i128 y = j == k ? d << h : fx_join4(w.G(gk + j)) << h;
+      const int4 y4 = fx_split4(y);
+      w.G(gk + j) = y4;
+      acc.zero();
+      acc.mad(y4, g2);
+      const i128 t = acc.value<57>();
+      w.W(k * ldx + j) = fx_split4(t + __mul64hi((long long)(t >> 57) << 6, r << 1));
+    }
+    team_sync();
+    // rows k + 1 .. mu - 1
+    int i = k + 1, row = 0;
+#pragma unroll 1
+    for (int idx = tid;; idx += TEAM) {
+      while (i < mu && idx - row >= ld - i) row += ld - i++;
+      if (i >= mu) break;
+      const int j = i + idx - row;
+      FxAcc4 a4;
+      a4.zero();
+      a4.mad(w.W(k * ldx + i), w.G(gk + j));
+      const int x = packed(i, j);
+      w.G(x) = fx_split4(fx_join4(w.G(x)) - a4.value());
+    }
+    team_sync();
+  }
+  // Schur complement on z
+  {
+    int a = 0, row = 0;
+#pragma unroll 1
+    for (int idx = tid; idx < nx * (nx + 1) / 2 + nx; idx += TEAM) {
+      while (idx - row > nx - a) row += nx + 1 - a++;
+      const int b = a + idx - row;
+      FxAcc4 acc;
+      acc.zero();
+#pragma unroll 1
+      for (int k = 0; k < mu; k++) acc.mad(w.W(k * ldx + mu + a), w.G(packed(k, mu + b)));
+      w.Gi(packed(mu + a, mu + b)) -= acc.value();
+    }
+  }
+  // the minimiser's rows y_j / sqrt(d 2^(2h))
+  const bool bad = w.bad() != 0;
+  if (Rv) {
+#pragma unroll 1
+    for (int k = 0; k < mu; k++) {
+      const int gk = packed(k, 0);
+      const unsigned long long rs = fx_rsqrt((unsigned long long)((fx_join4(w.G(gk + k)) << w.hp(k)) >> 50));
+#pragma unroll 1
+      for (int j = k + tid; j < ld; j += TEAM) {
+        int s;
+        const long long top = fx_lead(fx_join4(w.G(gk + j)), s);
+        // (4 d)^(-1/2) 2^62, so the value is 2 2^(s - 114 + 2) of the product's upper half
+        const double x = fx_to(__mul64hi(top, (long long)rs), s + 3 - kFxP + w.e(j));
+        Rv[k * (n + m + 1) + j] = bad ? __longlong_as_double(0x7ff8000000000000ll) : x;
+      }
+    }
+  }
+  team_sync();
+  riccati_value(w, nx, mu, Po, n, po);
+}
+
 static __device__ void riccati_task(const Group &g, int fin, int t, int per_task);
 __global__ void k_riccati_down(Group g, int fin, int per_task, int *queue) {
   for_tasks(g.nslot, queue, [&](int t) { riccati_task(g, fin, t, per_task); });
@@ -231,127 +594,108 @@ static __device__ void riccati_task(const Group &g, int fin, int t, int per_task
   if (skipped_by_mask(g, ci.prob)) return;
   if (g.fp64 != nullptr && g.fp64[P.id] == 0) return;  // mixed precision: k_riccati_down_f32 sweeps it
   if (ci.c >= P.nch) return;
-  const int n = g.n, m = g.m, tid = team_rank();
+  const int n = g.n, tid = team_rank();
   const int a = ci.c * P.L, b = min(a + P.L, P.N);
   // every chunk but the last re-sweeps the next chunk's stages from the same scan value, so that the
   // value function it starts from is, bit for bit, the one the next chunk computes at their boundary
   const bool resweep = ci.c + 1 < P.nch;
   const int start = resweep ? min(b + P.L, P.N) : b;
-  const int ldr = 2 * n + 1;
-  double *sm = team_smem(per_task);
-  const int rows_max = 2 * n + m, ldst = n + m + 1;
-  double *V = sm, *St = V + n * (n + 1), *v = St + rows_max * ldst, *w = v + rows_max;
-  // V_b, rows signed to a positive diagonal
-  int rv;
-  {
-    const int slot = resweep ? t + 2 : t + 1;
-    const double *src = crel_cost(g.CS[fin] + (size_t)slot * g.cs_stride, n);
-    const int *I = g.CI[fin] + (size_t)slot * CI_STRIDE;
-    const int nbz = I[CI_NA];
-    rv = I[CI_ROWS2];
-    for (int idx = tid; idx < rv * (nbz + 1); idx += TEAM) {
-      int r = idx / (nbz + 1), j = idx - r * (nbz + 1);
-      const double sg = (src[r * ldr + r] >= 0.0) ? 1.0 : -1.0;
-      V[r * (n + 1) + j] = sg * src[r * ldr + j];
+  const RiccatiFx w(n, g.m);
+  // V_b
+  if (tid == 0) w.bad() = 0;
+  if (start == P.N) {  // the terminal cost
+    double *ws = stage_ws(g, P.st0 + P.N);
+    const double *Qb = ws + g.ws.Qb, *qb = ws + g.ws.qb;
+    const int nz = stage_wi(g, P.st0 + P.N)[SI_NBAR];
+#pragma unroll 1
+    for (int j = tid; j < nz; j += TEAM) {
+      const int t2 = fx_expo(Qb[j * n + j]);
+      w.e(j) = t2 > kFxNone / 2 ? (t2 + 1) >> 1 : 0;
     }
-    tsync();
-    if (b == P.N) {  // P_N = C'C, p_N = C'c
-      double *wsN = stage_ws(g, P.st0 + b);
-      for (int idx = tid; idx < nbz * (nbz + 1); idx += TEAM) {
-        int r = idx / (nbz + 1), j = idx - r * (nbz + 1);
-        double s0 = 0.0;
-        for (int l = 0; l < rv; l++) s0 = fma(V[l * (n + 1) + r], V[l * (n + 1) + j], s0);
-        if (j < nbz) wsN[g.ws.P + r * n + j] = s0; else wsN[g.ws.p + r] = s0;
+    __syncthreads();
+    if (tid < 32) {
+      int mx = tid < nz ? fx_expo(qb[tid]) - w.e(tid) : kFxNone;
+      mx = __reduce_max_sync(kFull, mx);
+      if (tid == 0) w.e(nz) = mx > kFxNone / 2 ? mx : 0;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int idx = tid; idx < nz * (nz + 1); idx += TEAM) {
+      const int j = idx / (nz + 1), k = idx - j * (nz + 1);
+      if (k < j) continue;
+      const double x = k < nz ? Qb[j * n + k] : qb[j];
+      if (fx_nonfinite(x)) w.bad() = 1;
+      w.Gi(riccati_packed(nz + 1, j, k)) = fx_from4(x, w.e(j) + w.e(k));
+    }
+    __syncthreads();
+    riccati_value(w, nz, 0, b == P.N ? ws + g.ws.P : nullptr, n,
+                  ws + g.ws.p);
+  } else {  // P = C'C, p = C'c from the scan's cost rows, scaled by column and (at most 0, in al) by row
+    const int slot = t + 2, ldr = 2 * n + 1;
+    const double *src = crel_cost(g.CS[fin] + (size_t)slot * g.cs_stride, n);
+    const int nz = g.CI[fin][(size_t)slot * CI_STRIDE + CI_NA], rv = g.CI[fin][(size_t)slot * CI_STRIDE + CI_ROWS2];
+#pragma unroll 1
+      for (int j = tid; j <= nz; j += TEAM) {
+      int mx = kFxNone;
+#pragma unroll 1
+      for (int r = 0; r < rv; r++) mx = max(mx, fx_expo(src[r * ldr + j]));
+      w.e(j) = mx > kFxNone / 2 ? mx : 0;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int r = tid; r < rv; r += TEAM) {
+      int mx = kFxNone;
+#pragma unroll 1
+      for (int j = 0; j <= nz; j++) mx = max(mx, fx_expo(src[r * ldr + j]) - w.e(j));
+      w.al(r) = mx > kFxNone / 2 ? mx : 0;
+#pragma unroll 1
+      for (int j = 0; j <= nz; j++) {
+        w.A(r * w.ldx + j) = fx_split(fx_from(src[r * ldr + j], w.al(r) + w.e(j)));
+        if (fx_nonfinite(src[r * ldr + j])) w.bad() = 1;
       }
     }
+    __syncthreads();
+#pragma unroll 1
+    for (int idx = tid; idx < nz * (nz + 1); idx += TEAM) {
+      const int j = idx / (nz + 1), k = idx - j * (nz + 1);
+      if (k < j) continue;
+      i128 s = 0;
+#pragma unroll 1
+      for (int r = 0; r < rv; r++) {
+        const int2 x = w.A(r * w.ldx + j), y = w.A(r * w.ldx + k);
+        const i128 v = ((i128)fx_mad(x.x, y.x, 0) << (2 * kFxB)) + ((i128)fx_mad(x.x, y.y, fx_mad(x.y, y.x, 0)) << kFxB) +
+                       fx_mad(x.y, y.y, 0);
+        s += fx_shift(v, 2 * w.al(r));
+      }
+      w.Gi(riccati_packed(nz + 1, j, k)) = s;
+    }
+    __syncthreads();
+    riccati_value(w, nz, 0, nullptr, n, nullptr);
   }
+  int n1 = stage_wi(g, P.st0 + start)[SI_NBAR], nx = 0, mu = 0;
+  if (start > a) {
+    const int s = P.st0 + start - 1;
+    nx = stage_wi(g, s)[SI_NBAR];
+    mu = stage_wi(g, s)[SI_MBAR];
+    riccati_fetch(g, w, stage_ws(g, s), n1, nx, mu);
+  }
+#pragma unroll 1
   for (int i = start - 1; i >= a; --i) {
     const bool store = i < b;  // the next chunk's stages are stored by that chunk
     const int s = P.st0 + i;
     double *ws = stage_ws(g, s);
-    int *wi = stage_wi(g, s);
-    const int nx = wi[SI_NBAR], mu = wi[SI_MBAR], n1 = stage_wi(g, s + 1)[SI_NBAR];
-    const int kh = nx + mu, ld = kh + 1;
-    const double *Ab = ws + g.ws.Ab, *Bb = ws + g.ws.Bb, *cb = ws + g.ws.cb, *LT = ws + g.ws.LT, *lt = ws + g.ws.lt;
-    // value rows [V Bbar | V Abar | V cbar + s] at St rows kh .. kh + rv - 1; after the first
-    // stage V = [R_{i+1} | s_{i+1}] with R_{i+1} upper triangular (exact zeros below its
-    // diagonal), so row r's products start at column r
-    for (int idx = tid; idx < rv * ld; idx += TEAM) {
-      int r = idx / ld, j = idx - r * ld;
-      const double *row = V + r * (n + 1);
-      const int l0 = (i < start - 1) ? r : 0;
-      double val = 0.0;
-      if (j < mu) {
-        for (int l = l0; l < n1; l++) val = fma(row[l], Bb[l * m + j], val);
-      } else if (j < kh) {
-        for (int l = l0; l < n1; l++) val = fma(row[l], Ab[l * n + (j - mu)], val);
-      } else {
-        val = row[n1];
-        for (int l = l0; l < n1; l++) val = fma(row[l], cb[l], val);
-      }
-      St[(kh + r) * ld + j] = val;
+    int nx2 = 0, mu2 = 0;
+    if (i > a) {
+      nx2 = stage_wi(g, s - 1)[SI_NBAR];
+      mu2 = stage_wi(g, s - 1)[SI_MBAR];
     }
-    // QR of [L' l; value rows] with L' (columns v, z) upper triangular: the reflector of
-    // column k has entries only in row k of L' and in the value rows, so step k works on
-    // those rv + 1 rows alone.  Row k of L' is loaded into the slot right above the value
-    // rows (St row kh - 1), and the finished row moves to St row k before the next load.
-    // The next row of L' is read from global memory into registers before the current step
-    // runs (thread tid holds columns tid and tid + TEAM, kh + 1 <= 2 TEAM), so its latency
-    // hides behind the step.
-    double nxt[2];
-    for (int q = 0; q < 2; q++) {
-      const int j = tid + q * TEAM;
-      nxt[q] = (j <= kh && kh > 0) ? ((j < kh) ? LT[j] : lt[0]) : 0.0;
-    }
-    for (int k = 0; k < kh; k++) {
-      double *W = St + (kh - 1) * ld;
-      for (int q = 0; q < 2; q++) {
-        const int j = tid + q * TEAM;
-        if (j > kh) continue;
-        if (k > 0 && j >= k - 1) St[(k - 1) * ld + j] = W[j];
-        if (j >= k) W[j] = nxt[q];
-      }
-      tsync();
-      if (k + 1 < kh)
-        for (int q = 0; q < 2; q++) {
-          const int j = tid + q * TEAM;
-          if (j >= k + 1 && j <= kh) nxt[q] = (j < kh) ? LT[(k + 1) * (n + m) + j] : lt[k + 1];
-        }
-      HHLayout L = hh_layout(kh + 1 - k, rv + 1);
-      hh_core(W, ld, 0, rv + 1, k, nullptr, k, kh + 1 - k, L, v, w, 0.0);
-    }
-    // sign the z rows to a positive diagonal (rows mu .. kh - 1), on the integer pipe: a row
-    // whose diagonal is below zero (sign bit set, not -0, not NaN) has every sign bit flipped
-    for (int idx = tid; idx < nx * ld; idx += TEAM) {
-      int r = mu + idx / ld, j = idx - (idx / ld) * ld;
-      const long long db = __double_as_longlong(St[r * ld + r]);
-      const bool neg = db < 0 && (db & 0x7fffffffffffffffll) != 0 && (db & 0x7fffffffffffffffll) <= 0x7ff0000000000000ll;
-      if (neg && j != r) St[r * ld + j] = __longlong_as_double(__double_as_longlong(St[r * ld + j]) ^ (1ll << 63));
-    }
-    tsync();
-    for (int r = mu + tid; r < kh; r += TEAM)
-      St[r * ld + r] = __longlong_as_double(__double_as_longlong(St[r * ld + r]) & 0x7fffffffffffffffll);
-    tsync();
-    // the minimiser's rows (R_vv | R_vz | o_v) for k_riccati_finish, and the new value rows
-    // [R_i | s_i], kept here and stored in the slots of P_i, p_i (ld n + 1)
-    if (store) {
-      double *Rv = ws + g.ws.Rv;
-      for (int idx = tid; idx < mu * ld; idx += TEAM) {
-        int r = idx / ld, j = idx - r * ld;
-        Rv[r * (n + m + 1) + j] = St[r * ld + j];
-      }
-    }
-    for (int idx = tid; idx < nx * (nx + 1); idx += TEAM) {
-      int r = idx / (nx + 1), c = idx - r * (nx + 1);
-      V[r * (n + 1) + c] = (c < nx) ? ((c >= r) ? St[(mu + r) * ld + mu + c] : 0.0) : St[(mu + r) * ld + kh];
-    }
-    tsync();
-    rv = nx;
-    if (store)
-      for (int idx = tid; idx < nx * (nx + 1); idx += TEAM) {
-        int r = idx / (nx + 1), c = idx - r * (nx + 1);
-        ws[g.ws.P + r * (n + 1) + c] = V[r * (n + 1) + c];
-      }
+    riccati_stage(g, w, ws, n1, nx, mu, store ? ws + g.ws.Rv : nullptr, store ? ws + g.ws.P : nullptr, ws + g.ws.p,
+                  [&] {
+                    if (i > a) riccati_fetch(g, w, stage_ws(g, s - 1), nx, nx2, mu2);
+                  });
+    n1 = nx;
+    nx = nx2;
+    mu = mu2;
   }
 }
 
@@ -359,8 +703,7 @@ static __device__ void riccati_task(const Group &g, int fin, int t, int per_task
 // For each stage i < N that the sweep stored (FP64 sweeps only): from the
 // minimiser's rows, R_vv [K | k] = -[R_vz | o_v] by back substitution, the
 // Cholesky factor of H_uu = R_vv'R_vv (R_vv' with rows signed to a positive
-// diagonal), Phi = Abar + Bbar K (the closed-loop map of the affine chains), and
-// from [R_i | s_i], P_i = R_i'R_i and p_i = R_i's_i, which replace it.
+// diagonal) and Phi = Abar + Bbar K (the closed-loop map of the affine chains).
 __global__ void k_riccati_finish(Group g, int per_task) {
   for_stages(g, [&](const int s) {
     const StageInfo S = g.st[s];
@@ -374,15 +717,11 @@ __global__ void k_riccati_finish(Group g, int per_task) {
     const int nx = wi[SI_NBAR], mu = wi[SI_MBAR], n1 = stage_wi(g, s + 1)[SI_NBAR];
     const int ldr = n + m + 1;
     double *sm = team_smem(per_task);
-    double *R = sm, *V = R + m * ldr, *Kt = V + n * (n + 1);
+    double *R = sm, *Kt = R + m * ldr;
     const double *Rv = ws + g.ws.Rv, *Ab = ws + g.ws.Ab, *Bb = ws + g.ws.Bb;
     for (int idx = tid; idx < mu * (nx + mu + 1); idx += TEAM) {
       int r = idx / (nx + mu + 1), j = idx - r * (nx + mu + 1);
       R[r * ldr + j] = Rv[r * ldr + j];
-    }
-    for (int idx = tid; idx < nx * (nx + 1); idx += TEAM) {
-      int r = idx / (nx + 1), c = idx - r * (nx + 1);
-      V[r * (n + 1) + c] = ws[g.ws.P + r * (n + 1) + c];
     }
     tsync();
     // K, k:  R_vv [K | k] = -[R_vz | o_v]
@@ -392,12 +731,6 @@ __global__ void k_riccati_finish(Group g, int per_task) {
         for (int l = r + 1; l < mu; l++) s0 = fma(-R[r * ldr + l], Kt[l * (n + 1) + c], s0);
         Kt[r * (n + 1) + c] = s0 / R[r * ldr + r];
       }
-    }
-    for (int idx = tid; idx < nx * (nx + 1); idx += TEAM) {
-      int r = idx / (nx + 1), c = idx - r * (nx + 1);
-      double s0 = 0.0;
-      for (int l = 0; l <= r && l < nx; l++) s0 = fma(V[l * (n + 1) + r], V[l * (n + 1) + c], s0);
-      if (c < nx) ws[g.ws.P + r * n + c] = s0; else ws[g.ws.p + r] = s0;
     }
     for (int idx = tid; idx < mu * mu; idx += TEAM) {
       int r = idx / mu, j = idx - r * mu;

@@ -187,7 +187,7 @@ __device__ __forceinline__ int *stage_wi(const Group &g, int s) { return g.WI + 
 // whole dynamic allocation).
 __device__ __forceinline__ int team_task() { return blockIdx.x; }
 
-extern __shared__ double g_smem[];
+extern __shared__ __align__(16) double g_smem[];  // 16: the Riccati sweep's four-limb entries
 __device__ __forceinline__ double *team_smem(int /*per_task*/) { return g_smem; }
 
 // Runs body(s) for the stages of a per-stage launch: the CTA's own stage (one CTA per
