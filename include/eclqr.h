@@ -109,10 +109,11 @@ typedef struct {
   double tau_rank;   /* relative rank cut after row scaling (Sec. 8 items 1-2); default 1e-10 */
   double tau_inc;    /* inconsistency cut on a scaled offset (Sec. 8 item 4); default 1e-8    */
   int32_t refine;    /* refinement passes on the reduced LQR KKT residual; default 2          */
-  int32_t chunk;     /* stages per scan chunk; 0 = chosen from N and the SM count: one chunk
-                      * per problem when the longest horizon is at most the batch's stages
-                      * per SM, else 7 to 64 stages.  A problem that fits one chunk is swept once per
-                      * scan, from its terminal element, with no chunk aggregate           */
+  int32_t chunk;     /* stages per scan chunk; 0 = chosen from the horizons, n and the SM count: one
+                      * chunk per problem of a group unless its longest horizon exceeds
+                      * min(150, 40 + 8 n) stages by more than n / 2 times the batch's
+                      * stages per SM, else 7 to 64 stages.  A problem that fits one chunk is swept
+                      * once per scan, from its terminal element, with no chunk aggregate */
   int32_t team_warps; /* warps of the CTA that runs one task: 1, 2, 4 or 8 for every kernel;
                        * 0 (default) = per kernel: 4 when a launch has fewer tasks than
                        * SMs; with at least 4 tasks per SM the kernel's measured best for

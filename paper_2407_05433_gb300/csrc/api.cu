@@ -404,8 +404,6 @@ int eclqr_create(const eclqr_desc *d, const eclqr_options *opt, eclqr_handle **o
   std::map<std::pair<int, int>, std::vector<int>> by_dims;
   for (int j = 0; j < P; j++) by_dims[{d->n[j], d->m[j]}].push_back(j);
   long long total_stages = h->lay.stages;
-  int nmax = 1;  // the longest horizon of the batch
-  for (int j = 0; j < P; j++) nmax = std::max(nmax, d->N[j]);
   for (auto &kv : by_dims) {
     GroupHost gh;
     Group &g = gh.g;
@@ -475,22 +473,30 @@ int eclqr_create(const eclqr_desc *d, const eclqr_options *opt, eclqr_handle **o
     std::vector<StageInfo> gs;
     std::vector<ChunkInfo> gc;
     gh.any_skip = false;
+    // One chunk per problem runs without chunk aggregates, scan levels and next-chunk re-sweeps:
+    // the least work, but the longest horizon is swept stage by stage.  In units of one stage of
+    // that sweep (10 us at n = 4, 13 at 8, 20 at 16, 35 at 24, 55 at 32), the chunked scan costs a
+    // fixed 70 to 150 (its levels and shortest chunks) and about n / 2 for every stage that an SM
+    // has to do, mostly the aggregates' (measured, P problems of up to N stages, chunked / one
+    // chunk: n = 16, 1 x 128 3.2 / 2.9 ms, 1 x 256 3.9 / 5.7, 24 x 200 6.9 / 5.6, 152 x 200 27 / 10;
+    // n = 4, 1 x 64 1.13 / 1.09, 24 x 200 1.9 / 2.8, 64 x 200 3.4 / 3.0; n = 32, 8 x 200 21 / 13,
+    // 64 x 200 78 / 20).
+    const long long group_longest = d->N[gh.ids[0]];
+    const bool one_chunk =
+        group_longest * sms <= std::min(150, 40 + 8 * g.n) * (long long)sms + std::max(3, g.n / 2) * total_stages;
     for (int j : gh.ids) {
       ProbInfo pi = pinfo[j];
       int L = h->opt.chunk;
-      if (L <= 0 && (long long)nmax * sms <= total_stages) {
-        // the longest horizon is at most the stages per SM: one chunk per problem.  Its
-        // sweeps then run without chunk aggregates, scan levels or next-chunk re-sweeps,
-        // the least work, and no problem's sequential sweep outlasts an SM's share of the
-        // batch (256 problems of 256 stages: 37 ms against 83 ms chunked).
+      if (L <= 0 && one_chunk) {
         L = std::max(1, pi.N);
       } else if (L <= 0) {
-        // enough chunks to give every SM work, but never shorter than 7 stages: shorter
+        // about three chunks per SM (16384 stages at n = 16: 17.5 ms with 40-stage chunks, 20.3 with
+        // two chunks of 54 per SM, 22.1 with nine of 12), but never shorter than 7 stages: shorter
         // chunks place more boundaries, and where a boundary meets an ill-conditioned
         // stage the refinement needs more than its default passes (on the degenerate
         // n = 12 instance 6-stage chunks miss the 1e-9 gate after two).  A 1024-stage
         // problem then runs as 147 chunks, one CTA each, on a 152-SM GB300.
-        long long target = std::max<long long>(1, total_stages / (2LL * sms));
+        long long target = std::max<long long>(1, total_stages / (3LL * sms));
         L = (int)std::min<long long>(64, std::max<long long>(7, target));
         L = std::max(1, std::min(L, pi.N));
       }
@@ -524,7 +530,9 @@ int eclqr_create(const eclqr_desc *d, const eclqr_options *opt, eclqr_handle **o
     g.nprob = (int)gp.size();
     g.nstage = (int)gs.size();
     g.nslot = (int)gc.size();
-    gh.levels = ilog2ceil(gh.maxnch + 1);
+    // a group whose every problem is one chunk has nothing to scan: its sweeps start from the
+    // boundary elements where the up-sweeps left them
+    gh.levels = gh.maxnch == 1 ? 0 : ilog2ceil(gh.maxnch + 1);
     g.ws = make_ws_layout(g.n, g.m, pmax, qmax);
     g.cs_stride = ((8 * g.n * g.n + 4 * g.n) + 3) & ~3;  // cost relations: 2n constraint + 2n cost rows
     g.cr_stride = 0;
@@ -647,7 +655,7 @@ int run_build(eclqr_handle *h, GroupHost &gh, const Group &g, cudaStream_t gst, 
     }
   }
   TRY(launch(h, k_terminal, g.nprob, sw, gst, g, sw));
-  TRY(launch(h, k_primal_up, g.nslot, sw, gst, g, sw));
+  if (gh.levels > 0) TRY(launch(h, k_primal_up, g.nslot, sw, gst, g, sw));
   int src = 0;
   for (int k = 0; k < gh.levels; k++, src ^= 1)
     TRY(launch(h, k_rel_level, g.nslot, sl, gst, g, src, 1 << k, (int)ST_INFEASIBLE_SUFFIX, sl));
@@ -675,7 +683,8 @@ int aff_scan(eclqr_handle *h, const GroupHost &gh, const Group &g, int mode, cud
   TRY(launch(h, k_aff_up, g.nslot, sa, st, g, mode, sa));
   int src = 0;
   // radix-4 levels: strides 1, 4, 16, ... until they cover every slot
-  for (int d = 1; d < gh.maxnch + 1; d *= 4, src ^= 1) TRY(launch(h, k_aff_level, g.nslot, sa, st, g, src, d, fwd, sa));
+  for (int d = 1; gh.levels > 0 && d < gh.maxnch + 1; d *= 4, src ^= 1)
+    TRY(launch(h, k_aff_level, g.nslot, sa, st, g, src, d, fwd, sa));
   TRY(launch(h, k_aff_down, g.nslot, sa, st, g, mode, src, sa));
   return ECLQR_OK;
 }
@@ -707,7 +716,7 @@ int run_mult(eclqr_handle *h, const GroupHost &gh, const Group &g, cudaStream_t 
   const int sf = smem_dual_leaf(n, m, g.wmax);
   TRY(launch(h, k_dual_stage, g.nstage, sd, gst, g, x, u, sd));
   TRY(launch(h, k_dual_terminal, g.nprob, sw, gst, g, sw));
-  TRY(launch(h, k_dual_up, g.nslot, sw, gst, g, sw));
+  if (gh.levels > 0) TRY(launch(h, k_dual_up, g.nslot, sw, gst, g, sw));
   int src = 0;
   for (int k = 0; k < gh.levels; k++, src ^= 1)
     TRY(launch(h, k_rel_level, g.nslot, sl, gst, g, src, 1 << k, (int)ST_OK, sl));
