@@ -281,9 +281,7 @@ int eclqr_probe_fp64_peak(double *tflops);
  * build.  data: the built problem's matrices (A, B, C, D, E, Q, M, R, same
  * arrays or equal values), new qv and rv, and c, d, e pointing at zeros; the
  * call does not check these preconditions, and with nonzero c, d or e the
- * subsequent solve is wrong.  Zeroes t_i, y_i and cbar_i, recomputes
- * qbar_i = T_i'q_i + Y_i'r_i and rbar_i = Z_i'r_i (eq. reduced-cost-data with
- * t = y = 0) and the square-root Riccati's stage offsets, and sets the
+ * subsequent solve is wrong.  Zeroes t_i, y_i and cbar_i and sets the
  * Riccati's own offsets to zero, so that the following eclqr_solve starts
  * from z = v = 0 and its first refinement pass (the P-form offset recursion
  * on the stored factors) reaches the new solution, the default second pass

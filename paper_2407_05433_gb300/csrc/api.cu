@@ -95,29 +95,29 @@ namespace {
 // reduction and each triangular solve once, where four warps would each repeat
 // them, and needs no CTA barrier.  The entries are the fastest team measured per
 // kernel and state dimension on the 4096-problem uneven batch (each (n, m) group
-// alone, about seven problems per SM).  For example the affine chains take
-// 4 ms with two warps at n = 8 against 7 with eight, but 7 ms with eight at
-// n = 24 against 11 with two; the chunk up-sweeps of the long horizon (65536
-// stages in 1024 chunks) take 27 ms with two warps per chunk against 37 with one;
-// the stage elimination takes 14 ms with one warp at n = 8 against 29 ms with
-// four, but 86 ms with four at n = 24 against 120 ms with one, where its stage
-// matrices fill four warps.  The Riccati sweep's products have thousands of
-// independent integer multiply-adds per stage from n = 16 on: 48 stages of 1280
-// problems take 1.44 / 1.48 / 1.65 ms with 1 / 2 / 4 warps at n = 8, 2.56 / 2.09 /
-// 2.23 at n = 12, 3.85 / 3.40 / 3.09 at n = 16 and 8.49 / 6.00 / 5.86 at n = 24; with
-// 320 problems four warps are best at every n (0.60 against 0.71 ms with one at
-// n = 8, 2.6 against 4.7 at n = 24).
+// alone, about seven problems per SM) or on 1280 problems of 48 stages.  For example, the
+// chunk up-sweeps of the long horizon (65536 stages in 1024 chunks) take 27 ms with two
+// warps per chunk against 37 with one; the affine chains of 1280 problems take 0.37 / 0.82
+// ms with 1 / 2 warps at n = 8, 0.72 / 0.72 / 0.86 with 1 / 2 / 4 at n = 16 and 1.26 /
+// 0.85 / 1.61 with 2 / 4 / 8 at n = 24 (160 problems at n = 32 0.68 / 0.55 with 4 / 8; of 320 problems 0.22 / 0.29 at n = 8, so they
+// keep the entry there); the stage elimination takes 2.2 / 3.8 ms with 1 / 2 at n = 8, 8.0
+// / 7.3 / 8.6 with 1 / 2 / 4 at n = 16 and 14.6 / 15.1 / 14.2 at n = 24.  The Riccati
+// sweep's products have thousands of independent integer multiply-adds per stage from
+// n = 16 on: 1.44 / 1.48 / 1.65 ms with 1 / 2 / 4 warps at n = 8, 2.56 / 2.09 / 2.23 at
+// n = 12, 3.85 / 3.40 / 3.09 at n = 16 and 8.49 / 6.00 / 5.86 at n = 24; with 320 problems
+// four warps are best at every n (0.60 against 0.71 ms with one at n = 8, 2.6 against 4.7
+// at n = 24).
 int team_for(const eclqr_handle *h, const void *kern, int ntasks, int n) {
   if (h->opt.team_warps != 0) return h->opt.team_warps;
   if (ntasks < h->sms) return kTeamWarps;
-  // warps below n1, from n1 up and from n2 up; few: warps with one to four tasks per SM (0: the
-  // entry, at least two -- 256 problems of 256 stages, n = 16: 37 ms with two, 42 with one, 49 with four)
-  static const struct { const void *fn; int warps, n1, warps1, n2, warps2, few; } table[] = {
-      {(const void *)k_riccati_down, 1, 12, 2, 16, 4, 4},
+  // warps below n1, from n1, n2 and n3 up; few: warps with one to four tasks per SM (-1: the
+  // entry, 0: the entry, at least two -- 256 problems of 256 stages, n = 16: 37 ms with two, 42 with one, 49 with four)
+  static const struct { const void *fn; int warps, few, n1, warps1, n2, warps2, n3, warps3; } table[] = {
+      {(const void *)k_riccati_down, 1, 4, 12, 2, 16, 4},
       {(const void *)k_riccati_down_f32, 1},     {(const void *)k_riccati_finish, 1},
-      {(const void *)k_elim, 1, 16, 4},          {(const void *)k_primal_down, 1, 24, 2},
-      {(const void *)k_dual_down, 1},            {(const void *)k_primal_stage, 1, 24, 2},
-      {(const void *)k_aff_down, 2, 24, 8},      {(const void *)k_dual_leaf, 1},
+      {(const void *)k_elim, 1, 0, 16, 2, 24, 4}, {(const void *)k_primal_down, 1, 0, 24, 2},
+      {(const void *)k_dual_down, 1},            {(const void *)k_primal_stage, 1, 0, 24, 2},
+      {(const void *)k_aff_down, 1, -1, 16, 2, 24, 4, 28, 8}, {(const void *)k_dual_leaf, 1},
       {(const void *)k_aff_prep, 1},             {(const void *)k_stage_lists, 1},
       {(const void *)k_dual_stage, 2},           {(const void *)k_param, 1},
       {(const void *)k_resid, 1},                {(const void *)k_pcorr, 1},
@@ -127,14 +127,18 @@ int team_for(const eclqr_handle *h, const void *kern, int ntasks, int n) {
       {(const void *)k_refine_prep, 1},          {(const void *)k_refine_gate, 1},
       {(const void *)k_refine_parts, 1},         {(const void *)k_refine_post, 1},
       {(const void *)k_rescue_prep, 1},          {(const void *)k_scan_check, 1},
+      {(const void *)k_set_costs, 1},
       {(const void *)k_terminal, 1},             {(const void *)k_dual_terminal, 1},
       {(const void *)k_lqr_up, 2},               {(const void *)k_primal_up, 1},
       {(const void *)k_dual_up, 2}};
   const bool many = ntasks >= kManyTasksPerSm * h->sms;
   for (const auto &e : table)
     if (e.fn == kern) {
-      const int w = e.n2 && n >= e.n2 ? e.warps2 : (e.n1 && n >= e.n1 ? e.warps1 : e.warps);
-      return many ? w : (e.few ? e.few : std::max(w, 2));
+      const int w = e.n3 && n >= e.n3   ? e.warps3
+                    : e.n2 && n >= e.n2 ? e.warps2
+                    : e.n1 && n >= e.n1 ? e.warps1
+                                        : e.warps;
+      return many || e.few < 0 ? w : (e.few ? e.few : std::max(w, 2));
     }
   return kTeamWarps;
 }
@@ -898,7 +902,7 @@ int eclqr_refine(eclqr_handle *h, const double *s0, double *x, double *u, double
       gz.slist = gh.slists + 2 * (size_t)gu.nstage;
       gz.scount = gh.scounts + 2;
       gz.c = h->zeros; gz.d = h->zeros; gz.e = h->zeros; gz.qv = h->rows.qv; gz.rv = h->rows.rv;
-      TRY(launch(h, k_set_costs, gz.nstage, smem_set_costs(gz.n, gz.m), gst, gz, smem_set_costs(gz.n, gz.m)));
+      TRY(launch(h, k_set_costs, gz.nstage, 0, gst, gz));
       TRY(run_solve(h, gh, gz, gst, h->zeros, t.x, t.u, corr));
       TRY(run_mult(h, gh, gz, gst, t.x, t.u, t.lam, t.mu, t.eta, t.alpha));
       // trial point w + dw, its residual, and the choice
@@ -971,7 +975,7 @@ int eclqr_set_costs(eclqr_handle *h, const eclqr_data *data, void *stream) {
     g.A = data->A; g.B = data->B; g.c = data->c; g.C = data->C; g.D = data->D; g.d = data->d;
     g.E = data->E; g.e = data->e; g.Q = data->Q; g.M = data->M; g.R = data->R; g.qv = data->qv; g.rv = data->rv;
     g.active = nullptr;
-    TRY(launch(h, k_set_costs, g.nstage, smem_set_costs(g.n, g.m), group_stream(h, gh, st), g, smem_set_costs(g.n, g.m)));
+    TRY(launch(h, k_set_costs, g.nstage, 0, group_stream(h, gh, st), g));
   }
   TRY(join_groups(h, st));
   h->solved = false;

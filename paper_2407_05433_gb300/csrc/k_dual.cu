@@ -482,23 +482,21 @@ __global__ void __launch_bounds__(256, 4) k_dual_leaf(Group g, double *lam, doub
 // Values reduced here are magnitudes or NaN.  The bit pattern of a non-negative
 // double orders like its value, and a positive NaN's pattern is above +inf's, so
 // an integer maximum over the patterns is a maximum that keeps NaN (fmax drops it).
-__device__ __forceinline__ double nanmax(double a, double b) { return (a > b || a != a) ? a : b; }
-
-__device__ __forceinline__ double team_max_keep_nan(double v) {
+__device__ __forceinline__ long long team_max_bits(long long k) {
   __shared__ long long red_bits[32];
-  long long k = __double_as_longlong(fabs(v));
 #pragma unroll
   for (int o = 16; o; o >>= 1) k = max(k, __shfl_xor_sync(kFull, k, o));
+  if (blockDim.x == 32) return k;
   if ((threadIdx.x & 31) == 0) red_bits[threadIdx.x >> 5] = k;
   __syncthreads();
   long long r = red_bits[0];
   for (int w = 1; w < (int)(blockDim.x >> 5); w++) r = max(r, red_bits[w]);
   __syncthreads();
-  return __longlong_as_double(r);
+  return r;
 }
 
-__device__ __forceinline__ void atomic_max_nonneg(double *addr, double v) {
-  atomicMax((unsigned long long *)addr, (unsigned long long)__double_as_longlong(v));
+__device__ __forceinline__ void atomic_max_bits(double *addr, long long k) {
+  atomicMax((unsigned long long *)addr, (unsigned long long)k);
 }
 
 // One stage of the residual rows (Sec. 7 sign convention, lambda_0 = -alpha):
@@ -529,20 +527,23 @@ __global__ void __launch_bounds__(256, 3) k_kkt(Group g, const double *s0, const
     const bool wr = rows.c != nullptr;
     const double *xi = x + P.ox + (size_t)i * n, *li = lam + P.olam + (size_t)i * n;
     const double *Q = g.Q + P.oQ + (size_t)i * n * n, *q = g.qv + P.oqv + (size_t)i * n;
-    double r0 = 0.0, r1 = 0.0, r2 = 0.0, r3 = 0.0;
+    // largest magnitudes, as bit patterns (see above team_max_bits): compared on the integer pipe
+    long long r0 = 0, r1 = 0, r2 = 0, r3 = 0;
+    auto bits = [](double v) { return __double_as_longlong(fabs(v)); };
     if (i == 0)
       for (int a = tid; a < n; a += TEAM) {
         const double v = xi[a] - s0[P.os0 + a];
-        r0 = nanmax(r0, fabs(v));
+        r0 = max(r0, bits(v));
         if (wr) rows.s0[P.os0 + a] = -v;
       }
     // state-only rows, normalised
     for (int k = tid; k < S.q; k += TEAM) {
       const double *Ek = g.E + P.oE + (size_t)(S.qrow + k) * n;
-      double e = g.e[P.oe + S.qrow + k], v = e, sc = nanmax(1.0, fabs(e));
+      double e = g.e[P.oe + S.qrow + k], v = e;
+      long long sc = max(bits(1.0), bits(e));
 #pragma unroll 2
-      for (int j = 0; j < n; j++) { v = fma(Ek[j], xi[j], v); sc = nanmax(sc, fabs(Ek[j])); }
-      r2 = nanmax(r2, fabs(v) / sc);
+      for (int j = 0; j < n; j++) { v = fma(Ek[j], xi[j], v); sc = max(sc, bits(Ek[j])); }
+      r2 = max(r2, bits(v / __longlong_as_double(sc)));
       if (wr) rows.e[P.oe + S.qrow + k] = v;
     }
     const double *etai = eta + P.oeta + S.qrow;
@@ -553,63 +554,60 @@ __global__ void __launch_bounds__(256, 3) k_kkt(Group g, const double *s0, const
       const double *rv = g.rv + P.orv + (size_t)i * m;
       const double *ui = u + P.ou + (size_t)i * m, *xn = x + P.ox + (size_t)(i + 1) * n;
       const double *ln = lam + P.olam + (size_t)(i + 1) * n, *mui = mu + P.omu + S.prow;
-      for (int a = tid; a < n; a += TEAM) {
-        const double v = kkt_dot(kkt_dot(c[a] - xn[a], A + a * n, 1, xi, n), B + a * m, 1, ui, m);
-        r1 = nanmax(r1, fabs(v));
-        if (wr) rows.c[P.oc + (size_t)i * n + a] = v;
-      }
-      for (int k = tid; k < S.p; k += TEAM) {
-        const double *Ck = g.C + P.oC + (size_t)(S.prow + k) * n, *Dk = g.D + P.oD + (size_t)(S.prow + k) * m;
-        double dd = g.d[P.od + S.prow + k], v = dd, sc = nanmax(1.0, fabs(dd));
-#pragma unroll 2
-        for (int j = 0; j < n; j++) { v = fma(Ck[j], xi[j], v); sc = nanmax(sc, fabs(Ck[j])); }
-#pragma unroll 2
-        for (int j = 0; j < m; j++) { v = fma(Dk[j], ui[j], v); sc = nanmax(sc, fabs(Dk[j])); }
-        r2 = nanmax(r2, fabs(v) / sc);
-        if (wr) rows.d[P.od + S.prow + k] = v;
-      }
-      for (int a = tid; a < m; a += TEAM) {
-        double v = kkt_dot(rv[a], Mm + a, m, xi, n);
-        v = kkt_dot(v, R + a * m, 1, ui, m);
-        v = kkt_dot(v, B + a, m, ln, n);
-        v = kkt_dot(v, g.D + P.oD + (size_t)S.prow * m + a, m, mui, S.p);
-        r3 = nanmax(r3, fabs(v));
-        if (wr) rows.rv[P.orv + (size_t)i * m + a] = v;
-      }
-      for (int a = tid; a < n; a += TEAM) {
-        double v = kkt_dot(q[a] + ((i == 0) ? alpha[P.oalpha + a] : -li[a]), Q + a * n, 1, xi, n);
-        v = kkt_dot(v, Mm + a * m, 1, ui, m);
-        v = kkt_dot(v, A + a, n, ln, n);
-        v = kkt_dot(v, g.C + P.oC + (size_t)S.prow * n + a, n, mui, S.p);
-        v = kkt_dot(v, g.E + P.oE + (size_t)S.qrow * n + a, n, etai, S.q);
-        r3 = nanmax(r3, fabs(v));
-        if (wr) rows.qv[P.oqv + (size_t)i * n + a] = v;
+      const double *Cs = g.C + P.oC + (size_t)S.prow * n, *Ds = g.D + P.oD + (size_t)S.prow * m;
+      // one lane per row, the blocks' rows side by side (an FP64 instruction costs its warp the
+      // same whatever its active lanes): state stationarity (n), control stationarity (m), dynamics
+      // (n), mixed rows (p), all with a product with x_i and one with u_i first
+      for (int r = tid; r < 2 * n + m + S.p; r += TEAM) {
+        const bool rx = r < n, ru = !rx && r < n + m, rd = !rx && !ru && r < 2 * n + m;
+        const int a = rx ? r : (ru ? r - n : (rd ? r - n - m : r - 2 * n - m));
+        double v = rx ? q[a] + ((i == 0) ? alpha[P.oalpha + a] : -li[a])
+                      : (ru ? rv[a] : (rd ? c[a] - xn[a] : g.d[P.od + S.prow + a]));
+        const double *px = rx ? Q + a * n : (ru ? Mm + a : (rd ? A + a * n : Cs + (size_t)a * n));
+        const double *pu = rx ? Mm + a * m : (ru ? R + a * m : (rd ? B + a * m : Ds + (size_t)a * m));
+        long long sc = max(bits(1.0), bits(v));
+        v = kkt_dot(kkt_dot(v, px, ru ? m : 1, xi, n), pu, 1, ui, m);
+        if (rx || ru) {
+          v = kkt_dot(v, rx ? A + a : B + a, rx ? n : m, ln, n);
+          v = kkt_dot(v, rx ? Cs + a : Ds + a, rx ? n : m, mui, S.p);
+          if (rx) v = kkt_dot(v, g.E + P.oE + (size_t)S.qrow * n + a, n, etai, S.q);
+          r3 = max(r3, bits(v));
+          if (wr) (rx ? rows.qv + P.oqv + (size_t)i * n : rows.rv + P.orv + (size_t)i * m)[a] = v;
+        } else if (rd) {
+          r1 = max(r1, bits(v));
+          if (wr) rows.c[P.oc + (size_t)i * n + a] = v;
+        } else {
+          for (int j = 0; j < n; j++) sc = max(sc, bits(px[j]));
+          for (int j = 0; j < m; j++) sc = max(sc, bits(pu[j]));
+          r2 = max(r2, bits(v / __longlong_as_double(sc)));
+          if (wr) rows.d[P.od + S.prow + a] = v;
+        }
       }
     } else {
       for (int a = tid; a < n; a += TEAM) {
         double v = kkt_dot(q[a] - li[a], Q + a * n, 1, xi, n);
         v = kkt_dot(v, g.E + P.oE + (size_t)S.qrow * n + a, n, etai, S.q);
-        r3 = nanmax(r3, fabs(v));
+        r3 = max(r3, bits(v));
         if (wr) rows.qv[P.oqv + (size_t)i * n + a] = v;
       }
     }
     if (resid == nullptr) return;
     if (parts != nullptr) {
-      r0 = team_max_keep_nan(r0);
-      r1 = team_max_keep_nan(r1);
-      r2 = team_max_keep_nan(r2);
-      r3 = team_max_keep_nan(r3);
+      r0 = team_max_bits(r0);
+      r1 = team_max_bits(r1);
+      r2 = team_max_bits(r2);
+      r3 = team_max_bits(r3);
       if (tid == 0) {
         double *pp = parts + 4 * (size_t)P.id;
-        atomic_max_nonneg(pp + 0, r0);
-        atomic_max_nonneg(pp + 1, r1);
-        atomic_max_nonneg(pp + 2, r2);
-        atomic_max_nonneg(pp + 3, r3);
-        atomic_max_nonneg(resid + P.id, nanmax(nanmax(r0, r1), nanmax(r2, r3)));
+        atomic_max_bits(pp + 0, r0);
+        atomic_max_bits(pp + 1, r1);
+        atomic_max_bits(pp + 2, r2);
+        atomic_max_bits(pp + 3, r3);
+        atomic_max_bits(resid + P.id, max(max(r0, r1), max(r2, r3)));
       }
     } else {
-      const double r = team_max_keep_nan(nanmax(nanmax(r0, r1), nanmax(r2, r3)));
-      if (tid == 0) atomic_max_nonneg(resid + P.id, r);
+      const long long r = team_max_bits(max(max(r0, r1), max(r2, r3)));
+      if (tid == 0) atomic_max_bits(resid + P.id, r);
     }
   });
 }

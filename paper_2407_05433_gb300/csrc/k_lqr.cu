@@ -33,7 +33,7 @@ __host__ int smem_lqr_level(int n) {
   const int rows = 8 * n, ldm = 3 * n + 1;
   return rows * ldm + 2 * rows + 2 * (ldm + rows) + n + 16;
 }
-__host__ int smem_riccati_finish(int n, int m) { return m * (n + m + 1) + m * (n + 1) + 8; }
+__host__ int smem_riccati_finish(int n, int m) { return m * (n + m + 1) + m * (n + 1) + m + 8; }
 __host__ int smem_aff(int n, int m) { return 2 * (n * n + n) + n * n + 5 * n + 2 * m + 8; }
 
 // Cost-relation slot layout (ld 2n + 1): constraint rows at 0 (CI_ROWS of them),
@@ -724,12 +724,15 @@ __global__ void k_riccati_finish(Group g, int per_task) {
       R[r * ldr + j] = Rv[r * ldr + j];
     }
     tsync();
-    // K, k:  R_vv [K | k] = -[R_vz | o_v]
+    // K, k:  R_vv [K | k] = -[R_vz | o_v]; the diagonal's reciprocals up front
+    double *inv = Kt + m * (n + 1);
+    for (int r = tid; r < mu; r += TEAM) inv[r] = 1.0 / R[r * ldr + r];
+    tsync();
     for (int c = tid; c <= nx; c += TEAM) {
       for (int r = mu - 1; r >= 0; r--) {
         double s0 = -R[r * ldr + mu + c];
         for (int l = r + 1; l < mu; l++) s0 = fma(-R[r * ldr + l], Kt[l * (n + 1) + c], s0);
-        Kt[r * (n + 1) + c] = s0 / R[r * ldr + r];
+        Kt[r * (n + 1) + c] = s0 * inv[r];
       }
     }
     for (int idx = tid; idx < mu * mu; idx += TEAM) {
@@ -1172,24 +1175,20 @@ __global__ void k_post_roll(Group g, int corr) {
     const double *zz = ws + (corr ? g.ws.dz : g.ws.z);
     const double *kk = ws + (corr ? g.ws.dv : g.ws.k);
     const double *pp = ws + (corr ? g.ws.pp : g.ws.p);
-    // v (or dv) -- computed into registers of the lanes then written
-    double myv = 0.0, mypi = 0.0;
-    const int r = tid;
-    if (r < mu) {
-      myv = kk[r];
-      for (int l = 0; l < nx; l++) myv = fma(ws[g.ws.K + r * n + l], zz[l], myv);
+    // one lane per row of K and of P
+    for (int r = tid; r < mu + nx; r += TEAM) {
+      const int a = r < mu ? r : r - mu;
+      const double *row = ws + (r < mu ? g.ws.K : g.ws.P) + a * n;
+      double s0 = r < mu ? kk[a] : pp[a];
+      for (int l = 0; l < nx; l++) s0 = fma(row[l], zz[l], s0);
+      double *o = ws + (r < mu ? g.ws.v : g.ws.pi) + a;
+      *o = corr ? *o + s0 : s0;
     }
-    if (r < nx) {
-      mypi = pp[r];
-      for (int l = 0; l < nx; l++) mypi = fma(ws[g.ws.P + r * n + l], zz[l], mypi);
-    }
-    tsync();
     if (!corr) {
-      if (r < m) ws[g.ws.v + r] = (r < mu) ? myv : 0.0;
-      if (r < n) ws[g.ws.pi + r] = (r < nx) ? mypi : 0.0;
+      for (int r = mu + tid; r < m; r += TEAM) ws[g.ws.v + r] = 0.0;
+      for (int r = nx + tid; r < n; r += TEAM) ws[g.ws.pi + r] = 0.0;
     } else {
-      if (r < mu) ws[g.ws.v + r] += myv;
-      if (r < nx) { ws[g.ws.pi + r] += mypi; ws[g.ws.z + r] += zz[r]; }
+      for (int r = tid; r < nx; r += TEAM) ws[g.ws.z + r] += zz[r];
     }
   });
 }
@@ -1221,26 +1220,25 @@ __global__ void k_resid(Group g, int per_task) {
     double *xs = sm, *us = xs + n, *lh = us + m, *ga = lh + n, *gb = ga + n;
     // T_i = I, t_i = 0 (te) or T_{i+1} = I (tne): the products with them are their other factor
     const bool te = wi[SI_TEYE] != 0, tne = !last && stage_wi(g, s + 1)[SI_TEYE] != 0;
-    for (int a = tid; a < n; a += TEAM) {
-      double s0 = ws[g.ws.t + a];
-      if (te) s0 = z[a];
-      else
-        for (int j = 0; j < nx; j++) s0 = fma(T[a * n + j], z[j], s0);
-      xs[a] = s0;
-    }
-    if (!last) {
-      for (int a = tid; a < m; a += TEAM) {
-        double s0 = ws[g.ws.y + a];
-        for (int j = 0; j < nx; j++) s0 = fma(Y[a * n + j], z[j], s0);
-        for (int j = 0; j < mu; j++) s0 = fma(Z[a * m + j], v[j], s0);
-        us[a] = s0;
-      }
-      for (int l = tid; l < n; l += TEAM) {
-        double s0 = 0.0;
-        if (tne) s0 = pin[l];
-        else
-          for (int j = 0; j < ny; j++) s0 = fma(Tn[l * n + j], pin[j], s0);
-        lh[l] = s0;                                               // T_{i+1} pi_{i+1}
+    // One lane per row, rows of different blocks side by side: an FP64 instruction costs its warp
+    // the same whatever its active lanes, so rows of three blocks in one instruction take the
+    // time of the longest.  p[j sp] x[j] summed onto v in order of j.
+    auto dot = [](double v, const double *p, int sp, const double *x, int len) {
+#pragma unroll 4
+      for (int j = 0; j < len; j++) v = fma(p[(size_t)j * sp], x[j], v);
+      return v;
+    };
+    // u_i (m rows), x_i (n), T_{i+1} pi_{i+1} (n)
+    const int mm = last ? 0 : m;
+    for (int r = tid; r < (last ? n : mm + 2 * n); r += TEAM) {
+      if (r < mm) {
+        us[r] = dot(dot(ws[g.ws.y + r], Y + r * n, 1, z, nx), Z + r * m, 1, v, mu);
+      } else if (r < mm + n) {
+        const int a = r - mm;
+        xs[a] = te ? z[a] : dot(ws[g.ws.t + a], T + a * n, 1, z, nx);
+      } else {
+        const int l = r - mm - n;
+        lh[l] = tne ? pin[l] : dot(0.0, Tn + l * n, 1, pin, ny);
       }
     }
     tsync();
@@ -1248,43 +1246,30 @@ __global__ void k_resid(Group g, int per_task) {
     const double *A = g.A + P.oA + (size_t)i * n * n, *B = g.B + P.oB + (size_t)i * n * m;
     const double *Mm = g.M + P.oM + (size_t)i * n * m, *R = g.R + P.oR + (size_t)i * m * m;
     const double *rv = g.rv + P.orv + (size_t)i * m;
-    for (int a = tid; a < n; a += TEAM) {
-      double s0 = q[a];
-      for (int j = 0; j < n; j++) s0 = fma(Q[a * n + j], xs[j], s0);
+    // a = g^x + A'lh (n rows), b = g^u + B'lh (m), the dynamics' residual (ny)
+    for (int r = tid; r < (last ? n : n + m + ny); r += TEAM) {
+      const bool ra = r < n, rb = !ra && r < n + m;
+      const int a = ra ? r : (rb ? r - n : r - n - m);
+      double s0 = ra ? q[a] : (rb ? rv[a] : ws[g.ws.cb + a] - zn[a]);
+      s0 = dot(s0, ra ? Q + a * n : (rb ? Mm + a : Ab + a * n), rb ? m : 1, ra || rb ? xs : z, ra || rb ? n : nx);
       if (!last) {
-        for (int j = 0; j < m; j++) s0 = fma(Mm[a * m + j], us[j], s0);
-        for (int l = 0; l < n; l++) s0 = fma(A[l * n + a], lh[l], s0);
+        s0 = dot(s0, ra ? Mm + a * m : (rb ? R + a * m : Bb + a * m), 1, ra || rb ? us : v, ra || rb ? m : mu);
+        if (ra || rb) s0 = dot(s0, ra ? A + a : B + a, ra ? n : m, lh, n);
       }
-      ga[a] = s0;
+      if (ra) ga[a] = s0;
+      else if (rb) gb[a] = s0;
+      else ws[g.ws.rc + a] = s0;
     }
-    if (!last)
-      for (int a = tid; a < m; a += TEAM) {
-        double s0 = rv[a];
-        for (int j = 0; j < n; j++) s0 = fma(Mm[j * m + a], xs[j], s0);
-        for (int j = 0; j < m; j++) s0 = fma(R[a * m + j], us[j], s0);
-        for (int l = 0; l < n; l++) s0 = fma(B[l * m + a], lh[l], s0);
-        gb[a] = s0;
-      }
     tsync();
-    for (int r = tid; r < nx; r += TEAM) {
-      double s0 = -pi[r];
-      if (te) s0 = ga[r] - pi[r];
-      else
-        for (int l = 0; l < n; l++) s0 = fma(T[l * n + r], ga[l], s0);
-      if (!last)
-        for (int l = 0; l < m; l++) s0 = fma(Y[l * n + r], gb[l], s0);
-      ws[g.ws.rq + r] = s0;
-    }
-    for (int r = tid; r < mu; r += TEAM) {
-      double s0 = 0.0;
-      for (int l = 0; l < m; l++) s0 = fma(Z[l * m + r], gb[l], s0);
-      ws[g.ws.rr + r] = s0;
-    }
-    for (int r = tid; r < ny; r += TEAM) {
-      double s0 = ws[g.ws.cb + r] - zn[r];
-      for (int l = 0; l < nx; l++) s0 = fma(Ab[r * n + l], z[l], s0);
-      for (int l = 0; l < mu; l++) s0 = fma(Bb[r * m + l], v[l], s0);
-      ws[g.ws.rc + r] = s0;
+    for (int r = tid; r < nx + mu; r += TEAM) {
+      double s0;
+      if (r < nx) {
+        s0 = te ? ga[r] - pi[r] : dot(-pi[r], T + r, n, ga, n);
+        if (!last) s0 = dot(s0, Y + r, n, gb, m);
+        ws[g.ws.rq + r] = s0;
+      } else {
+        ws[g.ws.rr + r - nx] = dot(0.0, Z + r - nx, m, gb, m);
+      }
     }
   });
 }
@@ -1321,19 +1306,22 @@ __global__ void k_pcorr(Group g, int per_task) {
     }
     tsync();
     // dv = -H_uu^{-1} hu with H_uu = L L' (L = Ls, lower): forward then backward
-    // substitution by the first warp, lane a holding row a (mu <= 16), column by column
+    // substitution by the first warp, lane a holding row a (mu <= 16), column by column; the
+    // diagonal's reciprocals up front, one division for all lanes instead of one per column (a
+    // division is about fifteen FP64 instructions)
     if (tid < 32) {
       const int a = tid;
       double x = (a < mu) ? hu[a] : 0.0;
+      const double inv = (a < mu) ? 1.0 / Ls[a * m + a] : 0.0;
       for (int l = 0; l < mu; l++) {
-        const double xl = __shfl_sync(kFull, x, l) / Ls[l * m + l];
-        if (a == l) x = xl;
-        else if (a > l && a < mu) x = fma(-Ls[a * m + l], xl, x);
+        if (a == l) x *= inv;
+        const double xl = __shfl_sync(kFull, x, l);
+        if (a > l && a < mu) x = fma(-Ls[a * m + l], xl, x);
       }
       for (int l = mu - 1; l >= 0; l--) {
-        const double xl = __shfl_sync(kFull, x, l) / Ls[l * m + l];
-        if (a == l) x = xl;
-        else if (a < l) x = fma(-Ls[l * m + a], xl, x);
+        if (a == l) x *= inv;
+        const double xl = __shfl_sync(kFull, x, l);
+        if (a < l) x = fma(-Ls[l * m + a], xl, x);
       }
       if (a < mu) ws[g.ws.dv + a] = -x;
     }

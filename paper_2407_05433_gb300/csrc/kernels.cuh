@@ -14,7 +14,6 @@ __host__ int smem_lqr_up(int n, int m);
 __host__ int smem_lqr_level(int n);
 __host__ int smem_riccati(int n, int m);
 __host__ int smem_riccati_finish(int n, int m);
-__host__ int smem_set_costs(int n, int m);
 __host__ int smem_primal_stage(int n, int m, int wmax);
 __host__ int smem_aff(int n, int m);
 __host__ int smem_dual_stage(int n, int m);
@@ -59,7 +58,7 @@ __global__ void k_dual_down(Group g, int fin, int per_task);
 __global__ void k_dual_root(Group g, int per_task);
 __global__ void __launch_bounds__(256, 4) k_dual_leaf(Group g, double *lam, double *mu, double *eta, double *alpha, int per_task);
 __global__ void k_param_grads(Group g, Sol w, Sol wb, GradOut o);
-__global__ void k_set_costs(Group g, int per_task);
+__global__ void k_set_costs(Group g);
 __global__ void k_kkt(Group g, const double *s0, const double *x, const double *u, const double *lam,
                       const double *mu, const double *eta, const double *alpha, KktRows rows, double *resid,
                       double *parts);
