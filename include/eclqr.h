@@ -239,11 +239,12 @@ int eclqr_kkt_residual_parts(eclqr_handle *h, const double *s0, const double *x,
  *   When a pass ran, the offset-dependent parts of the workspace belong to
  *   the last correction: eclqr_solve and eclqr_multipliers return
  *   ECLQR_ESTATE until the next eclqr_build or eclqr_set_costs.
- *   Outside a stream capture the call waits, once per pass, for a 4-byte
- *   flag telling whether any problem takes part, and returns when none does
- *   (so it is host-synchronous); on a capturing stream it records all
- *   opt.kkt_refine passes, whose kernels return at once for the problems
- *   that take no part. */
+ *   Outside a stream capture the call waits, once per pass, for 12 bytes of
+ *   flags telling whether any problem takes part, and returns when none does
+ *   (so it is host-synchronous); on a capturing stream it records one pass as
+ *   the body of a conditional node that a replay runs while some problem takes
+ *   part (where the graph takes no such node, all opt.kkt_refine passes, whose
+ *   kernels return at once for the problems that take no part). */
 int eclqr_refine(eclqr_handle *h, const double *s0, double *x, double *u, double *lam, double *mu,
                  double *eta, double *alpha, double *resid, int32_t *status, void *stream);
 
@@ -257,8 +258,8 @@ int eclqr_riccati_fp64_flags(eclqr_handle *h, int32_t *flags, void *stream);
  * build, into device int32 arrays. */
 int eclqr_reduced_dims(eclqr_handle *h, int32_t *nbar, int32_t *mbar, void *stream);
 
-/* Kernel launches issued through this handle since eclqr_create (host counter,
- * for launch accounting). */
+/* Kernel launches issued or recorded through this handle since eclqr_create (host
+ * counter, for launch accounting; a captured refinement's loop counts once). */
 int64_t eclqr_launch_count(const eclqr_handle *h);
 
 /* Measurement hooks (not part of the method).

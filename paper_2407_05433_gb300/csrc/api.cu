@@ -31,6 +31,7 @@ constexpr int kListCtasPerSm = 32;    // CTAs per SM of a per-stage launch over 
 struct GroupHost {
   Group g;
   cudaStream_t s = nullptr;     // the group's own stream when the batch has several groups
+  cudaStream_t loop_s = nullptr;  // its stream inside the loop of a captured refinement
   cudaEvent_t done = nullptr;   // records the end of the group's work on s
   int maxnch = 0;
   int levels = 0;
@@ -73,7 +74,10 @@ struct eclqr_handle {
   RefineMasks mk{};
   double *parts = nullptr, *tparts = nullptr;  // residual parts of the point and of the trial point
   double *zeros = nullptr;  // offsets of the corrections with homogeneous constraints
-  int *any = nullptr;       // device: some problem takes part in the pass
+  int *any = nullptr;       // device: some problem takes part in the pass, rebuilds, takes the cheap
+                            // correction; passes of a captured refinement so far
+  cudaStream_t loop_s = nullptr;  // the capturing stream of a captured refinement's loop
+  bool in_loop = false;           // the launches being recorded are that loop's
   int *fp64 = nullptr;      // mixed precision: per-problem flags of the Riccati sweep's precision
   int *any_host = nullptr;  // pinned host copy of it
   bool stale = false;  // the offset-dependent factors are a correction's (after eclqr_refine)
@@ -236,16 +240,16 @@ int fork_groups(eclqr_handle *h, cudaStream_t st) {
   if (h->groups.size() < 2) return ECLQR_OK;
   if (cudaEventRecord(h->fork, st) != cudaSuccess) return ECLQR_ECUDA;
   for (auto &gh : h->groups)
-    if (cudaStreamWaitEvent(gh.s, h->fork, 0) != cudaSuccess) return ECLQR_ECUDA;
+    if (cudaStreamWaitEvent(h->in_loop ? gh.loop_s : gh.s, h->fork, 0) != cudaSuccess) return ECLQR_ECUDA;
   return ECLQR_OK;
 }
 cudaStream_t group_stream(const eclqr_handle *h, const GroupHost &gh, cudaStream_t st) {
-  return h->groups.size() < 2 ? st : gh.s;
+  return h->groups.size() < 2 ? st : (h->in_loop ? gh.loop_s : gh.s);
 }
 int join_groups(eclqr_handle *h, cudaStream_t st) {
   if (h->groups.size() < 2) return ECLQR_OK;
   for (auto &gh : h->groups) {
-    if (cudaEventRecord(gh.done, gh.s) != cudaSuccess) return ECLQR_ECUDA;
+    if (cudaEventRecord(gh.done, h->in_loop ? gh.loop_s : gh.s) != cudaSuccess) return ECLQR_ECUDA;
     if (cudaStreamWaitEvent(st, gh.done, 0) != cudaSuccess) return ECLQR_ECUDA;
   }
   return ECLQR_OK;
@@ -590,7 +594,7 @@ int eclqr_create(const eclqr_desc *d, const eclqr_options *opt, eclqr_handle **o
     const size_t o_c = take(L.c, 8), o_d = take(L.d, 8), o_e = take(L.e, 8), o_qv = take(L.qv, 8),
                  o_rv = take(L.rv, 8), o_s0 = take(L.s0, 8), o_x = take(L.x, 8), o_u = take(L.u, 8),
                  o_lam = take(L.lam, 8), o_mu = take(L.mu, 8), o_eta = take(L.eta, 8), o_al = take(L.alpha, 8),
-                 o_cs = take(P, 4), o_tr = take(P, 8), o_ac = take(P, 4), o_any = take(1, 4),
+                 o_cs = take(P, 4), o_tr = take(P, 8), o_ac = take(P, 4), o_any = take(4, 4),
                  o_fu = take(P, 4), o_ch = take(P, 4), o_pa = take(4 * (size_t)P, 8), o_tp = take(4 * (size_t)P, 8),
                  o_z = take(std::max({L.c, L.d, L.e, L.s0}), 8);
     if (cudaMalloc(&h->rmem, off) != cudaSuccess || cudaMemset(h->rmem, 0, off) != cudaSuccess) {
@@ -609,10 +613,17 @@ int eclqr_create(const eclqr_desc *d, const eclqr_options *opt, eclqr_handle **o
     h->tparts = (double *)(b + o_tp);
     h->zeros = (double *)(b + o_z);
     h->any = (int *)(b + o_any);
-    if (cudaMallocHost(&h->any_host, sizeof(int)) != cudaSuccess) {
+    if (cudaMallocHost(&h->any_host, 3 * sizeof(int)) != cudaSuccess) {
       h->any_host = nullptr;
       eclqr_destroy(h);
       return ECLQR_ENOMEM;
+    }
+    bool ok = cudaStreamCreateWithFlags(&h->loop_s, cudaStreamNonBlocking) == cudaSuccess;
+    for (auto &gh : h->groups)
+      ok = ok && (h->groups.size() < 2 || cudaStreamCreateWithFlags(&gh.loop_s, cudaStreamNonBlocking) == cudaSuccess);
+    if (!ok) {
+      eclqr_destroy(h);
+      return ECLQR_ECUDA;
     }
   }
   if (h->opt.riccati_fp32 && cudaMalloc(&h->fp64, sizeof(int) * (size_t)P) != cudaSuccess) {
@@ -839,37 +850,36 @@ int eclqr_refine(eclqr_handle *h, const double *s0, double *x, double *u, double
   const Sol tc{t.x, t.u, t.lam, t.mu, t.eta, t.alpha};
   const RefineMasks mk = h->mk;
   const int corr = h->opt.corr_refine < 0 ? h->opt.refine : h->opt.corr_refine;
-  // outside a stream capture the passes stop as soon as no problem takes part (one 4-byte read
-  // back per pass); a captured sequence holds every pass, whose kernels return at once for
-  // problems that take no part
+  // Outside a stream capture the passes stop as soon as no problem takes part (one 12-byte read
+  // back per pass, which also tells whether a pass rebuilds).  On a capturing stream the pass is
+  // recorded once, as the body of a conditional WHILE node whose condition k_refine_loop sets, so
+  // that a replay ends the same way (a 64-stage n = 4 problem that needs no pass: 1.9 ms with the
+  // eight passes recorded one after the other, 1.0 ms in the loop); where the stream's graph takes
+  // no conditional node, every pass is recorded, and its kernels return at once for problems that
+  // take no part.
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) return ECLQR_ECUDA;
   const bool eager = cap == cudaStreamCaptureStatusNone;
   bool corrected = false;
-  // up to opt.kkt_refine passes; first = 1 starts every problem afresh, 0 continues the problems
-  // that mk.active marks
-  auto passes = [&](int first) -> int {
-  for (int k = 0; k < h->opt.kkt_refine; k++) {
-    if (cudaMemsetAsync(h->any, 0, sizeof(int), st) != cudaSuccess) return ECLQR_ECUDA;
-    TRY(fork_groups(h, st));
+  // the masks of the next pass
+  auto prepare = [&](cudaStream_t q, int first) -> int {
+    if (cudaMemsetAsync(h->any, 0, 3 * sizeof(int), q) != cudaSuccess) return ECLQR_ECUDA;
+    TRY(fork_groups(h, q));
     for (auto &gh : h->groups) {
       Group gu = gh.g;  // unmasked, for the per-problem bookkeeping
       gu.active = nullptr;
-      TRY(launch(h, k_refine_prep, gu.nprob, 0, group_stream(h, gh, st), gu, (const int32_t *)status,
+      TRY(launch(h, k_refine_prep, gu.nprob, 0, group_stream(h, gh, q), gu, (const int32_t *)status,
                  (const double *)resid, (const double *)h->parts, mk, h->cstatus, h->tresid, h->tparts, h->opt.refine_tol,
-                 k == 0 ? first : 0, h->any));
+                 first, h->any));
     }
-    if (eager) {
-      TRY(join_groups(h, st));
-      if (cudaMemcpyAsync(h->any_host, h->any, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-          cudaStreamSynchronize(st) != cudaSuccess)
-        return ECLQR_ECUDA;
-      if (*h->any_host == 0) break;
-      TRY(fork_groups(h, st));
-    }
-    corrected = true;
+    return join_groups(h, q);
+  };
+  // one pass over the problems that the masks mark; full, cheap: some problem may rebuild, may take
+  // the cheap correction
+  auto pass = [&](cudaStream_t q, bool full, bool cheap) -> int {
+    TRY(fork_groups(h, q));
     for (auto &gh : h->groups) {
-      const cudaStream_t gst = group_stream(h, gh, st);
+      const cudaStream_t gst = group_stream(h, gh, q);
       Group gu = gh.g;
       gu.active = nullptr;
       // the stages of the problems that take part, of those that rebuild and of those that
@@ -892,9 +902,11 @@ int eclqr_refine(eclqr_handle *h, const double *s0, double *x, double *u, double
       gf.slist = gh.slists + gu.nstage;
       gf.scount = gh.scounts + 1;
       gf.c = h->rows.c; gf.d = h->rows.d; gf.e = h->rows.e; gf.qv = h->rows.qv; gf.rv = h->rows.rv;
-      TRY(run_build(h, gh, gf, gst, false));
-      TRY(run_solve(h, gh, gf, gst, h->rows.s0, t.x, t.u, corr));
-      TRY(run_mult(h, gh, gf, gst, t.x, t.u, t.lam, t.mu, t.eta, t.alpha));
+      if (full) {
+        TRY(run_build(h, gh, gf, gst, false));
+        TRY(run_solve(h, gh, gf, gst, h->rows.s0, t.x, t.u, corr));
+        TRY(run_mult(h, gh, gf, gst, t.x, t.u, t.lam, t.mu, t.eta, t.alpha));
+      }
       // primal rows within it: homogeneous constraints, so the build's factors serve as they
       // are and only the linear costs change (as for the adjoint, eclqr_set_costs)
       Group gz = g;
@@ -902,9 +914,11 @@ int eclqr_refine(eclqr_handle *h, const double *s0, double *x, double *u, double
       gz.slist = gh.slists + 2 * (size_t)gu.nstage;
       gz.scount = gh.scounts + 2;
       gz.c = h->zeros; gz.d = h->zeros; gz.e = h->zeros; gz.qv = h->rows.qv; gz.rv = h->rows.rv;
-      TRY(launch(h, k_set_costs, gz.nstage, 0, gst, gz));
-      TRY(run_solve(h, gh, gz, gst, h->zeros, t.x, t.u, corr));
-      TRY(run_mult(h, gh, gz, gst, t.x, t.u, t.lam, t.mu, t.eta, t.alpha));
+      if (cheap) {
+        TRY(launch(h, k_set_costs, gz.nstage, 0, gst, gz));
+        TRY(run_solve(h, gh, gz, gst, h->zeros, t.x, t.u, corr));
+        TRY(run_mult(h, gh, gz, gst, t.x, t.u, t.lam, t.mu, t.eta, t.alpha));
+      }
       // trial point w + dw, its residual, and the choice
       TRY(launch(h, k_refine_gate, gu.nprob, 0, gst, gu, (const int32_t *)h->cstatus, mk.active));
       TRY(launch(h, k_refine_trial, g.nstage, 0, gst, g, w, t));
@@ -916,9 +930,72 @@ int eclqr_refine(eclqr_handle *h, const double *s0, double *x, double *u, double
                  (const double *)h->tparts, (const double *)resid, (const double *)h->tresid));
       TRY(launch(h, k_refine_post, gu.nprob, 0, gst, gu, resid, (const double *)h->tresid, mk.active));
     }
-    TRY(join_groups(h, st));
-  }
-  return ECLQR_OK;
+    return join_groups(h, q);
+  };
+  // the passes as the body of a WHILE node; false where the capturing graph takes none (nothing is
+  // recorded then)
+  auto loop = [&](int first, int &rc) -> bool {
+    cudaGraph_t graph = nullptr;
+    cudaGraphConditionalHandle cond;
+    if (cudaStreamGetCaptureInfo(st, &cap, nullptr, &graph, nullptr, nullptr, nullptr) != cudaSuccess ||
+        cudaGraphConditionalHandleCreate(&cond, graph, 0, cudaGraphCondAssignDefault) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    rc = [&]() -> int {
+      TRY(prepare(st, first));
+      k_refine_loop<<<1, 1, 0, st>>>(cond, h->any, h->opt.kkt_refine, 1);
+      const cudaGraphNode_t *deps = nullptr;
+      const cudaGraphEdgeData *edges = nullptr;
+      size_t ndeps = 0;
+      if (cudaStreamGetCaptureInfo(st, &cap, nullptr, &graph, &deps, &edges, &ndeps) != cudaSuccess) return ECLQR_ECUDA;
+      cudaGraphNodeParams np = {};
+      np.type = cudaGraphNodeTypeConditional;
+      np.conditional.handle = cond;
+      np.conditional.type = cudaGraphCondTypeWhile;
+      np.conditional.size = 1;
+      cudaGraphNode_t node;
+      if (cudaGraphAddNode(&node, graph, deps, edges, ndeps, &np) != cudaSuccess ||
+          cudaStreamUpdateCaptureDependencies(st, &node, nullptr, 1, cudaStreamSetCaptureDependencies) != cudaSuccess)
+        return ECLQR_ECUDA;
+      cudaGraph_t body = np.conditional.phGraph_out[0];
+      if (cudaStreamBeginCaptureToGraph(h->loop_s, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed) !=
+          cudaSuccess)
+        return ECLQR_ECUDA;
+      h->in_loop = true;
+      int r = pass(h->loop_s, true, true);
+      if (r == ECLQR_OK) r = prepare(h->loop_s, 0);
+      if (r == ECLQR_OK) k_refine_loop<<<1, 1, 0, h->loop_s>>>(cond, h->any, h->opt.kkt_refine, 0);
+      h->in_loop = false;
+      if (cudaStreamEndCapture(h->loop_s, &body) != cudaSuccess) return ECLQR_ECUDA;
+      h->launches += 2;
+      return r;
+    }();
+    return true;
+  };
+  // up to opt.kkt_refine passes; first = 1 starts every problem afresh, 0 continues the problems
+  // that mk.active marks
+  auto passes = [&](int first) -> int {
+    int rc = ECLQR_OK;
+    if (!eager) {
+      corrected = true;
+      if (loop(first, rc)) return rc;
+    }
+    for (int k = 0; k < h->opt.kkt_refine; k++) {
+      TRY(prepare(st, k == 0 ? first : 0));
+      bool full = true, cheap = true;
+      if (eager) {
+        if (cudaMemcpyAsync(h->any_host, h->any, 3 * sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+            cudaStreamSynchronize(st) != cudaSuccess)
+          return ECLQR_ECUDA;
+        if (h->any_host[0] == 0) break;
+        full = h->any_host[1] != 0;
+        cheap = h->any_host[2] != 0;
+      }
+      corrected = true;
+      TRY(pass(st, full, cheap));
+    }
+    return ECLQR_OK;
   };
   TRY(passes(1));
   if (h->fp64) {
@@ -1049,9 +1126,11 @@ void eclqr_destroy(eclqr_handle *h) {
   for (auto &gh : h->groups) {
     cudaFree(gh.dmem);
     if (gh.s) cudaStreamDestroy(gh.s);
+    if (gh.loop_s) cudaStreamDestroy(gh.loop_s);
     if (gh.done) cudaEventDestroy(gh.done);
   }
   if (h->fork) cudaEventDestroy(h->fork);
+  if (h->loop_s) cudaStreamDestroy(h->loop_s);
   if (h->rmem) cudaFree(h->rmem);
   if (h->any_host) cudaFreeHost(h->any_host);
   if (h->fp64) cudaFree(h->fp64);

@@ -51,8 +51,8 @@ __global__ void k_check_inputs(Group g) {
 // residual start at 0.  A problem whose primal parts (initial condition,
 // dynamics, equality rows) are within tol takes the correction with homogeneous
 // constraints (full[id] = 0), which reuses the build's offset-free factors;
-// the others rebuild on the residual rows (full[id] = 1).  *any is set when some
-// problem takes part.
+// the others rebuild on the residual rows (full[id] = 1).  any[0] is set when some
+// problem takes part, any[1] when one rebuilds, any[2] when one takes the cheap correction.
 __global__ void k_refine_prep(Group g, const int32_t *status, const double *resid, const double *parts,
                               RefineMasks mk, int32_t *cstatus, double *tresid, double *tparts, double tol, int first,
                               int *any) {
@@ -69,7 +69,18 @@ __global__ void k_refine_prep(Group g, const int32_t *status, const double *resi
   cstatus[id] = ST_OK;
   tresid[id] = 0.0;
   for (int k = 0; k < 4; k++) tparts[4 * (size_t)id + k] = 0.0;
-  if (on) *any = 1;
+  if (on) {
+    any[0] = 1;
+    any[full ? 1 : 2] = 1;
+  }
+}
+
+// A captured refinement's loop condition: another pass runs while some problem takes part, up to
+// most passes.  first starts the count in any[3].
+__global__ void k_refine_loop(cudaGraphConditionalHandle loop, int *any, int most, int first) {
+  const int k = first ? 0 : any[3];
+  any[3] = k + 1;
+  cudaGraphSetConditional(loop, any[0] != 0 && k < most ? 1u : 0u);
 }
 
 // Per problem, after k_refine_prep: the stages of the problems in each of the

@@ -69,6 +69,7 @@ __global__ void k_stage_lists(Group g, RefineMasks mk, int *lists, int *counts);
 __global__ void k_refine_prep(Group g, const int32_t *status, const double *resid, const double *parts,
                               RefineMasks mk, int32_t *cstatus, double *tresid, double *tparts, double tol,
                               int first, int *any);
+__global__ void k_refine_loop(cudaGraphConditionalHandle loop, int *any, int most, int first);
 __global__ void k_refine_parts(Group g, const int *active, double *parts, const double *tparts,
                                const double *resid, const double *tresid);
 __global__ void k_refine_gate(Group g, const int32_t *cstatus, int *active);

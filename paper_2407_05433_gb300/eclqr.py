@@ -343,7 +343,7 @@ class Batch:
         The graph keeps the current device pointers: refresh the inputs in place (self.d)
         and call replay().  A first eager pass on a side stream sets every kernel's
         shared-memory attribute before capture.  Returns the number of kernel launches
-        one replay performs."""
+        recorded; those of the refinement's loop run once per pass that a replay needs."""
         torch = self.torch
         side = torch.cuda.Stream(self.device)
         side.wait_stream(torch.cuda.current_stream(self.device))
