@@ -23,6 +23,9 @@ namespace {
 // dynamic shared memory per task: the 227 KB opt-in limit less room for the
 // static scratch of the team reductions and the Householder core (< 8 KB)
 constexpr int kMaxSmemBytes = 219 * 1024;
+// doubles of static scratch that the multiplier kernels once had: the documented limit on the row
+// counts includes them, so that it stays where it is
+constexpr int kHeldScratch = 304;
 constexpr int kTeamWarps = 4;  // default team: one warp per SM sub-partition
 constexpr int kManyTasksPerSm = 4;  // a launch with at least this many tasks per SM takes the table's team
 constexpr int kPersistCtasPerSm = 8;  // default CTAs per SM of a persistent launch
@@ -147,11 +150,11 @@ int team_for(const eclqr_handle *h, const void *kern, int ntasks, int n) {
   return kTeamWarps;
 }
 
-// the state dimension of the group a launch works on (every kernel's first argument)
-inline int group_n(const Group &g) { return g.n; }
+// the group a launch works on (every kernel's first argument)
+inline const Group &group_of(const Group &g) { return g; }
 template <typename A0, typename... Rest>
-int group_n(const A0 &a0, const Rest &...) {
-  return group_n(a0);
+const Group &group_of(const A0 &a0, const Rest &...) {
+  return group_of(a0);
 }
 
 // grid CTAs (teams of team_for warps, chosen for ntasks tasks), with per_task
@@ -171,7 +174,10 @@ int launch_grid(eclqr_handle *h, void (*kern)(KArgs...), int ntasks, int grid, i
   }
   const bool timed = h->timed == (const void *)kern && h->nev + 2 <= (int)h->ev.size();
   if (timed) cudaEventRecord(h->ev[h->nev], st);
-  kern<<<grid, 32 * team_for(h, (const void *)kern, ntasks, group_n(args...)), smem, st>>>(args...);
+  const Group &g = group_of(args...);
+  // every problem has one slot more than it has chunks to sweep
+  const int work = (const void *)kern == (const void *)k_riccati_down ? g.nslot - g.nprob : ntasks;
+  kern<<<grid, 32 * team_for(h, (const void *)kern, work, g.n), smem, st>>>(args...);
   if (timed) {
     cudaEventRecord(h->ev[h->nev + 1], st);
     h->nev += 2;
@@ -460,8 +466,8 @@ int eclqr_create(const eclqr_desc *d, const eclqr_options *opt, eclqr_handle **o
           {(const void *)k_riccati_finish, smem_riccati_finish(n, m)}, {(const void *)k_aff_up, sa},
           {(const void *)k_aff_level, sa}, {(const void *)k_aff_down, sa}, {(const void *)k_resid, 3 * n + 2 * m},
           {(const void *)k_pcorr, n + m + m * m}, {(const void *)k_dual_stage, smem_dual_stage(n, m)},
-          {(const void *)k_dual_terminal, sdw}, {(const void *)k_dual_up, sdw}, {(const void *)k_dual_down, sdw},
-          {(const void *)k_dual_root, sdw}, {(const void *)k_dual_leaf, smem_dual_leaf(n, m, wmax)}};
+          {(const void *)k_dual_terminal, sdw}, {(const void *)k_dual_up, sdw}, {(const void *)k_dual_down, sdw + kHeldScratch},
+          {(const void *)k_dual_root, sdw + kHeldScratch}, {(const void *)k_dual_leaf, smem_dual_leaf(n, m, wmax) + kHeldScratch}};
       int optin = 0;
       int rc = (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device) == cudaSuccess)
                    ? ECLQR_OK : ECLQR_ECUDA;
@@ -681,7 +687,7 @@ int run_build(eclqr_handle *h, GroupHost &gh, const Group &g, cudaStream_t gst, 
   TRY(launch(h, k_param, g.nstage, sp, gst, g, sp));
   TRY(launch(h, k_elim, g.nstage, se, gst, g, se));
   const int su = smem_lqr_up(n, m), slv = smem_lqr_level(n), sr = smem_riccati(n, m);
-  TRY(launch(h, k_lqr_up, g.nslot, su, gst, g, su));
+  if (gh.levels > 0 || g.fp64) TRY(launch(h, k_lqr_up, g.nslot, su, gst, g, su));
   src = 0;
   for (int k = 0; k < gh.levels; k++, src ^= 1) TRY(launch(h, k_lqr_level, g.nslot, slv, gst, g, src, 1 << k, slv));
   TRY(launch_sweep(h, gh.queue, k_riccati_down, g.nslot, sr, gst, g, src, sr));

@@ -16,11 +16,23 @@
 // the highest (int2: x = high, y = low; int4: x = lowest ... w = highest).
 #pragma once
 #include <stdint.h>
-#include "la.cuh"
 
 namespace eclqr {
 
 typedef __int128 i128;
+
+// single-precision approximations (PTX rsqrt.approx / rcp.approx, relative
+// error about 2^-22), used only as seeds and for small integer quotients
+__device__ __forceinline__ float rsqrt_seed(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rcp_seed(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 
 constexpr int kFxA = 57;          // fractional bits of a two-limb entry
 constexpr int kFxP = 114;         // fractional bits of a four-limb entry
@@ -130,6 +142,23 @@ __device__ __forceinline__ long long fx_rcp(unsigned long long u) {
   const long long eh = e >> 20;
   const long long corr = e + ((eh * eh) >> 21);
   return ((long long)r0 << 26) + __mul64hi(corr << 20, (long long)r0 << 9);
+}
+
+// The scalars of FP64 factorizations on the integer pipe: the dozen dependent FP64 instructions of a
+// seeded FP64 step occupy the sub-partition for 64 to 76 cycles each.  A positive normal d is
+// 2^(2 h) s 2^-62 with s in [2^62, 2^64); ok is false, with the results unusable, unless d is positive
+// and within [2^-1000, 2^1001).
+__device__ __forceinline__ unsigned long long fx_even(double d, int &h, bool &ok) {
+  const int hi = __double2hiint(d), ex = ((hi >> 20) & 0x7ff) - 1023, odd = ex & 1;
+  h = (ex - odd) >> 1;
+  ok = hi > 0 && ex >= -1000 && ex <= 1000;
+  return ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32 | (unsigned)__double2loint(d)) << (10 + odd);
+}
+// d^(-1/2): relative error below 2^-59 before the rounding to FP64
+__device__ __forceinline__ double fx_rsqrt_f64(double d, bool &ok) {
+  int h;
+  const unsigned long long s = fx_even(d, h, ok);
+  return fx_to((long long)fx_rsqrt(s), -62 - h);
 }
 
 // sums of products of four-limb by two-limb entries: c[3] 2^116 + c[2] 2^87 + c[1] 2^58 + c[0] 2^29,

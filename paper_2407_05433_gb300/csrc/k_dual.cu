@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(256, 3) k_dual_stage(Group g, const double *x,
       X[l * n + b] = v;
     }
     tsync();
-    wgemm<true, false>(r0, r1, n, 1.0, U, n, X, n, 0.0, ws + g.ws.UA, n);   // U' A' U1
+    wgemm<true, false>(r0, r1, n, U, n, X, n, 0, ws + g.ws.UA, n);   // U' A' U1
     for (int idx = tid; idx < m * r1; idx += TEAM) {
       int a = idx / r1, b = idx - a * r1;
       double v = 0.0;

@@ -33,7 +33,7 @@ __host__ int smem_lqr_level(int n) {
   const int rows = 8 * n, ldm = 3 * n + 1;
   return rows * ldm + 2 * rows + 2 * (ldm + rows) + n + 16;
 }
-__host__ int smem_riccati_finish(int n, int m) { return m * (n + m + 1) + m * (n + 1) + m + 8; }
+__host__ int smem_riccati_finish(int n, int m) { return std::max(m * (n + m + 1) + m * (n + 1) + m + 8, n * n); }
 __host__ int smem_aff(int n, int m) { return 2 * (n * n + n) + n * n + 5 * n + 2 * m + 8; }
 
 // Cost-relation slot layout (ld 2n + 1): constraint rows at 0 (CI_ROWS of them),
@@ -57,39 +57,33 @@ __global__ void k_lqr_up(Group g, int per_task) {
   double *slot = g.CS[0] + (size_t)t * g.cs_stride;
   int *cm = g.CI[0] + (size_t)t * CI_STRIDE;
   double *sm = team_smem(per_task);
+  if (P.nch == 1 && (ci.c == 0 || g.fp64 == nullptr)) {
+    // one chunk: k_riccati_down starts from the terminal cost itself (the FP32 sweep from its
+    // square root, below), k_riccati_finish tests it
+    if (tid == 0) { cm[CI_ROWS] = 0; cm[CI_NA] = 0; cm[CI_NB] = 0; cm[CI_ROWS2] = 0; }
+    return;
+  }
   if (ci.c == P.nch) {
     // terminal value: rows [L' | L^{-1} qbar_N], L L' = Qbar_N (eq. terminal-cost-data)
     const int sN = P.st0 + P.N;
     const double *ws = stage_ws(g, sN);
     const int nN = stage_wi(g, sN)[SI_NBAR];
-    double *Hh = sm, *l = sm + n * n;
-    for (int idx = tid; idx < nN * nN; idx += TEAM) {
+    double *Hh = sm;  // bordered by qbar_N
+    for (int idx = tid; idx < (nN + 1) * nN; idx += TEAM) {
       int a = idx / nN, j = idx - a * nN;
-      Hh[idx] = ws[g.ws.Qb + a * n + j];
+      Hh[idx] = a < nN ? ws[g.ws.Qb + a * n + j] : ws[g.ws.qb + j];
     }
     tsync();
-    const int fail = wcholesky(Hh, nN, nN);
-    if (tid == 0) {
-      for (int a = 0; a < nN; a++) {
-        double s0 = ws[g.ws.qb + a];
-        for (int k = 0; k < a; k++) s0 = fma(-Hh[a * nN + k], l[k], s0);
-        l[a] = s0 / Hh[a * nN + a];
-      }
-    }
-    tsync();
+    const int fail = wchol(Hh, nN, nN, true);
     double *cost = crel_cost(slot, n);
     for (int idx = tid; idx < nN * (nN + 1); idx += TEAM) {
       int a = idx / (nN + 1), j = idx - a * (nN + 1);
-      cost[a * ldr + j] = (j < nN) ? Hh[j * nN + a] : l[a];
+      cost[a * ldr + j] = j == nN ? Hh[nN * nN + a] : (j >= a ? Hh[j * nN + a] : 0.0);
     }
     if (tid == 0) {
       cm[CI_ROWS] = 0; cm[CI_NA] = nN; cm[CI_NB] = 0; cm[CI_ROWS2] = nN;
       if (fail) set_status(g, ci.prob, ST_NONCONVEX);
     }
-    return;
-  }
-  if (P.nch == 1) {  // one chunk: k_riccati_down starts from the terminal value alone
-    if (tid == 0) { cm[CI_ROWS] = 0; cm[CI_NA] = 0; cm[CI_NB] = 0; cm[CI_ROWS2] = 0; }
     return;
   }
   const int a = ci.c * P.L, b = min(a + P.L, P.N);
@@ -709,11 +703,20 @@ __global__ void k_riccati_finish(Group g, int per_task) {
     const StageInfo S = g.st[s];
     const ProbInfo &P = g.prob[S.prob];
     if (skipped_by_mask(g, S.prob)) return;
-    if (S.i >= P.N) return;
-    if (g.fp64 != nullptr && g.fp64[P.id] == 0) return;  // k_riccati_down_f32 stored this problem's factors
     const int n = g.n, m = g.m, tid = team_rank();
     double *ws = stage_ws(g, s);
     const int *wi = stage_wi(g, s);
+    if (S.i >= P.N) {
+      // one chunk: the terminal cost has to be convex (otherwise tested by k_lqr_up)
+      if (P.nch > 1 || g.fp64 != nullptr) return;
+      const int nN = wi[SI_NBAR];
+      double *Hh = team_smem(per_task);
+      for (int idx = tid; idx < nN * nN; idx += TEAM) Hh[idx] = ws[g.ws.Qb + idx / nN * n + idx % nN];
+      tsync();
+      if (wchol(Hh, nN, nN, false) && tid == 0) set_status(g, S.prob, ST_NONCONVEX);
+      return;
+    }
+    if (g.fp64 != nullptr && g.fp64[P.id] == 0) return;  // k_riccati_down_f32 stored this problem's factors
     const int nx = wi[SI_NBAR], mu = wi[SI_MBAR], n1 = stage_wi(g, s + 1)[SI_NBAR];
     const int ldr = n + m + 1;
     double *sm = team_smem(per_task);
@@ -927,7 +930,7 @@ __global__ void k_aff_up(Group g, int mode, int per_task) {
     aff_stage_map(g, s, mode, Gs, gs, tmp);
     const int dout = fwd ? aff_dim(g, s + 1, mode) : aff_dim(g, s, mode);
     // Tm = Gs Gm (dout x d0), tmp = Gs gm + gs
-    wgemm<false, false>(dout, d0, dcur, 1.0, Gs, n, Gm, n, 0.0, Tm, n);
+    wgemm<false, false>(dout, d0, dcur, Gs, n, Gm, n, 0, Tm, n);
     for (int r = tid; r < dout; r += TEAM) {
       double s0 = gs[r];
       for (int l = 0; l < dcur; l++) s0 = fma(Gs[r * n + l], gm[l], s0);
@@ -999,7 +1002,7 @@ __global__ void k_aff_level(Group g, int src, int d, int fwd, int per_task) {
       nb = 0;
     } else {
       // (G G2, G g2 + g): input dimension na2, output nb
-      wgemm<false, false>(nb, na2, na, 1.0, acc, n, oth, n, 0.0, Tm, n);
+      wgemm<false, false>(nb, na2, na, acc, n, oth, n, 0, Tm, n);
       for (int r = tid; r < nb; r += TEAM) {
         double s0 = acc[n * n + r];
         for (int l = 0; l < na; l++) s0 = fma(acc[r * n + l], oth[n * n + l], s0);

@@ -171,8 +171,8 @@ __global__ void k_primal_up(Group g, int per_task) {
     const double *A = g.A + P.oA + (size_t)i * n * n, *B = g.B + P.oB + (size_t)i * n * m;
     const double *c = g.c + P.oc + (size_t)i * n;
     // [L B | L A | R | L c + l]
-    wgemm<false, false>(rr, m, n, 1.0, Rel, ldr, B, m, 0.0, M, ldm);
-    wgemm<false, false>(rr, n, n, 1.0, Rel, ldr, A, n, 0.0, M + m, ldm);
+    wgemm<false, false>(rr, m, n, Rel, ldr, B, m, 0, M, ldm);
+    wgemm<false, false>(rr, n, n, Rel, ldr, A, n, 0, M + m, ldm);
     for (int idx = tid; idx < rr * (n + 1); idx += TEAM) {
       int r = idx / (n + 1), j = idx - r * (n + 1);
       if (j < n) {
@@ -279,8 +279,8 @@ __device__ int primal_down_stage(const Group &g, const ProbInfo &P, int i, doubl
   const StageInfo S = g.st[P.st0 + i];
   const double *A = g.A + P.oA + (size_t)i * n * n, *B = g.B + P.oB + (size_t)i * n * m;
   const double *c = g.c + P.oc + (size_t)i * n;
-  wgemm<false, false>(rr, m, n, 1.0, Hs, ldh, B, m, 0.0, M, ldm);
-  wgemm<false, false>(rr, n, n, 1.0, Hs, ldh, A, n, 0.0, M + m, ldm);
+  wgemm<false, false>(rr, m, n, Hs, ldh, B, m, 0, M, ldm);
+  wgemm<false, false>(rr, n, n, Hs, ldh, A, n, 0, M + m, ldm);
   for (int r = tid; r < rr; r += TEAM) {
     double s0 = Hs[r * ldh + n];
     for (int l = 0; l < n; l++) s0 = fma(Hs[r * ldh + l], c[l], s0);
@@ -443,15 +443,15 @@ __global__ void k_param(Group g, int per_task) {
       const double *QN = g.Q + P.oQ + (size_t)P.N * n * n, *qN = g.qv + P.oqv + (size_t)P.N * n;
       double *QT = Wt;  // n x nb (reuse)
       double *T = Qf + rank;  // columns rank.. of Qf, ld n
-      wgemm<false, false>(n, nb, n, 1.0, QN, n, T, n, 0.0, QT, n);
-      wgemm<true, false>(nb, nb, n, 1.0, T, n, QT, n, 0.0, ws + g.ws.Qb, n);
+      wgemm<false, false>(n, nb, n, QN, n, T, n, 0, QT, n);
+      wgemm<true, false>(nb, nb, n, T, n, QT, n, 0, ws + g.ws.Qb, n);
       for (int l = tid; l < n; l += TEAM) {
         double s0 = qN[l];
         for (int j = 0; j < n; j++) s0 = fma(QN[l * n + j], X[j], s0);
         Hs[l] = s0;
       }
       tsync();
-      wgemm<true, false>(nb, 1, n, 1.0, T, n, Hs, 1, 0.0, ws + g.ws.qb, 1);
+      wgemm<true, false>(nb, 1, n, T, n, Hs, 1, 0, ws + g.ws.qb, 1);
     }
   });
 }
@@ -511,7 +511,7 @@ __global__ void __launch_bounds__(256, 4) k_elim(Group g, int per_task) {
       for (int idx = tid; idx < n * n; idx += TEAM) AT[idx] = A[idx];
       for (int l = tid; l < n; l += TEAM) Atc[l] = c[l];
     } else {
-      wgemm<false, false>(n, nb, n, 1.0, A, n, T, n, 0.0, AT, n);
+      wgemm<false, false>(n, nb, n, A, n, T, n, 0, AT, n);
       for (int l = tid; l < n; l += TEAM) {
         double s0 = c[l];
         for (int j = 0; j < n; j++) s0 = fma(A[l * n + j], t[j], s0);
@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(256, 4) k_elim(Group g, int per_task) {
       int a = idx / m, j = idx - a * m;
       Gm[a * m + j] = g.D[P.oD + (size_t)(S.prow + a) * m + j];
     }
-    wgemm<false, false>(r1, m, n, 1.0, Hn, n + 1, B, m, 0.0, Gm + S.p * m, m);
+    wgemm<false, false>(r1, m, n, Hn, n + 1, B, m, 0, Gm + S.p * m, m);
     // Lemma 4: Z = null(Gamma), [Y | y] = -Gamma^- [Phi | gamma] (min norm)
     // the small form only: this kernel runs many CTAs to an SM, and the large form's
     // registers and static scratch would cost it occupancy
@@ -570,10 +570,10 @@ __global__ void __launch_bounds__(256, 4) k_elim(Group g, int per_task) {
     for (int a = tid; a < m; a += TEAM) ys[a] = Sol[a * (nb + 1) + nb];
     tsync();
     // reduced dynamics (eq. reduced-dynamics-data), S_{i+1} = T_{i+1}^T
-    wgemm<false, false>(n, nb, m, 1.0, B, m, Yw, n, 1.0, AT, n);            // A T + B Y
-    if (!tne) wgemm<true, false>(nn, nb, n, 1.0, Tn, n, AT, n, 0.0, ws + g.ws.Ab, n);
-    wgemm<false, false>(n, mb, m, 1.0, B, m, Z, m, 0.0, BZ, m);             // B Z
-    if (!tne) wgemm<true, false>(nn, mb, n, 1.0, Tn, n, BZ, m, 0.0, ws + g.ws.Bb, m);
+    wgemm<false, false>(n, nb, m, B, m, Yw, n, 1, AT, n);            // A T + B Y
+    if (!tne) wgemm<true, false>(nn, nb, n, Tn, n, AT, n, 0, ws + g.ws.Ab, n);
+    wgemm<false, false>(n, mb, m, B, m, Z, m, 0, BZ, m);             // B Z
+    if (!tne) wgemm<true, false>(nn, mb, n, Tn, n, BZ, m, 0, ws + g.ws.Bb, m);
     for (int l = tid; l < n; l += TEAM) {
       double s0 = Atc[l] - tn[l];
       for (int j = 0; j < m; j++) s0 = fma(B[l * m + j], ys[j], s0);
@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(256, 4) k_elim(Group g, int per_task) {
       }
       for (int l = tid; l < n; l += TEAM) ws[g.ws.cb + l] = cv[l];
     } else {
-      wgemm<true, false>(nn, 1, n, 1.0, Tn, n, cv, 1, 0.0, ws + g.ws.cb, 1);
+      wgemm<true, false>(nn, 1, n, Tn, n, cv, 1, 0, ws + g.ws.cb, 1);
     }
     // state substitution (eq. state-cost-data)
     double *Qb = ws + g.ws.Qb, *Mb = ws + g.ws.Mb, *Rb = ws + g.ws.Rb;
@@ -602,9 +602,9 @@ __global__ void __launch_bounds__(256, 4) k_elim(Group g, int per_task) {
       for (int a = tid; a < m; a += TEAM) rz[a] = r[a];
       tsync();
     } else {
-      wgemm<false, false>(n, nb, n, 1.0, Q, n, T, n, 0.0, QT, n);             // Q T
-      wgemm<true, false>(nb, nb, n, 1.0, T, n, QT, n, 0.0, Qb, n);            // Q^z
-      wgemm<true, false>(nb, m, n, 1.0, T, n, Mm, m, 0.0, Mz, m);             // M^z
+      wgemm<false, false>(n, nb, n, Q, n, T, n, 0, QT, n);             // Q T
+      wgemm<true, false>(nb, nb, n, T, n, QT, n, 0, Qb, n);            // Q^z
+      wgemm<true, false>(nb, m, n, T, n, Mm, m, 0, Mz, m);             // M^z
       for (int l = tid; l < n; l += TEAM) {
         double s0 = q[l];
         for (int j = 0; j < n; j++) s0 = fma(Q[l * n + j], t[j], s0);
@@ -616,27 +616,27 @@ __global__ void __launch_bounds__(256, 4) k_elim(Group g, int per_task) {
         rz[a] = s0;                                                           // r^z
       }
       tsync();
-      wgemm<true, false>(nb, 1, n, 1.0, T, n, Qtq, 1, 0.0, qz, 1);            // q^z
+      wgemm<true, false>(nb, 1, n, T, n, Qtq, 1, 0, qz, 1);            // q^z
     }
     // reduced cost (eq. reduced-cost-data)
-    wgemm<false, false>(m, nb, m, 1.0, R, m, Yw, n, 0.0, RY, n);            // R Y
-    wgemm<false, false>(m, mb, m, 1.0, R, m, Z, m, 0.0, RZ, m);             // R Z
+    wgemm<false, false>(m, nb, m, R, m, Yw, n, 0, RY, n);            // R Y
+    wgemm<false, false>(m, mb, m, R, m, Z, m, 0, RZ, m);             // R Z
     for (int a = tid; a < m; a += TEAM) {
       double s0 = rz[a];
       for (int j = 0; j < m; j++) s0 = fma(R[a * m + j], ys[j], s0);
       Ry[a] = s0;                                                           // R y + r^z
     }
     tsync();
-    wgemm<false, false>(nb, nb, m, 1.0, Mz, m, Yw, n, 0.0, X2, n);          // M^z Y
+    wgemm<false, false>(nb, nb, m, Mz, m, Yw, n, 0, X2, n);          // M^z Y
     for (int idx = tid; idx < nb * nb; idx += TEAM) {
       int a = idx / nb, j = idx - a * nb;
       Qb[a * n + j] += X2[a * n + j] + X2[j * n + a];
     }
     tsync();
-    wgemm<true, false>(nb, nb, m, 1.0, Yw, n, RY, n, 1.0, Qb, n);           // + Y' R Y
-    wgemm<false, false>(nb, mb, m, 1.0, Mz, m, Z, m, 0.0, Mb, m);           // M^z Z
-    wgemm<true, false>(nb, mb, m, 1.0, Yw, n, RZ, m, 1.0, Mb, m);           // + Y' R Z
-    wgemm<true, false>(mb, mb, m, 1.0, Z, m, RZ, m, 0.0, Rb, m);            // Z' R Z
+    wgemm<true, false>(nb, nb, m, Yw, n, RY, n, 1, Qb, n);           // + Y' R Y
+    wgemm<false, false>(nb, mb, m, Mz, m, Z, m, 0, Mb, m);           // M^z Z
+    wgemm<true, false>(nb, mb, m, Yw, n, RZ, m, 1, Mb, m);           // + Y' R Z
+    wgemm<true, false>(mb, mb, m, Z, m, RZ, m, 0, Rb, m);            // Z' R Z
     double *qb = ws + g.ws.qb, *rb = ws + g.ws.rb;
     for (int a = tid; a < nb; a += TEAM) {
       double s0 = qz[a];
@@ -677,10 +677,12 @@ __global__ void __launch_bounds__(256, 4) k_elim(Group g, int per_task) {
         Hh[a * ldH + j] = h;
       }
       tsync();
-      int fail = 0;
-      if (tid < 32) fail = wchol_bordered(Hh, ldH, kh);
-      fail = __syncthreads_or(fail);
+      // the factor itself is read by the chunk aggregates and by the FP32 sweep; a problem of one
+      // chunk whose sweep starts from H only needs to know that H is positive definite
+      const bool keep = P.nch > 1 || g.fp64 != nullptr;
+      const int fail = wchol(Hh, ldH, kh, keep);
       if (fail && tid == 0) set_status(g, S.prob, ST_NONCONVEX);
+      if (!keep) return;
       double *LT = ws + g.ws.LT, *lt = ws + g.ws.lt;
       for (int idx = tid; idx < kh * kh; idx += TEAM) {
         int a = idx / kh, j = idx - a * kh;

@@ -12,6 +12,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include "fx.cuh"
 
 namespace eclqr {
 
@@ -21,12 +22,6 @@ constexpr unsigned kFull = 0xffffffffu;
 __device__ __forceinline__ int team_rank() { return threadIdx.x; }
 #define TEAM ((int)blockDim.x)
 __device__ __forceinline__ void tsync() { __syncthreads(); }
-
-__device__ __forceinline__ double warp_max(double v) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) v = fmax(v, __shfl_xor_sync(kFull, v, o));
-  return v;
-}
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -46,65 +41,47 @@ __device__ __forceinline__ void warp_argmax(long long &key, int &idx) {
   }
 }
 
-// Team reductions: warp shuffles, then one partial per warp through shared
+// The bit pattern of |v| for the integer maximum reductions: non-negative doubles order like their
+// patterns, and a NaN counts as nothing, as in fmax.
+__device__ __forceinline__ unsigned long long abs_key(double v) {
+  const unsigned long long k = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+  return k > 0x7ff0000000000000ull ? 0ull : k;
+}
+// Largest key over the warp, to every lane.
+__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long key) {
+  const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
+  const unsigned mhi = __reduce_max_sync(kFull, hi);
+  const unsigned mlo = __reduce_max_sync(kFull, hi == mhi ? lo : 0u);
+  return ((unsigned long long)mhi << 32) | mlo;
+}
+
+// Largest value over the team of keys from abs_key: one partial per warp through shared
 // memory.  The trailing barrier lets the next reduction reuse the slots.
-__device__ __forceinline__ double team_max(double v) {
-  __shared__ double red_max[32];
-  v = warp_max(v);
-  if ((threadIdx.x & 31) == 0) red_max[threadIdx.x >> 5] = v;
+__device__ __forceinline__ double team_max_key(unsigned long long key) {
+  __shared__ unsigned long long red_max[32];
+  key = warp_max_key(key);
+  if (blockDim.x == 32) return __longlong_as_double((long long)key);
+  if ((threadIdx.x & 31) == 0) red_max[threadIdx.x >> 5] = key;
   __syncthreads();
-  double r = red_max[0];
-  for (int w = 1; w < (int)(blockDim.x >> 5); w++) r = fmax(r, red_max[w]);
+  unsigned long long r = red_max[0];
+  for (int w = 1; w < (int)(blockDim.x >> 5); w++) r = max(r, red_max[w]);
   __syncthreads();
-  return r;
+  return __longlong_as_double((long long)r);
 }
+__device__ __forceinline__ double team_max(double v) { return team_max_key(abs_key(v)); }  // v >= 0
 
-__device__ __forceinline__ void team_argmax(double v, int idx, double &bv, int &bi) {
-  __shared__ long long red_key[32];
-  __shared__ int red_idx[32];
-  long long key = __double_as_longlong(v);
-  warp_argmax(key, idx);
-  if ((threadIdx.x & 31) == 0) {
-    red_key[threadIdx.x >> 5] = key;
-    red_idx[threadIdx.x >> 5] = idx;
-  }
-  __syncthreads();
-  key = red_key[0];
-  idx = red_idx[0];
-  for (int w = 1; w < (int)(blockDim.x >> 5); w++) {
-    const long long k2 = red_key[w];
-    const int i2 = red_idx[w];
-    if (k2 > key || (k2 == key && i2 < idx)) { key = k2; idx = i2; }
-  }
-  __syncthreads();
-  bv = __longlong_as_double(key);
-  bi = idx;
-}
-
-// C (m x n) = alpha * op(A) op(B) + beta * C; op(A) is m x k, op(B) is k x n.
-// C must not alias A or B.
+// C (m x n) = op(A) op(B) (beta = 0) or C + op(A) op(B) (beta = 1); op(A) is m x k, op(B) is
+// k x n.  C must not alias A or B.  One accumulator per element: FP64 instructions of one
+// sub-partition do not overlap, so a second one would only add an addition.
 template <bool TA, bool TB>
-static __device__ void wgemm(int m, int n, int k, double alpha, const double *A, int lda, const double *B,
-                      int ldb, double beta, double *C, int ldc) {
+static __device__ void wgemm(int m, int n, int k, const double *A, int lda, const double *B,
+                      int ldb, int beta, double *C, int ldc) {
   for (int idx = team_rank(); idx < m * n; idx += TEAM) {
     int i = idx / n, j = idx - i * n;
-    double s0 = 0.0, s1 = 0.0;
-    int l = 0;
-    for (; l + 1 < k; l += 2) {
-      double a0 = TA ? A[l * lda + i] : A[i * lda + l];
-      double a1 = TA ? A[(l + 1) * lda + i] : A[i * lda + l + 1];
-      double b0 = TB ? B[j * ldb + l] : B[l * ldb + j];
-      double b1 = TB ? B[j * ldb + l + 1] : B[(l + 1) * ldb + j];
-      s0 = fma(a0, b0, s0);
-      s1 = fma(a1, b1, s1);
-    }
-    if (l < k) {
-      double a0 = TA ? A[l * lda + i] : A[i * lda + l];
-      double b0 = TB ? B[j * ldb + l] : B[l * ldb + j];
-      s0 = fma(a0, b0, s0);
-    }
-    double s = alpha * (s0 + s1);
-    C[i * ldc + j] = (beta == 0.0) ? s : fma(beta, C[i * ldc + j], s);
+    double s = beta ? C[i * ldc + j] : 0.0;
+#pragma unroll 4
+    for (int l = 0; l < k; l++) s = fma(TA ? A[l * lda + i] : A[i * lda + l], TB ? B[j * ldb + l] : B[l * ldb + j], s);
+    C[i * ldc + j] = s;
   }
   tsync();
 }
@@ -129,55 +106,6 @@ __device__ __forceinline__ double *hh_part() {
 __device__ __forceinline__ double *hh_norms() {
   __shared__ double norms[2 * kMaxCols];
   return norms;
-}
-
-// Reflector H = I - beta v v' from column piv on rows [r0, r1) (nrm = the
-// column's 2-norm there, > 0), applied to the columns of [c0, c1) that are not
-// done and are not piv; column piv becomes (-sign(x_k) nrm, 0, ..., 0).  v
-// (indexed by row) keeps the reflector, beta = 1 / (nrm |v[r0]|).  The dot
-// products v'M_j are split over the team by column and by row segment, so a
-// column of R rows costs about R * columns / TEAM FMAs per thread.
-static __device__ void whouse_apply(double *M, int ld, int r0, int r1, int piv, int c0, int c1, const int *done,
-                                    double *v, double *w, double nrm) {
-  const int tid = team_rank(), T = TEAM;
-  double *part = hh_part();
-  const double xk = M[r0 * ld + piv];
-  const double sg = xk >= 0.0 ? 1.0 : -1.0;
-  for (int i = r0 + tid; i < r1; i += T) v[i] = (i == r0) ? xk + sg * nrm : M[i * ld + piv];
-  const double beta = 1.0 / (nrm * (nrm + fabs(xk)));
-  tsync();
-  const int nc = c1 - c0, nr = r1 - r0;
-  // thread -> (column c0 + jj, row segment sgm): rows r0 + sgm, r0 + sgm + S, ...
-  // S * nc <= T when S > 1; with S == 1 threads step over columns
-  const int S = max(1, min(nc > 0 ? T / nc : 1, nr));
-  const int jj0 = (S > 1) ? tid % nc : tid, sgm = (S > 1) ? tid / nc : 0;
-  const bool seg_ok = sgm < S;
-  for (int jj = jj0; seg_ok && jj < nc; jj += (S > 1 ? nc : T)) {
-    const int j = c0 + jj;
-    double acc = 0.0;
-    if (!((done && done[j]) || j == piv))
-      for (int i = r0 + sgm; i < r1; i += S) acc = fma(v[i], M[i * ld + j], acc);
-    if (S == 1) w[j] = beta * acc;
-    else part[sgm * nc + jj] = acc;
-  }
-  tsync();
-  if (S > 1) {
-    for (int j2 = tid; j2 < nc; j2 += T) {
-      double acc = part[j2];
-      for (int k2 = 1; k2 < S; k2++) acc += part[k2 * nc + j2];
-      w[c0 + j2] = beta * acc;
-    }
-    tsync();
-  }
-  for (int jj = jj0; seg_ok && jj < nc; jj += (S > 1 ? nc : T)) {
-    const int j = c0 + jj;
-    if ((done && done[j]) || j == piv) continue;
-    const double wj = w[j];
-    for (int i = r0 + sgm; i < r1; i += S) M[i * ld + j] = fma(-wj, v[i], M[i * ld + j]);
-  }
-  tsync();
-  for (int i = r0 + tid; i < r1; i += T) M[i * ld + piv] = (i == r0) ? -sg * nrm : 0.0;
-  tsync();
 }
 
 __device__ __forceinline__ double *hh_rowk() {
@@ -208,18 +136,6 @@ struct HHLayout {
   int lc;  // this lane's column within its warp's block
   int sg;  // this lane's segment
 };
-// single-precision approximations (PTX rsqrt.approx / rcp.approx, relative
-// error about 2^-22), used only as seeds and for small integer quotients
-__device__ __forceinline__ float rsqrt_seed(float x) {
-  float y;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ float rcp_seed(float x) {
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 // Branch-free, so that the compiler can schedule it inside the latency of
 // the FP64 chains around it.  Teams have 1, 2, 4 or 8 warps.
 __device__ __forceinline__ HHLayout hh_layout(int cnt, int nr) {
@@ -252,68 +168,33 @@ __device__ __forceinline__ double seg_sum(double acc, int sg, int S) {
 
 // Reflector of a column x with squared norm d = ||x||^2 and pivot entry x_k:
 // nrm = sqrt(d), shift = sign(x_k) nrm (sign(0) = +1, also for -0),
-// v_k = x_k + shift and beta = 2 / ||v||^2 with ||v||^2 = (d - x_k^2) + v_k^2
-// evaluated from the v actually formed, so H = I - beta v v' is orthogonal to
-// rounding whatever the last bits of nrm.  The FP64 square root and divide
-// are long dependent chains (about 690 and 440 cycles), so both come from
-// single-precision seeds (exponents handled on the integer pipe) refined by
-// one third-order step: for d^(-1/2) the Householder iteration
-// y = y0 (1 + e/2 + 3 e^2 / 8), e = 1 - d y0^2, and for 1/q the Newton-type
-// step r = r0 (1 + e + e^2), e = 1 - q r0.  From a 2^-21 seed each leaves a
-// truncation error below 2^-60 (5 e^3 / 16 and e^3).  The code is branch-
-// free; it returns false, with the outputs unset, when d is zero, subnormal,
-// above 2^1000 or not finite, where the seeds do not apply.
+// v_k = x_k + shift and beta = 2 / ||v||^2 = 1 / (nrm (nrm + |x_k|)), all in integers (fx.cuh): with
+// m = d 2^(-2 h) in [1, 4), N = sqrt(m) and X = |x_k| 2^-h as integers of 60 fractional bits,
+// V = N + X is |v_k| and 1 / (N V) is beta, each within 2^-55 of its value before the rounding to
+// FP64.  In FP64, from single-precision seeds and one third-order step each, the same scalars are
+// eleven dependent instructions in every warp of the team, most of a short step (n = 12, 147 chunks:
+// k_dual_down 787 us).  Branch-free; false, with the outputs unset, when d is zero, subnormal, above
+// 2^1000 or not finite.
 __device__ __forceinline__ bool hh_reflector(double d, double xk, double &nrm, double &shift, double &vk,
                                              double &beta) {
-  const long long db = __double_as_longlong(d);
-  const int dh = (int)(db >> 32);
-  const int ex = ((dh >> 20) & 0x7ff) - 1023;
-  // d = 2^(2 h) m, m in [1, 4): y0 = rsqrt(m) 2^-h
-  const int odd = ex & 1, h = (ex - odd) >> 1;
-  const unsigned m23 = ((unsigned)(dh & 0xfffff) << 3) | ((unsigned)db >> 29);
-  const int yf = __float_as_int(rsqrt_seed(__int_as_float(((127 + odd) << 23) | (int)m23)));
-  const double y0 =
-      __hiloint2double(((((yf >> 23) & 0xff) + (1023 - 127) - h) << 20) | ((yf & 0x7fffff) >> 3), (yf & 7) << 29);
-  const double dx = fma(-xk, xk, d);
-  const double t = d * y0;
-  const double e = fma(-t, y0, 1.0);
-  const double p = fma(0.375, e, 0.5);
-  nrm = fma(t * e, p, t);
+  int h;
+  bool ok;
+  const unsigned long long s = fx_even(d, h, ok);
+  const unsigned long long N = __umul64hi(s, fx_rsqrt(s));  // [2^60, 2^61]
   const bool neg = (__double_as_longlong(xk) < 0) && ((__double_as_longlong(xk) << 1) != 0);
+  const long long sig = fx_significand(xk);
+  // |x_k| <= nrm up to rounding; the bound on the shift only matters where the result is not used
+  const int sh = min(fx_expo(xk) - 53 - h + 60, 9);
+  const unsigned long long a = (unsigned long long)(sig < 0 ? -sig : sig);
+  const unsigned long long X = sh >= 0 ? a << sh : (sh > -63 ? a >> -sh : 0ull);
+  const unsigned long long V = N + X;
+  nrm = fx_to((long long)N, h - 60);
   shift = neg ? -nrm : nrm;
-  vk = xk + shift;
-  const double q = fma(vk, vk, dx);
-  // q = 2^g m, m in [1, 2): r0 = (1 / m) 2^-g ~ 1 / q, and beta = 2 / q from
-  // the doubled seed (exponent + 1)
-  const long long qb = __double_as_longlong(q);
-  const int qh = (int)(qb >> 32);
-  const int g = ((qh >> 20) & 0x7ff) - 1023;
-  const unsigned n23 = ((unsigned)(qh & 0xfffff) << 3) | ((unsigned)qb >> 29);
-  const int rf = __float_as_int(rcp_seed(__int_as_float((127 << 23) | (int)n23)));
-  const int rhi = ((((rf >> 23) & 0xff) + (1023 - 127) - g) << 20) | ((rf & 0x7fffff) >> 3), rlo = (rf & 7) << 29;
-  const double r0 = __hiloint2double(rhi, rlo), r2 = __hiloint2double(rhi + (1 << 20), rlo);
-  const double f = fma(-q, r0, 1.0);
-  beta = fma(r2, fma(f, f, f), r2);
-  return ex >= -1000 && ex <= 1000;
-}
-
-// d^(-1/2) by the method of hh_reflector: a single-precision seed (exponent
-// on the integer pipe) and one third-order step y = y0 (1 + e/2 + 3 e^2 / 8),
-// e = 1 - d y0^2, truncation error below 2^-60.  ok is false, with the result
-// unusable, unless d is positive, normal and within [2^-1000, 2^1001).
-__device__ __forceinline__ double seeded_rsqrt(double d, bool &ok) {
-  const long long db = __double_as_longlong(d);
-  const int dh = (int)(db >> 32);
-  const int ex = ((dh >> 20) & 0x7ff) - 1023;
-  const int odd = ex & 1, h = (ex - odd) >> 1;
-  const unsigned m23 = ((unsigned)(dh & 0xfffff) << 3) | ((unsigned)db >> 29);
-  const int yf = __float_as_int(rsqrt_seed(__int_as_float(((127 + odd) << 23) | (int)m23)));
-  const double y0 =
-      __hiloint2double(((((yf >> 23) & 0xff) + (1023 - 127) - h) << 20) | ((yf & 0x7fffff) >> 3), (yf & 7) << 29);
-  const double e = fma(-(d * y0), y0, 1.0);
-  const double p = fma(0.375, e, 0.5);
-  ok = (d > 0.0) && ex >= -1000 && ex <= 1000;
-  return fma(y0 * e, p, y0);
+  vk = fx_to(neg ? -(long long)V : (long long)V, h - 60);
+  const unsigned long long q = __umul64hi(N << 2, V << 1);  // N V 2^-61
+  const int z = __clzll((long long)q);
+  beta = fx_to(fx_rcp(q << z), z - 2 * h - 60);  // N V 2^(2 h - 120) = (q 2^z 2^-64) 2^(2 h + 5 - z)
+  return ok;
 }
 
 // Team arg-max with one barrier: partials alternate between two buffers by
@@ -786,14 +667,6 @@ __device__ __forceinline__ unsigned long long *colmax_keys() {
   return &k[0][0];
 }
 
-// Largest key (bit pattern of a non-negative double) over the warp, to lane 0.
-__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long key) {
-  const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
-  const unsigned mhi = __reduce_max_sync(kFull, hi);
-  const unsigned mlo = __reduce_max_sync(kFull, hi == mhi ? lo : 0u);
-  return ((unsigned long long)mhi << 32) | mlo;
-}
-
 // Scales each of the rows [0, r) of M to unit 2-norm over its columns
 // [0, ncoef), applying the factor to the columns [0, nscale); rows of zero
 // norm are left as they are.  Ends with a team barrier.
@@ -982,10 +855,9 @@ static __device__ ProjResult wproject(double *M, int ld, int r, int ng, const in
 // nk - rank are an orthonormal basis of null(K).  perm: rk ints.
 // ---------------------------------------------------------------------------
 static __device__ int wtqr_small(const double *K, int ldk, int rk, int nk, double tau_rank, double *W, int ldw,
-                    double *Q, int ldq, int *perm, double *scr /* >= nk + max(nk, rk) */) {
-  const int tid = team_rank(), T = TEAM;
-  double *v = scr, *w = scr + nk;
-  double *part = hh_part();
+                    double *Q, int ldq, int *perm, double *scr /* >= nk */) {
+  const int tid = team_rank(), T = TEAM, lane = tid & 31, wid = tid >> 5;
+  double *v = scr;
   for (int idx = tid; idx < nk * rk; idx += T) {
     int i = idx / rk, j = idx - i * rk;
     W[i * ldw + j] = K[j * ldk + i];
@@ -996,69 +868,75 @@ static __device__ int wtqr_small(const double *K, int ldk, int rk, int nk, doubl
   }
   for (int j = tid; j < rk; j += T) perm[j] = j;
   tsync();
-  double nu = 0.0;
-  for (int j = tid; j < rk; j += T) {
-    double acc = 0.0;
-    for (int i = 0; i < nk; i++) acc = fma(W[i * ldw + j], W[i * ldw + j], acc);
-    nu = fmax(nu, acc);
-  }
-  nu = sqrt(team_max(nu));
-  const double thr = tau_rank * nu;
+  double thr = 0.0;
   int rank = 0;
   for (int s = 0; s < rk && s < nk; s++) {
-    double mybest = -1.0;
-    int mypiv = 0x7fffffff;
+    // exact remaining norms of the columns [s, rk), one column per thread
+    unsigned long long bkey = 0ull;
+    int bidx = 0x7fffffff;
     for (int j = s + tid; j < rk; j += T) {
       double t = 0.0;
       for (int i = s; i < nk; i++) t = fma(W[i * ldw + j], W[i * ldw + j], t);
-      if (t > mybest) { mybest = t; mypiv = j; }
+      if (bidx == 0x7fffffff || abs_key(t) > bkey) { bkey = abs_key(t); bidx = j; }
     }
+    warp_argmax_key(bkey, bidx, s & 1);
+    tsync();
     double b2;
     int piv;
-    team_argmax(mybest < 0.0 ? 0.0 : mybest, mybest < 0.0 ? 0x7fffffff : mypiv, b2, piv);
+    argmax_finish(s & 1, b2, piv);
     if (piv == 0x7fffffff) break;
-    const double best = sqrt(b2);
-    if (!(best > thr)) break;
-    if (piv != s) {
-      for (int i = tid; i < nk; i += T) {
-        double t = W[i * ldw + s];
-        W[i * ldw + s] = W[i * ldw + piv];
-        W[i * ldw + piv] = t;
-      }
-      if (tid == 0) {
-        int t = perm[s]; perm[s] = perm[piv]; perm[piv] = t;
-      }
-      tsync();
+    const double xk = W[s * ldw + piv];
+    double nrm, shift, vk, beta;
+    if (!hh_reflector(b2, xk, nrm, shift, vk, beta)) {
+      nrm = sqrt(b2);
+      shift = xk >= 0.0 ? nrm : -nrm;
+      vk = xk + shift;
+      beta = 1.0 / (nrm * (nrm + fabs(xk)));
     }
-    // W columns > s (the reflector stays in v)
-    whouse_apply(W, ldw, s, nk, s, s + 1, rk, nullptr, v, w, best);
-    const double beta = 1.0 / (best * fabs(v[s]));
-    // Q <- Q H on columns [s, nk): row dots split by row of Q and segment of l
-    const int nl = nk - s;
-    const int S = max(1, min(T / nk, nl));
-    for (int idx = tid; idx < S * nk; idx += T) {
-      const int i = idx % nk, sgm = idx / nk;
-      double acc = 0.0;
-      for (int l = s + sgm; l < nk; l += S) acc = fma(Q[i * ldq + l], v[l], acc);
-      if (S == 1) w[i] = beta * acc;
-      else part[sgm * nk + i] = acc;
+    if (s == 0) thr = tau_rank * nrm;  // the largest norm of all
+    if (!hh_step_runs(b2, nrm, thr)) break;
+    tsync();  // every thread has read x_k
+    // the columns s and piv change places; v keeps the reflector, column s becomes R's
+    for (int i = tid; i < nk; i += T) {
+      const double x = W[i * ldw + piv];
+      W[i * ldw + piv] = W[i * ldw + s];
+      W[i * ldw + s] = i < s ? x : (i == s ? -shift : 0.0);
+      v[i] = i == s ? vk : x;
+    }
+    if (tid == 0) {
+      const int t = perm[s]; perm[s] = perm[piv]; perm[piv] = t;
     }
     tsync();
-    if (S > 1) {
-      for (int i = tid; i < nk; i += T) {
-        double acc = part[i];
-        for (int sgm = 1; sgm < S; sgm++) acc += part[sgm * nk + i];
-        w[i] = beta * acc;
+    // W's columns > s and Q's rows (Q <- Q H) side by side, each on one segment group of a warp
+    const int nl = nk - s, nw = rk - s - 1, cnt = nw + nk;
+    const HHLayout L = hh_layout(cnt, nl);
+    const int pw0 = wid * L.cw, pw1 = min(pw0 + L.cw, cnt);
+    if (L.S > 1) {
+      const int p = pw0 + L.lc;
+      const bool on = L.lc < L.cw && p < pw1;
+      double *e = p < nw ? W + s * ldw + s + 1 + p : Q + (p - nw) * ldq + s;
+      const int st = p < nw ? ldw : 1;
+      double acc = 0.0;
+      if (on)
+        for (int l = L.sg; l < nl; l += L.S) acc = fma(e[l * st], v[s + l], acc);
+      acc = seg_sum(acc, L.sg, L.S);
+      const double w = beta * __shfl_sync(kFull, acc, lane - L.sg);
+      if (on)
+        for (int l = L.sg; l < nl; l += L.S) e[l * st] = fma(-w, v[s + l], e[l * st]);
+    } else {
+      for (int p = pw0 + lane; p < pw1; p += 32) {
+        double *e = p < nw ? W + s * ldw + s + 1 + p : Q + (p - nw) * ldq + s;
+        const int st = p < nw ? ldw : 1;
+        double acc = 0.0;
+        for (int l = 0; l < nl; l++) acc = fma(e[l * st], v[s + l], acc);
+        const double w = beta * acc;
+        for (int l = 0; l < nl; l++) e[l * st] = fma(-w, v[s + l], e[l * st]);
       }
-      tsync();
-    }
-    for (int idx = tid; idx < nk * nl; idx += T) {
-      int i = idx / nl, l = s + idx % nl;
-      Q[i * ldq + l] = fma(-w[i], v[l], Q[i * ldq + l]);
     }
     tsync();
     rank++;
   }
+  tsync();
   return rank;
 }
 
@@ -1154,8 +1032,8 @@ static __device__ int wtqr_large(const double *K, int ldk, int rk, int nk, doubl
 }
 
 // Two forms with the same result contract.  wtqr_small (below 8 rows of
-// W): one thread per column for the norms and the classic reflector
-// application, little fixed cost per step, for the many small per-stage
+// W): one thread per column for the norms, the column exchange and the reflector's
+// forming in one pass, little fixed cost per step, for the many small per-stage
 // factorizations that run several CTAs to an SM.  wtqr_large: norms on the
 // balanced layout, the one-barrier arg-max, the fused Householder step with
 // seeded scalars, and a warp-local update of Q, for the factorizations on
@@ -1174,18 +1052,18 @@ static __device__ double wtqr_solve(const double *W, int ldw, const double *Q, i
                              int rk, int nk, int rank, const double *B, int ldb, int nb, double *X,
                              int ldx, double *Y, int ldy) {
   const int tid = team_rank();
-  double bmax = 0.0;
+  unsigned long long key = abs_key(1.0);  // magnitudes are compared on the integer pipe
   for (int idx = tid; idx < rk * nb; idx += TEAM) {
     int i = idx / nb, j = idx - i * nb;
-    bmax = fmax(bmax, fabs(B[i * ldb + j]));
+    key = max(key, abs_key(B[i * ldb + j]));
   }
-  bmax = fmax(1.0, team_max(bmax));
+  const double bmax = team_max_key(key);
+  key = 0ull;
   // reciprocals of R's diagonal (into X's first column, rewritten below), so that the
   // substitution chains carry multiplies instead of divides
   double *rdiag = X;
   for (int i = tid; i < rank; i += TEAM) rdiag[i * ldx] = 1.0 / W[i * ldw + i];
   tsync();
-  double rmax = 0.0;
   for (int c = tid; c < nb; c += TEAM) {
     for (int i = 0; i < rank; i++) {
       double s = B[perm[i] * ldb + c];
@@ -1195,7 +1073,7 @@ static __device__ double wtqr_solve(const double *W, int ldw, const double *Q, i
     for (int j = rank; j < rk; j++) {
       double s = B[perm[j] * ldb + c];
       for (int l = 0; l < rank; l++) s = fma(-W[l * ldw + j], Y[l * ldy + c], s);
-      rmax = fmax(rmax, fabs(s));
+      key = max(key, abs_key(s));
     }
   }
   tsync();
@@ -1206,80 +1084,38 @@ static __device__ double wtqr_solve(const double *W, int ldw, const double *Q, i
     X[i * ldx + c] = -s;
   }
   tsync();
-  return team_max(rmax) / bmax;
+  return team_max_key(key) / bmax;
 }
 
-// In-place Cholesky L L^T of an SPD n x n matrix (lower triangle, upper set
-// to zero).  Returns 0 on success, 1 if a pivot is not positive.
-// Cholesky factor of a bordered matrix, by ONE warp: on entry the lower
-// triangle of the leading kh x kh block of Hm (row-major, ld) holds the
-// symmetric H and row kh holds g (columns 0..kh-1); on exit the lower triangle
-// holds L with L L' = H and row kh holds L^{-1} g (the factor of [H g; g' *]
-// without its last diagonal).  Left-looking by columns: lane i owns rows i and
-// i + 32 (kh + 1 <= 64), and column j is one dot product of length j per row,
-// so each FP64 instruction carries every row still below the diagonal; the
-// pivot's reciprocal square root comes from seeded_rsqrt.  The upper triangle
-// is left as it was.  Returns nonzero when a pivot is not positive.
-// Rows 32 .. kh (kh + 1 > 32) go to the lanes whose own row is already done:
-// at column j lane l < j has finished row l, so it takes row l + 32, and one
-// chain of length j per lane covers every open row; only for j < kh + 1 - 32
-// does a lane hold two open rows and run a second chain.
-static __device__ int wchol_bordered(double *Hm, int ld, int kh) {
-  const int lane = threadIdx.x & 31;
-  const int extra = kh + 1 - 32;  // rows beyond the warp's first 32 (<= 0: none)
+// Cholesky factor of a matrix, by the whole team: on entry the lower triangle of the leading
+// kh x kh block of Hm (row-major, ld) holds the symmetric H and, with border, row kh holds g
+// (columns 0..kh-1); on exit the lower triangle holds L with L L' = H and row kh holds L^{-1} g.
+// The upper triangle is left as it was.  Returns nonzero when a pivot is not positive.
+// Right-looking: the trailing block's entries are dealt to all lanes, kh^3 / 6 multiply-adds in
+// about a 32nd as many instructions per warp.  A row per lane, column by column, takes kh^2 / 2
+// of them whatever kh, because an FP64 instruction costs its warp the same with one lane active
+// as with 32; and the pivot's reciprocal root is formed in integers.
+static __device__ int wchol(double *Hm, int ld, int kh, bool border) {
+  const int tid = team_rank(), rows = kh + (border ? 1 : 0);
   int fail = 0;
   for (int j = 0; j < kh; j++) {
-    // this lane's open rows: ia (its chain), ib (a second chain, only while j < extra)
-    int ia = (lane >= j && lane <= kh) ? lane : -1, ib = -1;
-    if (lane + 32 <= kh && lane + 32 >= j) {
-      if (ia < 0) ia = lane + 32;
-      else ib = lane + 32;
-    }
-    const double *rj = Hm + j * ld;
-    double s0 = 0.0, s1 = 0.0;
-    if (ia >= 0) {
-      const double *ri = Hm + ia * ld;
-      s0 = ri[j];
-      for (int l = 0; l < j; l++) s0 = fma(-ri[l], rj[l], s0);
-    }
-    if (j < extra && ib >= 0) {
-      const double *ri = Hm + ib * ld;
-      s1 = ri[j];
-      for (int l = 0; l < j; l++) s1 = fma(-ri[l], rj[l], s1);
-    }
-    // row j is lane j's first row (j < 32) or lane j - 32's (then its only open row)
-    const double sd = __shfl_sync(kFull, s0, j & 31);
+    const double sd = Hm[j * ld + j];
     bool ok;
-    double inv = seeded_rsqrt(sd, ok);
-    if (!(sd > 0.0)) fail = 1;
+    double inv = fx_rsqrt_f64(sd, ok);
+    const long long sb = __double_as_longlong(sd);
+    if (!(sb > 0 && sb <= 0x7ff0000000000000ll)) fail = 1;  // not sd > 0
     if (!ok) inv = 1.0 / sqrt(fmax(sd, 1e-300));
-    const double dj = sd * inv;
-    if (ia >= 0) Hm[ia * ld + j] = (ia == j) ? dj : s0 * inv;
-    if (ib >= 0) Hm[ib * ld + j] = s1 * inv;
-    __syncwarp();
-  }
-  return fail;
-}
-
-static __device__ int wcholesky(double *Hm, int ld, int n) {
-  const int tid = team_rank();
-  int fail = 0;
-  for (int j = 0; j < n; j++) {
-    // diagonal
-    double s = Hm[j * ld + j];
-    for (int l = 0; l < j; l++) s = fma(-Hm[j * ld + l], Hm[j * ld + l], s);
-    if (!(s > 0.0)) fail = 1;
-    const double d = sqrt(fmax(s, 1e-300));
-    const double inv = 1.0 / d;
-    for (int i = j + 1 + tid; i < n; i += TEAM) {
-      double t = Hm[i * ld + j];
-      for (int l = 0; l < j; l++) t = fma(-Hm[i * ld + l], Hm[j * ld + l], t);
-      Hm[i * ld + j] = t * inv;
-    }
+    for (int i = j + 1 + tid; i < rows; i += TEAM) Hm[i * ld + j] *= inv;
     tsync();
-    if (tid == 0) {
-      Hm[j * ld + j] = d;
-      for (int i = 0; i < j; i++) Hm[i * ld + j] = 0.0;
+    if (tid == 0) Hm[j * ld + j] = sd * inv;
+    // entry idx of the trailing rows a = 0 .. K (K: the border), columns b <= a: a = the floor of
+    // (sqrt(8 idx + 1) - 1) / 2, from a root that 8 idx + 2 keeps clear of every step
+    const int K = kh - 1 - j, cnt = K * (K + 1) / 2 + (border ? K : 0);
+    for (int idx = tid; idx < cnt; idx += TEAM) {
+      const float r = (float)(8 * idx + 2);
+      const int a = (int)((r * rsqrt_seed(r) - 1.0f) * 0.5f), b = idx - a * (a + 1) / 2;
+      double *e = Hm + (j + 1 + a) * ld + j + 1 + b;
+      *e = fma(-Hm[(j + 1 + a) * ld + j], Hm[(j + 1 + b) * ld + j], *e);
     }
     tsync();
   }
