@@ -116,6 +116,8 @@ namespace {
 // at n = 24).
 int team_for(const eclqr_handle *h, const void *kern, int ntasks, int n) {
   if (h->opt.team_warps != 0) return h->opt.team_warps;
+  // the affine chains' rows and their segments fill one warp up to n = 8, two to 16
+  if (ntasks < h->sms && kern == (const void *)k_aff_down) return n <= 8 ? 1 : n <= 16 ? 2 : kTeamWarps;
   if (ntasks < h->sms) return kTeamWarps;
   // warps below n1, from n1, n2 and n3 up; few: warps with one to four tasks per SM (-1: the
   // entry, 0: the entry, at least two -- 256 problems of 256 stages, n = 16: 37 ms with two, 42 with one, 49 with four)
@@ -446,7 +448,7 @@ int eclqr_create(const eclqr_desc *d, const eclqr_options *opt, eclqr_handle **o
       const int need = std::max({smem_primal_sweep(n, m, pmax, qmax), smem_rel_level(n, pmax, qmax), smem_param(n),
                                  smem_elim(n, m, pmax), smem_lqr_up(n, m), smem_lqr_level(n), smem_riccati(n, m),
                                  smem_riccati_finish(n, m),
-                                 smem_aff(n, m), smem_dual_stage(n, m), smem_dual_sweep(n, m, pmax, qmax),
+                                 smem_aff(n, m), smem_aff_down(n), smem_dual_stage(n, m), smem_dual_sweep(n, m, pmax, qmax),
                                  smem_dual_leaf(n, m, wmax), smem_scan_check(n, m, pmax)});
       if ((size_t)need * sizeof(double) > (size_t)kMaxSmemBytes) {
         for (auto &x : h->groups) cudaFree(x.dmem);
@@ -464,7 +466,7 @@ int eclqr_create(const eclqr_desc *d, const eclqr_options *opt, eclqr_handle **o
           {(const void *)k_lqr_up, smem_lqr_up(n, m)}, {(const void *)k_lqr_level, smem_lqr_level(n)},
           {(const void *)k_riccati_down, smem_riccati(n, m)},
           {(const void *)k_riccati_finish, smem_riccati_finish(n, m)}, {(const void *)k_aff_up, sa},
-          {(const void *)k_aff_level, sa}, {(const void *)k_aff_down, sa}, {(const void *)k_resid, 3 * n + 2 * m},
+          {(const void *)k_aff_level, sa}, {(const void *)k_aff_down, smem_aff_down(n)}, {(const void *)k_resid, 3 * n + 2 * m},
           {(const void *)k_pcorr, n + m + m * m}, {(const void *)k_dual_stage, smem_dual_stage(n, m)},
           {(const void *)k_dual_terminal, sdw}, {(const void *)k_dual_up, sdw}, {(const void *)k_dual_down, sdw + kHeldScratch},
           {(const void *)k_dual_root, sdw + kHeldScratch}, {(const void *)k_dual_leaf, smem_dual_leaf(n, m, wmax) + kHeldScratch}};
@@ -701,12 +703,13 @@ int aff_scan(eclqr_handle *h, const GroupHost &gh, const Group &g, int mode, cud
   const int sa = smem_aff(g.n, g.m);
   const int fwd = (mode == AFF_PLIN_) ? 0 : 1;
   TRY(launch(h, k_aff_prep, g.nstage, g.n + 8, st, g, mode, g.n + 8));
-  TRY(launch(h, k_aff_up, g.nslot, sa, st, g, mode, sa));
+  if (gh.levels > 0) TRY(launch(h, k_aff_up, g.nslot, sa, st, g, mode, sa));
   int src = 0;
   // radix-4 levels: strides 1, 4, 16, ... until they cover every slot
   for (int d = 1; gh.levels > 0 && d < gh.maxnch + 1; d *= 4, src ^= 1)
     TRY(launch(h, k_aff_level, g.nslot, sa, st, g, src, d, fwd, sa));
-  TRY(launch(h, k_aff_down, g.nslot, sa, st, g, mode, src, sa));
+  const int sd = smem_aff_down(g.n);
+  TRY(launch(h, k_aff_down, g.nslot, sd, st, g, mode, src, sd));
   return ECLQR_OK;
 }
 

@@ -35,6 +35,8 @@ __host__ int smem_lqr_level(int n) {
 }
 __host__ int smem_riccati_finish(int n, int m) { return std::max(m * (n + m + 1) + m * (n + 1) + m + 8, n * n); }
 __host__ int smem_aff(int n, int m) { return 2 * (n * n + n) + n * n + 5 * n + 2 * m + 8; }
+constexpr int kAffRing = 6;  // stages of k_aff_down in shared memory: one in use, five on their way
+__host__ int smem_aff_down(int n) { return kAffRing * n * (n + 1) + 2 * n; }
 
 // Cost-relation slot layout (ld 2n + 1): constraint rows at 0 (CI_ROWS of them),
 // cost rows at offset 2n (2n + 1) (CI_ROWS2 of them); CI_NA / CI_NB are the
@@ -272,6 +274,12 @@ __host__ int smem_riccati(int n, int m) {
 __device__ __forceinline__ void copy_async(double *dst, const double *src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
 }
+__device__ __forceinline__ void copy_async16(double *dst, const double *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int K>  // at most the K newest groups are still in flight
+__device__ __forceinline__ void copy_wait_ring() { asm volatile("cp.async.wait_group %0;" ::"n"(K) : "memory"); }
 __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 __device__ __forceinline__ void team_sync() {
@@ -1025,103 +1033,127 @@ __global__ void k_aff_level(Group g, int src, int d, int fwd, int per_task) {
 
 // The chain of one chunk: y_out = G_i y_in + gv_i stage after stage, G_i = Phi_i
 // (ROLL, CROLL), Phi_i' (PLIN, backward) or Pnu_i (NU), gv_i from k_aff_prep (pnu
-// for NU).  Each output row is a dot product split over seg lanes (seg a power of
-// two with seg * n <= the team), so its dependent chain is about n / seg FMAs and
-// log2(seg) shuffle additions; the lanes load the next stage's G and gv into
-// registers while the current stage runs, and y alternates between two buffers,
-// one barrier per stage.
-__global__ void k_aff_down(Group g, int mode, int fin, int per_task) {
+// for NU).  Each output row is a dot product split over seg lanes, so its dependent
+// chain is about n / seg FMAs and log2(seg) shuffle additions, one barrier per stage
+// (y alternates between two buffers).
+//
+// What bounds it: the latency of one stage, 64 cycles for each FP64 instruction of that
+// chain.  A stage's G and gv are one block of n (n + 1) doubles that does not depend on the
+// chain, so they are copied to shared memory kAffRing - 1 stages ahead: with the next stage
+// alone in flight (in registers) every stage waited for memory instead, 0.70 us a stage at
+// n = 4 and n = 16.  seg = 4 from n = 8 and 2 below; a wider split adds a shuffle and an
+// addition for the FMAs it saves, which pays from n = 24 on where the team has the lanes.
+template <int SEG>
+static __device__ __forceinline__ void aff_chain(const Group &g, const ProbInfo &P, int mode, int a, int b, int dcur,
+                                                 const double *sv) {
+  const int n = g.n, tid = team_rank(), lane = tid & 31;
+  const bool fwd = aff_forward(mode), tr = mode == AFF_PLIN;
+  const int off = aff_out(g, mode), blk = n * (n + 1), steps = b - a;
+  double *ya = g_smem + kAffRing * blk, *yb = ya + n;
+  const int q = tid & (SEG - 1), row = tid / SEG;  // this lane's row and column offset
+  // stages in the order of the sweep
+  const int first = P.st0 + (fwd ? a : b - 1), dir = fwd ? 1 : -1;
+  const ptrdiff_t step = (ptrdiff_t)dir * g.ws.stride;
+  const double *src = stage_ws(g, first) + (mode == AFF_NU ? g.ws.Pnu : g.ws.Phi) + 2 * tid;
+  double *o = stage_ws(g, first) + off + tid;
+  int sent = 0;
+  auto fetch = [&](int slot) {
+    if (sent < steps) {
+      double *dst = g_smem + slot * blk;
+      for (int i = 2 * tid; i < blk; i += 2 * TEAM) copy_async16(dst + i, src + (i - 2 * tid));
+      src += step;
+      sent++;
+    }
+    copy_commit();
+  };
+#pragma unroll
+  for (int k = 0; k < kAffRing - 1; k++) fetch(k);
+  // output dimensions of the stages k0 .. k0 + 31, one per lane, and of the 32 after them
+  auto dims = [&](int k0) {
+    const int k = k0 + lane;
+    return k < steps ? aff_dim(g, first + dir * k + (fwd ? 1 : 0), mode) : 0;
+  };
+  int dreg = dims(0), dnext = dims(32);
+  for (int i = tid; i < n; i += TEAM) {
+    const double v = sv && i < dcur ? sv[i] : 0.0;
+    ya[i] = v;
+    if (!fwd && b == P.N) stage_ws(g, P.st0 + b)[off + i] = v;
+  }
+  // this lane's first entry of a block, and the distance to the next ones
+  const int g0 = tr ? q * n + row : row * n + q, gs = tr ? SEG * n : SEG;
+  constexpr int KP = 4;
+  int slot = 0;
+  const double *G = g_smem;
+  for (int k = 0; k < steps; k++) {
+    copy_wait_ring<kAffRing - 2>();  // this thread's share of stage k
+    if (blockDim.x == 32) __syncwarp();
+    else __syncthreads();  // every thread's; y of the stage before; its block is free
+    const int dout = __shfl_sync(kFull, dreg, k & 31);
+    const bool on = row < dout;
+    // batches of KP entries and y's: the loads of a batch are in flight together
+    double acc = on && q == 0 ? G[n * n + row] : 0.0;
+    const double *Gr = G + g0, *yq = ya + q;
+    for (int l = q; l - q < dcur; l += KP * SEG, Gr += KP * gs, yq += KP * SEG) {
+      double gr[KP], yr[KP];
+#pragma unroll
+      for (int j = 0; j < KP; j++) {
+        const bool in = on && l + j * SEG < dcur;
+        gr[j] = in ? Gr[j * gs] : 0.0;
+        yr[j] = in ? yq[j * SEG] : 0.0;
+      }
+#pragma unroll
+      for (int j = 0; j < KP; j++)
+        if (l - q + j * SEG < dcur) acc = fma(gr[j], yr[j], acc);
+    }
+    fetch(slot == 0 ? kAffRing - 1 : slot - 1);
+    if (fwd && tid < n) *o = tid < dcur ? ya[tid] : 0.0;  // the value of the stage is the chain's input
+#pragma unroll
+    for (int s = SEG >> 1; s > 0; s >>= 1) acc += __shfl_xor_sync(kFull, acc, s);
+    if (q == 0 && row < n) {
+      yb[row] = acc;
+      if (!fwd) o[row - tid] = acc;  // the chain's output is the value of the stage
+    }
+    if ((k & 31) == 31) {
+      dreg = dnext;
+      dnext = dims(k + 33);
+    }
+    o += step;
+    double *tmp = ya; ya = yb; yb = tmp;
+    dcur = dout;
+    G += blk;
+    if (++slot == kAffRing) {
+      slot = 0;
+      G = g_smem;
+    }
+  }
+  if (fwd && b == P.N) {
+    tsync();
+    if (tid < n) *o = tid < dcur ? ya[tid] : 0.0;
+  }
+}
+
+__global__ void k_aff_down(Group g, int mode, int fin, int /*per_task*/) {
   const int t = team_task();
   if (t >= g.nslot) return;
   const ChunkInfo ci = g.chunk[t];
   const ProbInfo &P = g.prob[ci.prob];
   if (skipped_by_mask(g, ci.prob)) return;
   if (ci.c >= P.nch) return;
-  const int n = g.n, tid = team_rank();
-  const bool fwd = aff_forward(mode), tr = mode == AFF_PLIN;
-  const int a = ci.c * P.L, b = min(a + P.L, P.N);
-  const int off = aff_out(g, mode);
-  const int goff = mode == AFF_NU ? g.ws.Pnu : g.ws.Phi, voff = mode == AFF_NU ? g.ws.pnu : g.ws.gv;
-  double *sm = team_smem(per_task);
-  double *ya = sm, *yb = ya + n;
-  int seg = 8;
-  while (seg > 1 && seg * n > TEAM) seg >>= 1;
-  const int q = tid & (seg - 1), row = tid / seg;  // this lane's row and column offset
-  // boundary value after the scan: forward slot (ch0 + c) = y_a; backward slot (ch0 + c + 1) = y_b
+  const int n = g.n, a = ci.c * P.L, b = min(a + P.L, P.N);
+  const bool fwd = aff_forward(mode);
+  // boundary value: with one chunk the problem's own (z_0, 0, rq_N or nu_0); after the scan the
+  // forward slot (ch0 + c) = y_a, the backward slot (ch0 + c + 1) = y_b
   const int slot = fwd ? P.ch0 + ci.c : P.ch0 + ci.c + 1;
-  const double *sv = g.CS[fin] + (size_t)slot * g.cs_stride + n * n;
-  int dcur = fwd ? aff_dim(g, P.st0 + a, mode) : aff_dim(g, P.st0 + b, mode);
-  for (int i = tid; i < n; i += TEAM) ya[i] = (i < dcur) ? sv[i] : 0.0;
-  // stage k of the sweep (k = 0 .. b - a - 1): its stage, and its output dimension
-  auto stage_of = [&](int k) { return P.st0 + (fwd ? a + k : b - 1 - k); };
-  auto dout_of = [&](int s) { return fwd ? aff_dim(g, s + 1, mode) : aff_dim(g, s, mode); };
-  // registers: this lane's entries of G (columns q, q + seg, q + 2 seg, q + 3 seg) and gv
-  constexpr int KP = 4;
-  double gr[KP], gvr = 0.0;
-  auto load = [&](int s, int din, int dout, double *gx, double &gvx) {
-    const double *G = stage_ws(g, s) + goff;
-#pragma unroll
-    for (int k = 0; k < KP; k++) {
-      const int l = q + k * seg;
-      gx[k] = (row < dout && l < din) ? (tr ? G[l * n + row] : G[row * n + l]) : 0.0;
-    }
-    gvx = (row < dout && q == 0) ? stage_ws(g, s)[voff + row] : 0.0;
-  };
-  const int steps = b - a;
-  if (!fwd && b == P.N) {
-    double *o = stage_ws(g, P.st0 + b) + off;
-    for (int r = tid; r < n; r += TEAM) o[r] = (r < dcur) ? ya[r] : 0.0;
-  }
-  int s = steps > 0 ? stage_of(0) : 0;
-  int dout = steps > 0 ? dout_of(s) : 0;
-  // the output dimension of the next stage, read one stage ahead of its map's entries so
-  // that the two global reads do not follow each other on the chain
-  int dpre = steps > 1 ? dout_of(stage_of(1)) : 0;
-  if (steps > 0) load(s, dcur, dout, gr, gvr);
-  tsync();
-  for (int k = 0; k < steps; k++) {
-    if (fwd) {  // the value of stage s is the chain's input
-      double *o = stage_ws(g, s) + off;
-      for (int r = tid; r < n; r += TEAM) o[r] = (r < dcur) ? ya[r] : 0.0;
-    }
-    // next stage's entries, in flight while this stage runs
-    double gn[KP], gvn = 0.0;
-    int sn = s, dn = 0;
-    if (k + 1 < steps) {
-      sn = stage_of(k + 1);
-      dn = dpre;
-      load(sn, dout, dn, gn, gvn);
-      if (k + 2 < steps) dpre = dout_of(stage_of(k + 2));
-    }
-    double acc = 0.0;
-#pragma unroll
-    for (int kk = 0; kk < KP; kk++) {
-      const int l = q + kk * seg;
-      if (l < dcur) acc = fma(gr[kk], ya[l], acc);
-    }
-    if (row < dout) {  // columns beyond the registers (teams too small for seg = 8)
-      const double *G = stage_ws(g, s) + goff;
-      for (int l = q + KP * seg; l < dcur; l += seg) acc = fma(tr ? G[l * n + row] : G[row * n + l], ya[l], acc);
-    }
-    for (int o = seg >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
-    if (q == 0 && row < dout) yb[row] = gvr + acc;
-    tsync();
-    double *tmp = ya; ya = yb; yb = tmp;
-    if (!fwd) {  // the chain's output is the value of stage s
-      double *o = stage_ws(g, s) + off;
-      for (int r = tid; r < n; r += TEAM) o[r] = (r < dout) ? ya[r] : 0.0;
-    }
-    dcur = dout;
-    s = sn;
-    dout = dn;
-#pragma unroll
-    for (int kk = 0; kk < KP; kk++) gr[kk] = gn[kk];
-    gvr = gvn;
-  }
-  if (fwd && b == P.N) {
-    double *o = stage_ws(g, P.st0 + b) + off;
-    for (int r = tid; r < n; r += TEAM) o[r] = (r < dcur) ? ya[r] : 0.0;
-  }
+  const double *end = stage_ws(g, fwd ? P.st0 : P.st0 + P.N);
+  const double *sv = P.nch > 1 ? g.CS[fin] + (size_t)slot * g.cs_stride + n * n
+                               : mode == AFF_CROLL ? nullptr
+                                                   : end + (mode == AFF_ROLL ? g.ws.z : mode == AFF_PLIN ? g.ws.rq : g.ws.nu);
+  const int d0 = aff_dim(g, P.st0 + (fwd ? a : b), mode);
+  const int lanes = TEAM / n;
+  if (n >= 24 && lanes >= 8) aff_chain<8>(g, P, mode, a, b, d0, sv);
+  else if (n >= 8 && lanes >= 4) aff_chain<4>(g, P, mode, a, b, d0, sv);
+  else if (lanes >= 2) aff_chain<2>(g, P, mode, a, b, d0, sv);
+  else aff_chain<1>(g, P, mode, a, b, d0, sv);
 }
 
 // ----------------------------------------------------------- stage-parallel helpers of the solve

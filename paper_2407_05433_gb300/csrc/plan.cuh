@@ -44,7 +44,7 @@ struct WsLayout {
   int LT, lt;   // Cholesky factor L' of the reduced stage Hessian in the order (v, z), upper
                 // triangular (L L' = [Rbar Mbar'; Mbar Qbar]), and L^{-1} [rbar; qbar]
   int Rv;       // the Riccati QR's rows of the minimiser, (R_vv | R_vz | o_v), ld n + m + 1
-  int gv;       // offset of the affine chain's stage map (k_aff_prep), n
+  int gv;       // offset of the affine chain's stage map (k_aff_prep), n, right after Phi
   int Hpre;     // the stage's own rows projected onto x_i (k_primal_stage), n x (n + 1)
   int stride;
 };
@@ -72,7 +72,9 @@ __host__ __device__ inline WsLayout make_ws_layout(int n, int m, int pmax, int q
   L.K = take(m * n);
   L.k = take(m);
   L.Lh = take(m * m);
+  o = (o + 1) & ~1;  // k_aff_down copies [Phi | gv] and [Pnu | pnu] as blocks of 16-byte units
   L.Phi = take(n * n);
+  L.gv = take(n);
   L.z = take(n);
   L.v = take(m);
   L.pi = take(n);
@@ -85,6 +87,7 @@ __host__ __device__ inline WsLayout make_ws_layout(int n, int m, int pmax, int q
   L.pp = take(n);
   L.nu = take(n);
   L.NH = take(n * (n + 1));
+  o = (o + 1) & ~1;
   L.Pnu = take(n * n);
   L.pnu = take(n);
   L.UA = take(n * n);
@@ -95,7 +98,6 @@ __host__ __device__ inline WsLayout make_ws_layout(int n, int m, int pmax, int q
   L.LT = take((n + m) * (n + m));
   L.lt = take(n + m);
   L.Rv = take(m * (n + m + 1));
-  L.gv = take(n);
   L.Hpre = take(n * (n + 1));
   L.stride = (o + 3) & ~3;
   return L;
