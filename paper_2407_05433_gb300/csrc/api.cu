@@ -118,11 +118,15 @@ int team_for(const eclqr_handle *h, const void *kern, int ntasks, int n) {
   if (h->opt.team_warps != 0) return h->opt.team_warps;
   // the affine chains' rows and their segments fill one warp up to n = 8, two to 16
   if (ntasks < h->sms && kern == (const void *)k_aff_down) return n <= 8 ? 1 : n <= 16 ? 2 : kTeamWarps;
+  if (kern == (const void *)k_riccati_down && ntasks < kManyTasksPerSm * h->sms) {
+    // up to two sweeps per SM: the products of a stage spread over more warps
+    return ntasks > 2 * h->sms || n < 16 ? kTeamWarps : n < 24 ? 8 : 16;
+  }
   if (ntasks < h->sms) return kTeamWarps;
   // warps below n1, from n1, n2 and n3 up; few: warps with one to four tasks per SM (-1: the
   // entry, 0: the entry, at least two -- 256 problems of 256 stages, n = 16: 37 ms with two, 42 with one, 49 with four)
   static const struct { const void *fn; int warps, few, n1, warps1, n2, warps2, n3, warps3; } table[] = {
-      {(const void *)k_riccati_down, 1, 4, 12, 2, 16, 4},
+      {(const void *)k_riccati_down, 1, 0, 12, 2, 16, 4},
       {(const void *)k_riccati_down_f32, 1},     {(const void *)k_riccati_finish, 1},
       {(const void *)k_elim, 1, 0, 16, 2, 24, 4}, {(const void *)k_primal_down, 1, 0, 24, 2},
       {(const void *)k_dual_down, 1},            {(const void *)k_primal_stage, 1, 0, 24, 2},

@@ -229,10 +229,10 @@ __global__ void k_lqr_level(Group g, int src, int d, int per_task) {
 // The blocks are offsets into the task's shared memory (in elements of their type), so that every
 // access compiles to a shared-memory instruction with a 32-bit address.
 struct RiccatiFx {
-  int oP, oW, oG, oA, oI, ldp, ldx;
+  int oP, oW, oG, oA, oI, oV, ldp, ldx;
   __host__ __device__ static int words(int n, int m) {  // 8-byte words
     const int ldx = n + m + 1, big = n > m ? n : m;
-    return 2 * (p_size(n, m) + big * ldx + (n + m) * (n + m + 1) / 2 + n + m) + n * ldx + (3 * ldx + m + 2) / 2 + 1;
+    return 2 * (p_size(n, m) + big * ldx + (n + m) * (n + m + 1) / 2 + n + m) + n * ldx + (3 * ldx + m + 2) / 2 + 4;
   }
   // the block of P, which later holds the stage Hessian's doubles
   __host__ __device__ static int p_size(int n, int m) {
@@ -247,6 +247,7 @@ struct RiccatiFx {
     oG = oW + (n > m ? n : m) * ldx;
     oA = 2 * (oG + (n + m) * (n + m + 1) / 2 + n + m);
     oI = 2 * (oA + n * ldx);
+    oV = oA + n * ldx + (3 * ldx + m + 2) / 2;
   }
   __device__ int4 &P(int i) const { return ((int4 *)g_smem)[oP + i]; }  // [P | p] (ld n + 1)
   __device__ int4 &W(int i) const { return ((int4 *)g_smem)[oW + i]; }  // P [Bbar Abar cbar]; the pivots' multipliers
@@ -261,6 +262,8 @@ struct RiccatiFx {
   __device__ int &e(int i) const { return ((int *)g_smem)[oI + ldx + i]; }
   __device__ int &eP(int i) const { return ((int *)g_smem)[oI + 2 * ldx + i]; }
   __device__ int &hp(int i) const { return ((int *)g_smem)[oI + 3 * ldx + 1 + i]; }
+  // the current pivot's reciprocal, its residual and the offsets' excess bits
+  __device__ long long &piv(int i) const { return ((long long *)g_smem)[oV + i]; }
   __device__ int &bad() const { return ((int *)g_smem)[oI + 3 * ldx]; }
 };
 // the blocks of RiccatiFx, or the FP32 sweep's (V, stacked rows, two vectors, gains and stage
@@ -497,21 +500,31 @@ static __device__ __forceinline__ void riccati_stage(const Group &g, const Ricca
 #pragma unroll 1
   for (int k = 0; k < mu; k++) {
     const int gk = packed(k, 0);
-    i128 d = fx_join4(w.G(gk + k));
-    if (d <= 0) d = (i128)1 << (kFxP - 53);  // rounding noise of a singular pivot
-    const int h = (kFxP - fx_bits(d)) >> 1;
-    const i128 dp = d << (2 * h);
-    const long long g0 = fx_rcp((unsigned long long)(dp >> 50));
-    const int2 g2 = fx_split(g0);
-    FxAcc acc;
-    acc.zero();
-    acc.mad(fx_split4(dp), g2);
-    const long long r = (long long)(((i128)1 << kFxP) - acc.value<55>());
-    // the offsets' column has no bound by the diagonal: where the shift would pass 2^116, its
-    // exponent is raised first
-    const int over = fx_bits(fx_join4(w.G(gk + kh))) + h - 116;
+    if (tid < 32) {  // one long chain of scalars: the other warps wait for it instead of repeating it
+      i128 d = fx_join4(w.G(gk + k));
+      const bool noise = d <= 0;
+      if (noise) d = (i128)1 << (kFxP - 53);  // rounding noise of a singular pivot
+      const int h = (kFxP - fx_bits(d)) >> 1;
+      const i128 dp = d << (2 * h);
+      const unsigned long long g0 = (unsigned long long)fx_rcp((unsigned long long)(dp >> 50));
+      // 2^114 - (dp g0 >> 55), below 2^63: the low 64 bits are all of it
+      const unsigned long long lo = (unsigned long long)dp, t = (__umul64hi(lo, g0) << 9) | ((lo * g0) >> 55);
+      // the offsets' column has no bound by the diagonal: where the shift would pass 2^116, its
+      // exponent is raised first
+      const int over = fx_bits(fx_join4(w.G(gk + kh))) + h - 116;
+      if (tid == 0) {
+        if (noise) w.G(gk + k) = fx_split4(d);
+        w.hp(k) = h;
+        w.piv(0) = (long long)g0;
+        w.piv(1) = (long long)(0ull - (((unsigned long long)(dp >> 64) * g0) << 9) - t);
+        w.piv(2) = over;
+      }
+    }
+    team_sync();
+    const int h = w.hp(k), over = (int)w.piv(2);
+    const int2 g2 = fx_split(w.piv(0));
+    const long long r = w.piv(1);
     if (over > 0) {
-      team_sync();
 #pragma unroll 1
       for (int i = tid; i < kh; i += TEAM) {
         const int x = packed(i, kh);
@@ -521,11 +534,10 @@ static __device__ __forceinline__ void riccati_stage(const Group &g, const Ricca
       if (tid == 0) w.e(kh) += over;
       team_sync();
     }
-    if (tid == 0) w.hp(k) = h;
-    team_sync();  // every thread has read row k before it is rewritten
+    FxAcc acc;
 #pragma unroll 1
     for (int j = k + tid; j < ld; j += TEAM) {
-      const i128 y = j == k ? d << h : fx_join4(w.G(gk + j)) << h;
+      const i128 y = fx_join4(w.G(gk + j)) << h;
       const int4 y4 = fx_split4(y);
       w.G(gk + j) = y4;
       acc.zero();
@@ -566,18 +578,18 @@ static __device__ __forceinline__ void riccati_stage(const Group &g, const Ricca
   // the minimiser's rows y_j / sqrt(d 2^(2h))
   const bool bad = w.bad() != 0;
   if (Rv) {
+    // every row at once, from the packed rows 0 .. mu - 1
+    int k = 0, row = 0;
 #pragma unroll 1
-    for (int k = 0; k < mu; k++) {
-      const int gk = packed(k, 0);
-      const unsigned long long rs = fx_rsqrt((unsigned long long)((fx_join4(w.G(gk + k)) << w.hp(k)) >> 50));
-#pragma unroll 1
-      for (int j = k + tid; j < ld; j += TEAM) {
-        int s;
-        const long long top = fx_lead(fx_join4(w.G(gk + j)), s);
-        // (4 d)^(-1/2) 2^62, so the value is 2 2^(s - 114 + 2) of the product's upper half
-        const double x = fx_to(__mul64hi(top, (long long)rs), s + 3 - kFxP + w.e(j));
-        Rv[k * (n + m + 1) + j] = bad ? __longlong_as_double(0x7ff8000000000000ll) : x;
-      }
+    for (int idx = tid; idx < packed(mu, mu); idx += TEAM) {
+      while (idx - row >= ld - k) row += ld - k++;
+      const int j = k + idx - row;
+      const unsigned long long rs = fx_rsqrt((unsigned long long)((fx_join4(w.G(row)) << w.hp(k)) >> 50));
+      int s;
+      const long long top = fx_lead(fx_join4(w.G(idx)), s);
+      // (4 d)^(-1/2) 2^62, so the value is 2 2^(s - 114 + 2) of the product's upper half
+      const double x = fx_to(__mul64hi(top, (long long)rs), s + 3 - kFxP + w.e(j));
+      Rv[k * (n + m + 1) + j] = bad ? __longlong_as_double(0x7ff8000000000000ll) : x;
     }
   }
   team_sync();
