@@ -120,7 +120,7 @@ int team_for(const eclqr_handle *h, const void *kern, int ntasks, int n) {
   if (ntasks < h->sms && kern == (const void *)k_aff_down) return n <= 8 ? 1 : n <= 16 ? 2 : kTeamWarps;
   if (kern == (const void *)k_riccati_down && ntasks < kManyTasksPerSm * h->sms) {
     // up to two sweeps per SM: the products of a stage spread over more warps
-    return ntasks > 2 * h->sms || n < 16 ? kTeamWarps : n < 24 ? 8 : 16;
+    return ntasks > 2 * h->sms || n < 12 ? kTeamWarps : n < 24 ? 8 : 16;
   }
   if (ntasks < h->sms) return kTeamWarps;
   // warps below n1, from n1, n2 and n3 up; few: warps with one to four tasks per SM (-1: the

@@ -229,25 +229,23 @@ __global__ void k_lqr_level(Group g, int src, int d, int per_task) {
 // The blocks are offsets into the task's shared memory (in elements of their type), so that every
 // access compiles to a shared-memory instruction with a 32-bit address.
 struct RiccatiFx {
-  int oP, oW, oG, oA, oI, oV, ldp, ldx;
+  int oP, oW, oG, oA, oH, oI, oV, ldp, ldx;
   __host__ __device__ static int words(int n, int m) {  // 8-byte words
     const int ldx = n + m + 1, big = n > m ? n : m;
-    return 2 * (p_size(n, m) + big * ldx + (n + m) * (n + m + 1) / 2 + n + m) + n * ldx + (3 * ldx + m + 2) / 2 + 4;
+    return 2 * (n * (n + 1) + big * ldx + g_size(n, m)) + n * ldx + g_size(n, m) + (3 * ldx + m + 2) / 2 + 4;
   }
-  // the block of P, which later holds the stage Hessian's doubles
-  __host__ __device__ static int p_size(int n, int m) {
-    const int h = ((n + m) * (n + m + 1) / 2 + n + m + 1) / 2;
-    return n * (n + 1) > h ? n * (n + 1) : h;
-  }
+  // entries of G's and H's packed rows
+  __host__ __device__ static int g_size(int n, int m) { return (n + m) * (n + m + 1) / 2 + n + m; }
   __device__ RiccatiFx(int n, int m) {
     ldp = n + 1;
     ldx = n + m + 1;
     oP = 0;
-    oW = p_size(n, m);
+    oW = n * (n + 1);
     oG = oW + (n > m ? n : m) * ldx;
-    oA = 2 * (oG + (n + m) * (n + m + 1) / 2 + n + m);
-    oI = 2 * (oA + n * ldx);
-    oV = oA + n * ldx + (3 * ldx + m + 2) / 2;
+    oA = 2 * (oG + g_size(n, m));
+    oH = oA + n * ldx;
+    oI = 2 * (oH + g_size(n, m));
+    oV = oH + g_size(n, m) + (3 * ldx + m + 2) / 2;
   }
   __device__ int4 &P(int i) const { return ((int4 *)g_smem)[oP + i]; }  // [P | p] (ld n + 1)
   __device__ int4 &W(int i) const { return ((int4 *)g_smem)[oW + i]; }  // P [Bbar Abar cbar]; the pivots' multipliers
@@ -255,7 +253,7 @@ struct RiccatiFx {
   __device__ i128 &Gi(int i) const { return ((i128 *)g_smem)[oG + i]; }
   __device__ int2 &A(int i) const { return ((int2 *)g_smem)[oA + i]; }  // [Bbar | Abar | cbar] (n x ldx)
   __device__ double &Ad(int i) const { return g_smem[oA + i]; }         // the same as doubles
-  __device__ double &H(int i) const { return g_smem[2 * oP + i]; }      // [Rbar Mbar'; Mbar Qbar | rbar; qbar], packed
+  __device__ double &H(int i) const { return g_smem[oH + i]; }          // [Rbar Mbar'; Mbar Qbar | rbar; qbar], packed
   // column exponents of A (rows weighted by P's), of G, and of P (eP(nx): that of p); the pivots'
   // shifts; a flag: a value that is not finite was met
   __device__ int &al(int i) const { return ((int *)g_smem)[oI + i]; }
@@ -354,20 +352,102 @@ static __device__ __forceinline__ void riccati_fetch(const Group &g, const Ricca
   }
 }
 
-// One stage: from w.P, w.eP (n1 states) and the fetched w.Ad to the value of the stage's nx
-// states.  Rv: the minimiser's rows (ld n + m + 1); Po, po: P_i and p_i; null where the stage is not
-// stored.  fetch() starts the copy of the next stage's w.Ad.
-template <typename Fetch>
-static __device__ __forceinline__ void riccati_stage(const Group &g, const RiccatiFx w, const double *ws, int n1, int nx,
-                                                     int mu, double *Rv, double *Po, double *po, Fetch fetch) {
-  const int n = g.n, m = g.m, tid = team_rank();
-  const int kh = nx + mu, ld = kh + 1, ldx = w.ldx, ldp = w.ldp;
+// Starts the copy of a stage's H and h in the order (v, z, 1), packed rows, into w.H.
+static __device__ __forceinline__ void riccati_fetch_h(const Group &g, const RiccatiFx w, const double *ws, int nx, int mu) {
+  const int n = g.n, m = g.m, kh = nx + mu, ld = kh + 1;
   const double *Qb = ws + g.ws.Qb, *Mb = ws + g.ws.Mb, *Rb = ws + g.ws.Rb, *qb = ws + g.ws.qb, *rb = ws + g.ws.rb;
-  auto hess = [&](int j, int k) {  // H and h in the order (v, z, 1), j <= k
-    if (k == kh) return j < mu ? rb + j : qb + (j - mu);
-    if (k < mu) return Rb + j * m + k;
-    return j < mu ? Mb + (k - mu) * m + j : Qb + (j - mu) * n + (k - mu);
-  };
+  int j = 0, row = 0;
+#pragma unroll 1
+  for (int idx = team_rank(); idx < kh * (kh + 1) / 2 + kh; idx += TEAM) {
+    while (idx - row >= ld - j) row += ld - j++;
+    const int k = j + idx - row;
+    const double *src;
+    if (k == kh) src = j < mu ? rb + j : qb + (j - mu);
+    else if (k < mu) src = Rb + j * m + k;
+    else src = j < mu ? Mb + (k - mu) * m + j : Qb + (j - mu) * n + (k - mu);
+    copy_async(&w.H(idx), src);
+  }
+}
+
+// W = P [Bbar | Abar | cbar] + [0 | 0 | p] in units of 2^-111: T x T entries per item
+template <int T>
+static __device__ __forceinline__ void riccati_w(const RiccatiFx w, int n1, int kh) {
+  const int ld = kh + 1, ldx = w.ldx, ldp = w.ldp, cols = (ld + T - 1) / T;
+  const float rcols = rcp_seed((float)cols);
+#pragma unroll 1
+  for (int it = team_rank(); it < cols * ((n1 + T - 1) / T); it += TEAM) {
+    const int rp = (int)(((float)it + 0.5f) * rcols), c = T * (it - rp * cols), r = T * rp;
+    const int r1 = min(r + T - 1, n1 - 1), c1 = min(c + T - 1, kh);
+    FxAcc acc[T * T];
+#pragma unroll
+    for (int q = 0; q < T * T; q++) acc[q].zero();
+    int i0 = r * ldp, i1 = r1 * ldp, j0 = c, j1 = c1;
+#pragma unroll 2
+    for (int l = 0; l < n1; l++, i0++, i1++, j0 += ldx, j1 += ldx) {
+      const int4 x0 = w.P(i0);
+      const int2 a0 = w.A(j0);
+      acc[0].mad(x0, a0);
+      if (T == 2) {
+        const int4 x1 = w.P(i1);
+        const int2 a1 = w.A(j1);
+        acc[1 % (T * T)].mad(x0, a1);
+        acc[2 % (T * T)].mad(x1, a0);
+        acc[3 % (T * T)].mad(x1, a1);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < T * T; q++) {
+      const int rr = q < T ? r : r1, cc = T == 2 && (q & 1) ? c1 : c;
+      i128 v = acc[q].template value<60>();
+      if (cc == kh) v += fx_shift(fx_join4(w.P(rr * ldp + n1)), w.eP(n1) - w.al(kh) - 3);
+      w.W(rr * ldx + cc) = fx_split4(v);
+    }
+  }
+}
+
+// raw G = [Bbar Abar]' W in units of 2^-114: T x T entries (j, k), j <= k, per item
+template <int T>
+static __device__ __forceinline__ void riccati_g(const RiccatiFx w, int n1, int kh) {
+  const int ld = kh + 1, ldx = w.ldx, cols = (ld + T - 1) / T;
+  int jt = 0, start = 0;  // block row jt: block columns jt .. cols - 1
+#pragma unroll 1
+  for (int it = team_rank();; it += TEAM) {
+    while (T * jt < kh && it - start >= cols - jt) start += cols - jt++;
+    if (T * jt >= kh) break;
+    const int j = T * jt, j1 = min(j + T - 1, kh - 1), k = j + T * (it - start), k1 = min(k + T - 1, kh);
+    FxAcc acc[T * T];
+#pragma unroll
+    for (int q = 0; q < T * T; q++) acc[q].zero();
+    int ia = j, ib = j1, ka = k, kb = k1;
+#pragma unroll 2
+    for (int l = 0; l < n1; l++, ia += ldx, ib += ldx, ka += ldx, kb += ldx) {
+      const int4 x0 = w.W(ka);
+      const int2 a0 = w.A(ia);
+      acc[0].mad(x0, a0);
+      if (T == 2) {
+        const int4 x1 = w.W(kb);
+        const int2 a1 = w.A(ib);
+        acc[1 % (T * T)].mad(x1, a0);
+        acc[2 % (T * T)].mad(x0, a1);
+        acc[3 % (T * T)].mad(x1, a1);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < T * T; q++) {
+      const int jj = q < T ? j : j1, kk = T == 2 && (q & 1) ? k1 : k;
+      if (jj <= kk) w.Gi(riccati_packed(ld, jj, kk)) = acc[q].template value<54>();
+    }
+  }
+}
+
+// One stage: from w.P, w.eP (n1 states) and the fetched w.Ad and w.H to the value of the stage's nx
+// states.  Rv: the minimiser's rows (ld n + m + 1); Po, po: P_i and p_i; null where the stage is not
+// stored.  fetch() and fetch_h() start the copies of the next stage's w.Ad and w.H.
+template <typename Fetch, typename FetchH>
+static __device__ __forceinline__ void riccati_stage(const Group &g, const RiccatiFx w, int n1, int nx, int mu,
+                                                     double *Rv, double *Po, double *po, Fetch fetch, FetchH fetch_h) {
+  const int n = g.n, m = g.m, tid = team_rank();
+  const int kh = nx + mu, ld = kh + 1, ldx = w.ldx;
   auto packed = [&](int j, int k) { return riccati_packed(ld, j, k); };
   // [Bbar | Abar | cbar] and its column exponents, the rows weighted by P's exponents
 #pragma unroll 1
@@ -390,73 +470,16 @@ static __device__ __forceinline__ void riccati_stage(const Group &g, const Ricca
     w.A(l * ldx + j) = fx_split(fx_from(w.Ad(l * ldx + j), w.al(j) - w.eP(l)));
   }
   team_sync();
-  // W = P [Bbar | Abar | cbar] + [0 | 0 | p] in units of 2^-111: 2 x 2 entries per item
-  const int c2 = (ld + 1) >> 1;
-  const float rc2 = rcp_seed((float)c2);
-#pragma unroll 1
-  for (int it = tid; it < c2 * ((n1 + 1) >> 1); it += TEAM) {
-    const int rp = (int)(((float)it + 0.5f) * rc2), c = 2 * (it - rp * c2), r = 2 * rp;
-    const int r1 = min(r + 1, n1 - 1), c1 = min(c + 1, kh);
-    FxAcc acc[4];
-#pragma unroll
-    for (int q = 0; q < 4; q++) acc[q].zero();
-    int i0 = r * ldp, i1 = r1 * ldp, j0 = c, j1 = c1;
-#pragma unroll 2
-    for (int l = 0; l < n1; l++, i0++, i1++, j0 += ldx, j1 += ldx) {
-      const int4 x0 = w.P(i0), x1 = w.P(i1);
-      const int2 a0 = w.A(j0), a1 = w.A(j1);
-      acc[0].mad(x0, a0);
-      acc[1].mad(x0, a1);
-      acc[2].mad(x1, a0);
-      acc[3].mad(x1, a1);
-    }
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-      const int rr = q < 2 ? r : r1, cc = (q & 1) ? c1 : c;
-      i128 v = acc[q].value<60>();
-      if (cc == kh) v += fx_shift(fx_join4(w.P(rr * ldp + n1)), w.eP(n1) - w.al(kh) - 3);
-      w.W(rr * ldx + cc) = fx_split4(v);
-    }
-  }
+  // The tiles: 2 x 2 entries per item share their operands, single entries spread over four times the
+  // lanes.  Single entries while the team takes them in one pass and a half: with many sweeps per
+  // SM, whose teams are small, they only add shared-memory loads (640 problems at n = 16, four
+  // warps: 2.7 ms with 2 x 2 tiles, 3.2 with single entries in G alone); with few, the lanes idle
+  // otherwise (one 64-stage sweep at n = 4 410 -> 353 us, 147 chunks at n = 12 178 -> 137).
+  if (2 * n1 * ld > 3 * TEAM) riccati_w<2>(w, n1, kh);
+  else riccati_w<1>(w, n1, kh);
   team_sync();
-  // H and h, into the block of P while G is formed
-  {
-    int j = 0, row = 0;
-#pragma unroll 1
-    for (int idx = tid; idx < kh * (kh + 1) / 2 + kh; idx += TEAM) {
-      while (idx - row >= ld - j) row += ld - j++;
-      copy_async(&w.H(idx), hess(j, j + idx - row));
-    }
-  }
-  // raw G = [Bbar Abar]' W in units of 2^-114: 2 x 2 entries (j, k), j <= k, per item
-  {
-    int jt = 0, start = 0;  // row pair jt: column pairs jt .. c2 - 1
-#pragma unroll 1
-    for (int it = tid;; it += TEAM) {
-      while (2 * jt < kh && it - start >= c2 - jt) start += c2 - jt++;
-      if (2 * jt >= kh) break;
-      const int j = 2 * jt, j1 = min(j + 1, kh - 1), k = j + 2 * (it - start), k1 = min(k + 1, kh);
-      FxAcc acc[4];
-#pragma unroll
-      for (int q = 0; q < 4; q++) acc[q].zero();
-      int ia = j, ib = j1, ka = k, kb = k1;
-#pragma unroll 2
-      for (int l = 0; l < n1; l++, ia += ldx, ib += ldx, ka += ldx, kb += ldx) {
-        const int4 x0 = w.W(ka), x1 = w.W(kb);
-        const int2 a0 = w.A(ia), a1 = w.A(ib);
-        acc[0].mad(x0, a0);
-        acc[1].mad(x1, a0);
-        acc[2].mad(x0, a1);
-        acc[3].mad(x1, a1);
-      }
-#pragma unroll
-      for (int q = 0; q < 4; q++) {
-        const int jj = q < 2 ? j : j1, kk = (q & 1) ? k1 : k;
-        if (jj <= kk) w.Gi(packed(jj, kk)) = acc[q].value<54>();
-      }
-    }
-  }
-  copy_wait();
+  if (kh * (kh + 1) + 2 * kh > 3 * TEAM) riccati_g<2>(w, n1, kh);
+  else riccati_g<1>(w, n1, kh);
   team_sync();
   fetch();
   // exponents of the columns of G + H from its diagonal, of the offsets from their largest entry
@@ -495,6 +518,7 @@ static __device__ __forceinline__ void riccati_stage(const Group &g, const Ricca
     }
   }
   team_sync();
+  fetch_h();
   // pivots on v: y_j = G_kj 2^h, l_j = y_j / (d 2^(2h)) (units of 2^-112, in
   // w.W), G_ij -= l_i y_j for rows i < mu
 #pragma unroll 1
@@ -692,6 +716,7 @@ static __device__ void riccati_task(const Group &g, int fin, int t, int per_task
     nx = stage_wi(g, s)[SI_NBAR];
     mu = stage_wi(g, s)[SI_MBAR];
     riccati_fetch(g, w, stage_ws(g, s), n1, nx, mu);
+    riccati_fetch_h(g, w, stage_ws(g, s), nx, mu);
   }
 #pragma unroll 1
   for (int i = start - 1; i >= a; --i) {
@@ -703,9 +728,12 @@ static __device__ void riccati_task(const Group &g, int fin, int t, int per_task
       nx2 = stage_wi(g, s - 1)[SI_NBAR];
       mu2 = stage_wi(g, s - 1)[SI_MBAR];
     }
-    riccati_stage(g, w, ws, n1, nx, mu, store ? ws + g.ws.Rv : nullptr, store ? ws + g.ws.P : nullptr, ws + g.ws.p,
+    riccati_stage(g, w, n1, nx, mu, store ? ws + g.ws.Rv : nullptr, store ? ws + g.ws.P : nullptr, ws + g.ws.p,
                   [&] {
                     if (i > a) riccati_fetch(g, w, stage_ws(g, s - 1), nx, nx2, mu2);
+                  },
+                  [&] {
+                    if (i > a) riccati_fetch_h(g, w, stage_ws(g, s - 1), nx2, mu2);
                   });
     n1 = nx;
     nx = nx2;
