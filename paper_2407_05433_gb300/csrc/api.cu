@@ -470,7 +470,7 @@ int eclqr_create(const eclqr_desc *d, const eclqr_options *opt, eclqr_handle **o
           {(const void *)k_lqr_up, smem_lqr_up(n, m)}, {(const void *)k_lqr_level, smem_lqr_level(n)},
           {(const void *)k_riccati_down, smem_riccati(n, m)},
           {(const void *)k_riccati_finish, smem_riccati_finish(n, m)}, {(const void *)k_aff_up, sa},
-          {(const void *)k_aff_level, sa}, {(const void *)k_aff_down, smem_aff_down(n)}, {(const void *)k_resid, 3 * n + 2 * m},
+          {(const void *)k_aff_level, sa}, {(const void *)k_aff_down, smem_aff_down(n)}, {(const void *)k_resid, 4 * n + 2 * m},
           {(const void *)k_pcorr, n + m + m * m}, {(const void *)k_dual_stage, smem_dual_stage(n, m)},
           {(const void *)k_dual_terminal, sdw}, {(const void *)k_dual_up, sdw}, {(const void *)k_dual_down, sdw + kHeldScratch},
           {(const void *)k_dual_root, sdw + kHeldScratch}, {(const void *)k_dual_leaf, smem_dual_leaf(n, m, wmax) + kHeldScratch}};
@@ -706,7 +706,7 @@ int run_build(eclqr_handle *h, GroupHost &gh, const Group &g, cudaStream_t gst, 
 int aff_scan(eclqr_handle *h, const GroupHost &gh, const Group &g, int mode, cudaStream_t st) {
   const int sa = smem_aff(g.n, g.m);
   const int fwd = (mode == AFF_PLIN_) ? 0 : 1;
-  TRY(launch(h, k_aff_prep, g.nstage, g.n + 8, st, g, mode, g.n + 8));
+  if (mode == AFF_ROLL_) TRY(launch(h, k_aff_prep, g.nstage, 0, st, g));
   if (gh.levels > 0) TRY(launch(h, k_aff_up, g.nslot, sa, st, g, mode, sa));
   int src = 0;
   // radix-4 levels: strides 1, 4, 16, ... until they cover every slot
@@ -724,7 +724,7 @@ int run_solve(eclqr_handle *h, const GroupHost &gh, const Group &g, cudaStream_t
   TRY(aff_scan(h, gh, g, AFF_ROLL_, gst));
   TRY(launch(h, k_post_roll, g.nstage, 0, gst, g, 0));
   for (int r = 0; r < refine_passes; r++) {
-    const int sres = 3 * g.n + 2 * g.m;
+    const int sres = 4 * g.n + 2 * g.m;
     TRY(launch(h, k_resid, g.nstage, sres, gst, g, sres));
     TRY(aff_scan(h, gh, g, AFF_PLIN_, gst));
     const int sc = g.n + g.m + g.m * g.m;

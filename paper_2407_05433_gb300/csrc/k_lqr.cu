@@ -824,97 +824,33 @@ __device__ __forceinline__ int aff_out(const Group &g, int mode) {
 
 // map of stage i: y_out = G y_in + gv.  Forward: in = stage i, out = stage i+1;
 // backward: in = stage i+1, out = stage i.  G (dout x din, ld n) and gv into smem.
-__device__ void aff_stage_map(const Group &g, int s, int mode, double *G, double *gv, double *tmp) {
-  const int n = g.n, m = g.m, tid = team_rank();
-  const double *ws = stage_ws(g, s), *wn = stage_ws(g, s + 1);
-  const int *wi = stage_wi(g, s);
-  if (mode == AFF_NU) {
-    const int din = wi[SI_UR], dout = stage_wi(g, s + 1)[SI_UR];
-    for (int idx = tid; idx < dout * din; idx += TEAM) {
-      int i = idx / din, j = idx - i * din;
-      G[i * n + j] = ws[g.ws.Pnu + i * n + j];
-    }
-    for (int i = tid; i < dout; i += TEAM) gv[i] = ws[g.ws.pnu + i];
-    tsync();
-    return;
+__device__ void aff_stage_map(const Group &g, int s, int mode, double *G, double *gv) {
+  const int n = g.n, tid = team_rank();
+  const double *ws = stage_ws(g, s), *src = ws + (mode == AFF_NU ? g.ws.Pnu : g.ws.Phi), *v = src + n * n;
+  const int d0 = aff_dim(g, s, mode), d1 = aff_dim(g, s + 1, mode), dout = mode == AFF_PLIN ? d0 : d1;
+  for (int idx = tid; idx < d1 * d0; idx += TEAM) {
+    const int i = idx / d0, j = idx - i * d0;
+    G[mode == AFF_PLIN ? j * n + i : i * n + j] = src[i * n + j];
   }
-  const int nx = wi[SI_NBAR], ny = stage_wi(g, s + 1)[SI_NBAR], mu = wi[SI_MBAR];
-  const double *Phi = ws + g.ws.Phi, *Bb = ws + g.ws.Bb;
-  if (mode == AFF_ROLL || mode == AFF_CROLL) {
-    const double *kk = ws + (mode == AFF_ROLL ? g.ws.k : g.ws.dv);
-    const double *cc = ws + (mode == AFF_ROLL ? g.ws.cb : g.ws.rc);
-    for (int idx = tid; idx < ny * nx; idx += TEAM) {
-      int i = idx / nx, j = idx - i * nx;
-      G[i * n + j] = Phi[i * n + j];
-    }
-    for (int i = tid; i < ny; i += TEAM) {
-      double s0 = cc[i];
-      for (int l = 0; l < mu; l++) s0 = fma(Bb[i * m + l], kk[l], s0);
-      gv[i] = s0;
-    }
-    tsync();
-    return;
-  }
-  // AFF_PLIN: G = Phi' (nx x ny), gv = rq + K' rr + Phi' (P_{i+1} rc)
-  const double *K = ws + g.ws.K, *Pn = wn + g.ws.P, *rc = ws + g.ws.rc;
-  for (int b = tid; b < ny; b += TEAM) {
-    double s0 = 0.0;
-    for (int l = 0; l < ny; l++) s0 = fma(Pn[b * n + l], rc[l], s0);
-    tmp[b] = s0;
-  }
-  for (int idx = tid; idx < nx * ny; idx += TEAM) {
-    int i = idx / ny, j = idx - i * ny;
-    G[i * n + j] = Phi[j * n + i];
-  }
-  tsync();
-  for (int i = tid; i < nx; i += TEAM) {
-    double s0 = ws[g.ws.rq + i];
-    for (int l = 0; l < mu; l++) s0 = fma(K[l * n + i], ws[g.ws.rr + l], s0);
-    for (int b = 0; b < ny; b++) s0 = fma(Phi[b * n + i], tmp[b], s0);
-    gv[i] = s0;
-  }
+  for (int i = tid; i < dout; i += TEAM) gv[i] = v[i];
   tsync();
 }
 
-// The offsets of every stage's map, stage-parallel, before a chain sweeps
-// them (ws.gv; the same arithmetic as aff_stage_map): ROLL cbar + Bbar k,
-// CROLL rc + Bbar k', PLIN rq + K' rr + Phi' P_{i+1} rc.  NU reads pnu.
-__global__ void k_aff_prep(Group g, int mode, int per_task) {
+// The offsets cbar + Bbar k of every stage's map, stage-parallel, before the rollout's chain sweeps
+// them (ws.gv).  k_resid and k_pcorr form those of PLIN and CROLL; NU reads pnu.
+__global__ void k_aff_prep(Group g) {
   for_stages(g, [&](const int s) {
     const StageInfo S = g.st[s];
     const ProbInfo &P = g.prob[S.prob];
     if (skipped_by_mask(g, S.prob)) return;
-    if (S.i >= P.N || mode == AFF_NU) return;
-    const int n = g.n, m = g.m, tid = team_rank();
+    if (S.i >= P.N) return;
+    const int m = g.m, ny = stage_wi(g, s + 1)[SI_NBAR], mu = stage_wi(g, s)[SI_MBAR];
     double *ws = stage_ws(g, s);
-    const double *wn = stage_ws(g, s + 1);
-    const int *wi = stage_wi(g, s);
-    const int nx = wi[SI_NBAR], ny = stage_wi(g, s + 1)[SI_NBAR], mu = wi[SI_MBAR];
-    const double *Phi = ws + g.ws.Phi, *Bb = ws + g.ws.Bb;
-    double *gv = ws + g.ws.gv;
-    if (mode == AFF_ROLL || mode == AFF_CROLL) {
-      const double *kk = ws + (mode == AFF_ROLL ? g.ws.k : g.ws.dv);
-      const double *cc = ws + (mode == AFF_ROLL ? g.ws.cb : g.ws.rc);
-      for (int i = tid; i < ny; i += TEAM) {
-        double s0 = cc[i];
-        for (int l = 0; l < mu; l++) s0 = fma(Bb[i * m + l], kk[l], s0);
-        gv[i] = s0;
-      }
-      return;
-    }
-    double *tmp = team_smem(per_task);  // P_{i+1} rc (ny)
-    const double *K = ws + g.ws.K, *Pn = wn + g.ws.P, *rc = ws + g.ws.rc;
-    for (int b = tid; b < ny; b += TEAM) {
-      double s0 = 0.0;
-      for (int l = 0; l < ny; l++) s0 = fma(Pn[b * n + l], rc[l], s0);
-      tmp[b] = s0;
-    }
-    tsync();
-    for (int i = tid; i < nx; i += TEAM) {
-      double s0 = ws[g.ws.rq + i];
-      for (int l = 0; l < mu; l++) s0 = fma(K[l * n + i], ws[g.ws.rr + l], s0);
-      for (int b = 0; b < ny; b++) s0 = fma(Phi[b * n + i], tmp[b], s0);
-      gv[i] = s0;
+    const double *Bb = ws + g.ws.Bb, *kk = ws + g.ws.k, *cc = ws + g.ws.cb;
+    for (int i = team_rank(); i < ny; i += TEAM) {
+      double s0 = cc[i];
+      for (int l = 0; l < mu; l++) s0 = fma(Bb[i * m + l], kk[l], s0);
+      ws[g.ws.gv + i] = s0;
     }
   });
 }
@@ -975,7 +911,7 @@ __global__ void k_aff_up(Group g, int mode, int per_task) {
   for (int k = 0; k < b - a; k++) {
     const int i = fwd ? a + k : b - 1 - k;
     const int s = P.st0 + i;
-    aff_stage_map(g, s, mode, Gs, gs, tmp);
+    aff_stage_map(g, s, mode, Gs, gs);
     const int dout = fwd ? aff_dim(g, s + 1, mode) : aff_dim(g, s, mode);
     // Tm = Gs Gm (dout x d0), tmp = Gs gm + gs
     wgemm<false, false>(dout, d0, dcur, Gs, n, Gm, n, 0, Tm, n);
@@ -1275,7 +1211,9 @@ __global__ void k_post_roll(Group g, int corr) {
 // cbar + Abar z + Bbar v - z_{i+1}.  Forming Qbar z + qbar instead would sum
 // terms of size |Y|^2 that cancel down to pi: where the mixed rows leave D_i
 // ill-conditioned |Y| is large, and that cancellation would set the accuracy
-// of the costates and so of the multipliers.  Per task: 3n + 2m doubles.
+// of the costates and so of the multipliers.  The offsets that the next pass's chain (PLIN) adds to
+// its maps, rq + K' rr + Phi' P_{i+1} rc (ws.gv), follow from the stage's residual at once, while it
+// is in shared memory.  Per task: 4n + 2m doubles.
 __global__ void k_resid(Group g, int per_task) {
   for_stages(g, [&](const int s) {
     const StageInfo S = g.st[s];
@@ -1292,7 +1230,7 @@ __global__ void k_resid(Group g, int per_task) {
     const double *T = ws + g.ws.UT + ur, *Tn = wn + g.ws.UT + ur1;
     const double *Y = ws + g.ws.Y, *Z = ws + g.ws.Z, *Ab = ws + g.ws.Ab, *Bb = ws + g.ws.Bb;
     double *sm = team_smem(per_task);
-    double *xs = sm, *us = xs + n, *lh = us + m, *ga = lh + n, *gb = ga + n;
+    double *xs = sm, *us = xs + n, *lh = us + m, *ga = lh + n, *gb = ga + n, *rcs = gb + m;
     // T_i = I, t_i = 0 (te) or T_{i+1} = I (tne): the products with them are their other factor
     const bool te = wi[SI_TEYE] != 0, tne = !last && stage_wi(g, s + 1)[SI_TEYE] != 0;
     // One lane per row, rows of different blocks side by side: an FP64 instruction costs its warp
@@ -1333,24 +1271,34 @@ __global__ void k_resid(Group g, int per_task) {
       }
       if (ra) ga[a] = s0;
       else if (rb) gb[a] = s0;
-      else ws[g.ws.rc + a] = s0;
+      else ws[g.ws.rc + a] = rcs[a] = s0;
     }
     tsync();
-    for (int r = tid; r < nx + mu; r += TEAM) {
+    // rq (nx rows, kept in xs), rr (mu, in us), P_{i+1} rc (ny, in lh)
+    const double *Pn = wn + g.ws.P;
+    for (int r = tid; r < nx + mu + ny; r += TEAM) {
       double s0;
       if (r < nx) {
         s0 = te ? ga[r] - pi[r] : dot(-pi[r], T + r, n, ga, n);
         if (!last) s0 = dot(s0, Y + r, n, gb, m);
-        ws[g.ws.rq + r] = s0;
+        ws[g.ws.rq + r] = xs[r] = s0;
+      } else if (r < nx + mu) {
+        s0 = dot(0.0, Z + r - nx, m, gb, m);
+        ws[g.ws.rr + r - nx] = us[r - nx] = s0;
       } else {
-        ws[g.ws.rr + r - nx] = dot(0.0, Z + r - nx, m, gb, m);
+        lh[r - nx - mu] = dot(0.0, Pn + (r - nx - mu) * n, 1, rcs, ny);
       }
     }
+    if (last) return;
+    tsync();
+    const double *K = ws + g.ws.K, *Phi = ws + g.ws.Phi;
+    for (int r = tid; r < nx; r += TEAM) ws[g.ws.gv + r] = dot(dot(xs[r], K + r, n, us, mu), Phi + r, n, lh, ny);
   });
 }
 
 // Correction controls of a refinement pass: with w = P_{i+1} rc_i + p'_{i+1},
-// k'_i = -H_uu^{-1} (rr_i + Bbar' w) through the Cholesky factor of H_uu (-> dv).
+// k'_i = -H_uu^{-1} (rr_i + Bbar' w) through the Cholesky factor of H_uu (-> dv), and the offsets
+// rc + Bbar k' of the chain that follows (CROLL, ws.gv).
 __global__ void k_pcorr(Group g, int per_task) {
   for_stages(g, [&](const int s) {
     const StageInfo S = g.st[s];
@@ -1398,7 +1346,13 @@ __global__ void k_pcorr(Group g, int per_task) {
         const double xl = __shfl_sync(kFull, x, l);
         if (a < l) x = fma(-Ls[l * m + a], xl, x);
       }
-      if (a < mu) ws[g.ws.dv + a] = -x;
+      if (a < mu) ws[g.ws.dv + a] = hu[a] = -x;
+    }
+    tsync();
+    for (int r = tid; r < ny; r += TEAM) {
+      double s0 = rc[r];
+      for (int l = 0; l < mu; l++) s0 = fma(Bb[r * m + l], hu[l], s0);
+      ws[g.ws.gv + r] = s0;
     }
   });
 }
