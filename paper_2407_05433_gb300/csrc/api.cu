@@ -116,8 +116,8 @@ namespace {
 // at n = 24).
 int team_for(const eclqr_handle *h, const void *kern, int ntasks, int n) {
   if (h->opt.team_warps != 0) return h->opt.team_warps;
-  // the affine chains' rows and their segments fill one warp up to n = 8, two to 16
-  if (ntasks < h->sms && kern == (const void *)k_aff_down) return n <= 8 ? 1 : n <= 16 ? 2 : kTeamWarps;
+  // four lanes a row of an affine chain (two below n = 5), and never more than a row's latency pays for
+  if (kern == (const void *)k_aff_down) return n <= 8 ? 1 : n <= 16 ? 2 : 4;
   if (kern == (const void *)k_riccati_down && ntasks < kManyTasksPerSm * h->sms) {
     // up to two sweeps per SM: the products of a stage spread over more warps
     return ntasks > 2 * h->sms || n < 12 ? kTeamWarps : n < 24 ? 8 : 16;
@@ -130,7 +130,7 @@ int team_for(const eclqr_handle *h, const void *kern, int ntasks, int n) {
       {(const void *)k_riccati_down_f32, 1},     {(const void *)k_riccati_finish, 1},
       {(const void *)k_elim, 1, 0, 16, 2, 24, 4}, {(const void *)k_primal_down, 1, 0, 24, 2},
       {(const void *)k_dual_down, 1},            {(const void *)k_primal_stage, 1, 0, 24, 2},
-      {(const void *)k_aff_down, 1, -1, 16, 2, 24, 4, 28, 8}, {(const void *)k_dual_leaf, 1},
+      {(const void *)k_dual_leaf, 1},
       {(const void *)k_aff_prep, 1},             {(const void *)k_stage_lists, 1},
       {(const void *)k_dual_stage, 2},           {(const void *)k_param, 1},
       {(const void *)k_resid, 1},                {(const void *)k_pcorr, 1},
@@ -183,7 +183,9 @@ int launch_grid(eclqr_handle *h, void (*kern)(KArgs...), int ntasks, int grid, i
   const Group &g = group_of(args...);
   // every problem has one slot more than it has chunks to sweep
   const int work = (const void *)kern == (const void *)k_riccati_down ? g.nslot - g.nprob : ntasks;
-  kern<<<grid, 32 * team_for(h, (const void *)kern, work, g.n), smem, st>>>(args...);
+  // k_aff_down has one warp more than its rows take
+  const int warps = team_for(h, (const void *)kern, work, g.n) + ((const void *)kern == (const void *)k_aff_down ? 1 : 0);
+  kern<<<grid, 32 * warps, smem, st>>>(args...);
   if (timed) {
     cudaEventRecord(h->ev[h->nev + 1], st);
     h->nev += 2;

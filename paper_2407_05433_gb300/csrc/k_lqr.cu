@@ -35,8 +35,9 @@ __host__ int smem_lqr_level(int n) {
 }
 __host__ int smem_riccati_finish(int n, int m) { return std::max(m * (n + m + 1) + m * (n + 1) + m + 8, n * n); }
 __host__ int smem_aff(int n, int m) { return 2 * (n * n + n) + n * n + 5 * n + 2 * m + 8; }
-constexpr int kAffRing = 6;  // stages of k_aff_down in shared memory: one in use, five on their way
-__host__ int smem_aff_down(int n) { return kAffRing * n * (n + 1) + 2 * n; }
+constexpr int kAffRing = 6;  // stages of k_aff_down on their way to shared memory
+constexpr int kAffY = 32;    // its vectors, with room for whole segments
+__host__ int smem_aff_down(int n) { return kAffRing * n * (n + 1) + 2 * kAffY + 2; }
 
 // Cost-relation slot layout (ld 2n + 1): constraint rows at 0 (CI_ROWS of them),
 // cost rows at offset 2n (2n + 1) (CI_ROWS2 of them); CI_NA / CI_NB are the
@@ -1008,104 +1009,109 @@ __global__ void k_aff_level(Group g, int src, int d, int fwd, int per_task) {
 }
 
 // The chain of one chunk: y_out = G_i y_in + gv_i stage after stage, G_i = Phi_i
-// (ROLL, CROLL), Phi_i' (PLIN, backward) or Pnu_i (NU), gv_i from k_aff_prep (pnu
-// for NU).  Each output row is a dot product split over seg lanes, so its dependent
-// chain is about n / seg FMAs and log2(seg) shuffle additions, one barrier per stage
-// (y alternates between two buffers).
+// (ROLL, CROLL), Phi_i' (PLIN, backward) or Pnu_i (NU), gv_i from k_aff_prep, k_resid and k_pcorr
+// (pnu for NU).
 //
-// What bounds it: the latency of one stage, 64 cycles for each FP64 instruction of that
-// chain.  A stage's G and gv are one block of n (n + 1) doubles that does not depend on the
-// chain, so they are copied to shared memory kAffRing - 1 stages ahead: with the next stage
-// alone in flight (in registers) every stage waited for memory instead, 0.70 us a stage at
-// n = 4 and n = 16.  seg = 4 from n = 8 and 2 below; a wider split adds a shuffle and an
-// addition for the FMAs it saves, which pays from n = 24 on where the team has the lanes.
-template <int SEG>
-static __device__ __forceinline__ void aff_chain(const Group &g, const ProbInfo &P, int mode, int a, int b, int dcur,
-                                                 const double *sv) {
-  const int n = g.n, tid = team_rank(), lane = tid & 31;
-  const bool fwd = aff_forward(mode), tr = mode == AFF_PLIN;
-  const int off = aff_out(g, mode), blk = n * (n + 1), steps = b - a;
-  double *ya = g_smem + kAffRing * blk, *yb = ya + n;
-  const int q = tid & (SEG - 1), row = tid / SEG;  // this lane's row and column offset
-  // stages in the order of the sweep
+// What bounds it: the latency of one stage.  Of that only the FP64 chain of a row (n / SEG
+// multiply-adds and log2(SEG) shuffled additions of 64 cycles each) and the exchange of y are
+// needed; a warp issues in order, so everything else has to leave its way.  The last warp of the CTA
+// does it: it copies the blocks [G | gv] asynchronously kAffRing stages ahead into shared memory,
+// stores y and looks up the dimensions.  The others hold a row over SEG lanes, read the coming
+// stage's entries into registers while the FP64 instructions run, and meet it at one barrier per
+// stage.  Per stage, 256 problems of 256 stages at n = 16 and 64 stages at n = 4: 0.70 and 0.72 us with the
+// next stage's entries read one stage ahead by the same warps, 0.63 and 0.57 with the ring alone.
+template <int SEG, int KP>
+static __device__ __forceinline__ void aff_rows(const double *ring, double *ya, double *yb, const int *sdim, int n, bool tr,
+                                                int steps, int dcur) {
+  const int blk = n * (n + 1), q = threadIdx.x & (SEG - 1), row = threadIdx.x / SEG;
+  const int g0 = tr ? q * n + row : row * n + q, gs = tr ? SEG * n : SEG;
+  double gr[KP], gv = 0.0;
+  bool on = false;
+  // this lane's entries of block G, din x dout (zero outside)
+  auto load = [&](const double *G, int din, int dout) {
+    on = row < dout;
+    const double *e = G + g0;
+#pragma unroll
+    for (int j = 0; j < KP; j++, e += gs) gr[j] = on && q + j * SEG < din ? *e : 0.0;
+    gv = on && q == 0 ? G[n * n + row] : 0.0;
+  };
+  __syncthreads();
+  int dout = sdim[0], slot = 0;
+  load(ring, dcur, dout);
+  const double *G = ring;
+  for (int k = 0; k < steps; k++) {
+    double acc = gv;
+#pragma unroll
+    for (int j = 0; j < KP; j++)
+      if (j * SEG < n) acc = fma(gr[j], ya[q + j * SEG], acc);
+    const bool was = on;
+    G += blk;
+    if (++slot == kAffRing) {
+      slot = 0;
+      G = ring;
+    }
+    const int d1 = sdim[(k + 1) & 3];
+    load(G, dout, d1);
+    dout = d1;
+#pragma unroll
+    for (int s = SEG >> 1; s > 0; s >>= 1) acc += __shfl_xor_sync(kFull, acc, s);
+    if (q == 0 && row < n) yb[row] = was ? acc : 0.0;
+    double *t = ya; ya = yb; yb = t;
+    __syncthreads();
+  }
+}
+
+// the last warp of the CTA
+static __device__ __forceinline__ void aff_helper(const Group &g, const ProbInfo &P, int mode, int a, int b, double *ring,
+                                                  double *ya, double *yb, int *sdim) {
+  const int n = g.n, lane = threadIdx.x & 31, blk = n * (n + 1), steps = b - a;
+  const bool fwd = aff_forward(mode);
   const int first = P.st0 + (fwd ? a : b - 1), dir = fwd ? 1 : -1;
   const ptrdiff_t step = (ptrdiff_t)dir * g.ws.stride;
-  const double *src = stage_ws(g, first) + (mode == AFF_NU ? g.ws.Pnu : g.ws.Phi) + 2 * tid;
-  double *o = stage_ws(g, first) + off + tid;
+  const double *src = stage_ws(g, first) + (mode == AFF_NU ? g.ws.Pnu : g.ws.Phi) + 2 * lane;
+  // y_k belongs to stage a + k forwards, b - k backwards; stage b is the next chunk's unless it is the last
+  double *o = stage_ws(g, P.st0 + (fwd ? a : b)) + aff_out(g, mode) + lane;
   int sent = 0;
   auto fetch = [&](int slot) {
     if (sent < steps) {
-      double *dst = g_smem + slot * blk;
-      for (int i = 2 * tid; i < blk; i += 2 * TEAM) copy_async16(dst + i, src + (i - 2 * tid));
+      double *dst = ring + slot * blk + 2 * lane;
+#pragma unroll 4
+      for (int i = 2 * lane; i < blk; i += 64, dst += 64) copy_async16(dst, src + (i - 2 * lane));
       src += step;
       sent++;
     }
     copy_commit();
   };
 #pragma unroll
-  for (int k = 0; k < kAffRing - 1; k++) fetch(k);
+  for (int k = 0; k < kAffRing; k++) fetch(k);
   // output dimensions of the stages k0 .. k0 + 31, one per lane, and of the 32 after them
   auto dims = [&](int k0) {
     const int k = k0 + lane;
     return k < steps ? aff_dim(g, first + dir * k + (fwd ? 1 : 0), mode) : 0;
   };
   int dreg = dims(0), dnext = dims(32);
-  for (int i = tid; i < n; i += TEAM) {
-    const double v = sv && i < dcur ? sv[i] : 0.0;
-    ya[i] = v;
-    if (!fwd && b == P.N) stage_ws(g, P.st0 + b)[off + i] = v;
-  }
-  // this lane's first entry of a block, and the distance to the next ones
-  const int g0 = tr ? q * n + row : row * n + q, gs = tr ? SEG * n : SEG;
-  constexpr int KP = 4;
+  if (lane < 2) sdim[lane] = dreg;
+  copy_wait_ring<kAffRing - 2>();  // stages 0 and 1
+  __syncthreads();
   int slot = 0;
-  const double *G = g_smem;
   for (int k = 0; k < steps; k++) {
-    copy_wait_ring<kAffRing - 2>();  // this thread's share of stage k
-    if (blockDim.x == 32) __syncwarp();
-    else __syncthreads();  // every thread's; y of the stage before; its block is free
-    const int dout = __shfl_sync(kFull, dreg, k & 31);
-    const bool on = row < dout;
-    // batches of KP entries and y's: the loads of a batch are in flight together
-    double acc = on && q == 0 ? G[n * n + row] : 0.0;
-    const double *Gr = G + g0, *yq = ya + q;
-    for (int l = q; l - q < dcur; l += KP * SEG, Gr += KP * gs, yq += KP * SEG) {
-      double gr[KP], yr[KP];
-#pragma unroll
-      for (int j = 0; j < KP; j++) {
-        const bool in = on && l + j * SEG < dcur;
-        gr[j] = in ? Gr[j * gs] : 0.0;
-        yr[j] = in ? yq[j * SEG] : 0.0;
-      }
-#pragma unroll
-      for (int j = 0; j < KP; j++)
-        if (l - q + j * SEG < dcur) acc = fma(gr[j], yr[j], acc);
-    }
-    fetch(slot == 0 ? kAffRing - 1 : slot - 1);
-    if (fwd && tid < n) *o = tid < dcur ? ya[tid] : 0.0;  // the value of the stage is the chain's input
-#pragma unroll
-    for (int s = SEG >> 1; s > 0; s >>= 1) acc += __shfl_xor_sync(kFull, acc, s);
-    if (q == 0 && row < n) {
-      yb[row] = acc;
-      if (!fwd) o[row - tid] = acc;  // the chain's output is the value of the stage
-    }
-    if ((k & 31) == 31) {
-      dreg = dnext;
-      dnext = dims(k + 33);
-    }
+    if (lane < n && (fwd || k > 0 || b == P.N)) *o = ya[lane];
     o += step;
-    double *tmp = ya; ya = yb; yb = tmp;
-    dcur = dout;
-    G += blk;
-    if (++slot == kAffRing) {
-      slot = 0;
-      G = g_smem;
+    if (k > 0) {  // into the block of stage k - 1, whose entries went to registers before this barrier
+      fetch(slot);
+      if (++slot == kAffRing) slot = 0;
     }
+    if (((k + 2) & 31) == 0) {
+      dreg = dnext;
+      dnext = dims(k + 34);
+    }
+    const int d = __shfl_sync(kFull, dreg, (k + 2) & 31);
+    if (lane == 0) sdim[(k + 2) & 3] = d;
+    copy_wait_ring<kAffRing - 3>();  // stage k + 2
+    double *t = ya; ya = yb; yb = t;
+    __syncthreads();
   }
-  if (fwd && b == P.N) {
-    tsync();
-    if (tid < n) *o = tid < dcur ? ya[tid] : 0.0;
-  }
+  if (lane < n && (!fwd || b == P.N)) *o = ya[lane];
 }
 
 __global__ void k_aff_down(Group g, int mode, int fin, int /*per_task*/) {
@@ -1115,8 +1121,10 @@ __global__ void k_aff_down(Group g, int mode, int fin, int /*per_task*/) {
   const ProbInfo &P = g.prob[ci.prob];
   if (skipped_by_mask(g, ci.prob)) return;
   if (ci.c >= P.nch) return;
-  const int n = g.n, a = ci.c * P.L, b = min(a + P.L, P.N);
-  const bool fwd = aff_forward(mode);
+  const int n = g.n, a = ci.c * P.L, b = min(a + P.L, P.N), steps = b - a;
+  const bool fwd = aff_forward(mode), tr = mode == AFF_PLIN;
+  double *ring = g_smem, *ya = ring + kAffRing * n * (n + 1), *yb = ya + kAffY;
+  int *sdim = (int *)(yb + kAffY);
   // boundary value: with one chunk the problem's own (z_0, 0, rq_N or nu_0); after the scan the
   // forward slot (ch0 + c) = y_a, the backward slot (ch0 + c + 1) = y_b
   const int slot = fwd ? P.ch0 + ci.c : P.ch0 + ci.c + 1;
@@ -1124,12 +1132,24 @@ __global__ void k_aff_down(Group g, int mode, int fin, int /*per_task*/) {
   const double *sv = P.nch > 1 ? g.CS[fin] + (size_t)slot * g.cs_stride + n * n
                                : mode == AFF_CROLL ? nullptr
                                                    : end + (mode == AFF_ROLL ? g.ws.z : mode == AFF_PLIN ? g.ws.rq : g.ws.nu);
-  const int d0 = aff_dim(g, P.st0 + (fwd ? a : b), mode);
-  const int lanes = TEAM / n;
-  if (n >= 24 && lanes >= 8) aff_chain<8>(g, P, mode, a, b, d0, sv);
-  else if (n >= 8 && lanes >= 4) aff_chain<4>(g, P, mode, a, b, d0, sv);
-  else if (lanes >= 2) aff_chain<2>(g, P, mode, a, b, d0, sv);
-  else aff_chain<1>(g, P, mode, a, b, d0, sv);
+  const int d0 = aff_dim(g, P.st0 + (fwd ? a : b), mode), lanes = TEAM - 32;
+  if (threadIdx.x >= lanes) {
+    const int lane = threadIdx.x & 31;
+    // y_0, and zeros beyond the dimensions of either buffer
+    ya[lane] = sv && lane < d0 ? sv[lane] : 0.0;
+    yb[lane] = 0.0;
+    __syncwarp();
+    aff_helper(g, P, mode, a, b, ring, ya, yb, sdim);
+    return;
+  }
+  // a row over four lanes (two below n = 5), over fewer where the team has not as many
+  if (n <= 4) aff_rows<2, 2>(ring, ya, yb, sdim, n, tr, steps, d0);
+  else if (n <= 8) aff_rows<4, 2>(ring, ya, yb, sdim, n, tr, steps, d0);
+  else if (4 * n > lanes && 2 * n <= lanes && n <= 16) aff_rows<2, 8>(ring, ya, yb, sdim, n, tr, steps, d0);
+  else if (4 * n > lanes && 2 * n <= lanes) aff_rows<2, 16>(ring, ya, yb, sdim, n, tr, steps, d0);
+  else if (4 * n > lanes) aff_rows<1, 32>(ring, ya, yb, sdim, n, tr, steps, d0);
+  else if (n <= 16) aff_rows<4, 4>(ring, ya, yb, sdim, n, tr, steps, d0);
+  else aff_rows<4, 8>(ring, ya, yb, sdim, n, tr, steps, d0);
 }
 
 // ----------------------------------------------------------- stage-parallel helpers of the solve
