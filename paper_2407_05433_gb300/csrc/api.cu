@@ -117,7 +117,7 @@ namespace {
 int team_for(const eclqr_handle *h, const void *kern, int ntasks, int n) {
   if (h->opt.team_warps != 0) return h->opt.team_warps;
   // four lanes a row of an affine chain (two below n = 5), and never more than a row's latency pays for
-  if (kern == (const void *)k_aff_down) return n <= 8 ? 1 : n <= 16 ? 2 : 4;
+  if (kern == (const void *)k_aff_down || kern == (const void *)k_aff_up_again) return n <= 8 ? 1 : n <= 16 ? 2 : 4;
   if (kern == (const void *)k_riccati_down && ntasks < kManyTasksPerSm * h->sms) {
     // up to two sweeps per SM: the products of a stage spread over more warps
     return ntasks > 2 * h->sms || n < 12 ? kTeamWarps : n < 24 ? 8 : 16;
@@ -183,8 +183,9 @@ int launch_grid(eclqr_handle *h, void (*kern)(KArgs...), int ntasks, int grid, i
   const Group &g = group_of(args...);
   // every problem has one slot more than it has chunks to sweep
   const int work = (const void *)kern == (const void *)k_riccati_down ? g.nslot - g.nprob : ntasks;
-  // k_aff_down has one warp more than its rows take
-  const int warps = team_for(h, (const void *)kern, work, g.n) + ((const void *)kern == (const void *)k_aff_down ? 1 : 0);
+  // the affine chains have one warp more than their rows take
+  const bool chain = (const void *)kern == (const void *)k_aff_down || (const void *)kern == (const void *)k_aff_up_again;
+  const int warps = team_for(h, (const void *)kern, work, g.n) + (chain ? 1 : 0);
   kern<<<grid, 32 * warps, smem, st>>>(args...);
   if (timed) {
     cudaEventRecord(h->ev[h->nev + 1], st);
@@ -472,7 +473,7 @@ int eclqr_create(const eclqr_desc *d, const eclqr_options *opt, eclqr_handle **o
           {(const void *)k_lqr_up, smem_lqr_up(n, m)}, {(const void *)k_lqr_level, smem_lqr_level(n)},
           {(const void *)k_riccati_down, smem_riccati(n, m)},
           {(const void *)k_riccati_finish, smem_riccati_finish(n, m)}, {(const void *)k_aff_up, sa},
-          {(const void *)k_aff_level, sa}, {(const void *)k_aff_down, smem_aff_down(n)}, {(const void *)k_resid, 4 * n + 2 * m},
+          {(const void *)k_aff_level, sa}, {(const void *)k_aff_down, smem_aff_down(n)}, {(const void *)k_aff_up_again, smem_aff_down(n)}, {(const void *)k_resid, 4 * n + 2 * m},
           {(const void *)k_pcorr, n + m + m * m}, {(const void *)k_dual_stage, smem_dual_stage(n, m)},
           {(const void *)k_dual_terminal, sdw}, {(const void *)k_dual_up, sdw}, {(const void *)k_dual_down, sdw + kHeldScratch},
           {(const void *)k_dual_root, sdw + kHeldScratch}, {(const void *)k_dual_leaf, smem_dual_leaf(n, m, wmax) + kHeldScratch}};
@@ -557,7 +558,7 @@ int eclqr_create(const eclqr_desc *d, const eclqr_options *opt, eclqr_handle **o
     gh.levels = gh.maxnch == 1 ? 0 : ilog2ceil(gh.maxnch + 1);
     g.ws = make_ws_layout(g.n, g.m, pmax, qmax);
     g.cs_stride = ((8 * g.n * g.n + 4 * g.n) + 3) & ~3;  // cost relations: 2n constraint + 2n cost rows
-    g.cr_stride = 0;
+    g.cr_stride = gh.levels > 0 ? g.n * g.n : 0;
     g.tau_rank = h->opt.tau_rank;
     g.tau_inc = h->opt.tau_inc;
     // one allocation: descriptors, stage workspace, chunk slots
@@ -569,6 +570,7 @@ int eclqr_create(const eclqr_desc *d, const eclqr_options *opt, eclqr_handle **o
     size_t o_WI = take(sizeof(int) * (size_t)SI_STRIDE * g.nstage);
     size_t o_CS0 = take(sizeof(double) * (size_t)g.cs_stride * g.nslot);
     size_t o_CS1 = take(sizeof(double) * (size_t)g.cs_stride * g.nslot);
+    size_t o_CR = take(sizeof(double) * (size_t)g.cr_stride * g.nslot);
     size_t o_CI0 = take(sizeof(int) * CI_STRIDE * g.nslot), o_CI1 = take(sizeof(int) * CI_STRIDE * g.nslot);
     size_t o_need = take(sizeof(int) * (size_t)g.nprob), o_queue = take(sizeof(int));
     size_t o_sl = take(sizeof(int) * 3 * (size_t)g.nstage), o_sc = take(sizeof(int) * 3);
@@ -593,6 +595,7 @@ int eclqr_create(const eclqr_desc *d, const eclqr_options *opt, eclqr_handle **o
     g.WI = (int *)(base + o_WI);
     g.CS[0] = (double *)(base + o_CS0);
     g.CS[1] = (double *)(base + o_CS1);
+    g.CR = (double *)(base + o_CR);
     g.CI[0] = (int *)(base + o_CI0);
     g.CI[1] = (int *)(base + o_CI1);
     g.need_scan = (int *)(base + o_need);
@@ -709,12 +712,15 @@ int aff_scan(eclqr_handle *h, const GroupHost &gh, const Group &g, int mode, cud
   const int sa = smem_aff(g.n, g.m);
   const int fwd = (mode == AFF_PLIN_) ? 0 : 1;
   if (mode == AFF_ROLL_) TRY(launch(h, k_aff_prep, g.nstage, 0, st, g));
-  if (gh.levels > 0) TRY(launch(h, k_aff_up, g.nslot, sa, st, g, mode, sa));
+  const int sd = smem_aff_down(g.n);
+  if (gh.levels > 0) {
+    if (mode == AFF_CROLL_ || mode == AFF_PLIN_) TRY(launch(h, k_aff_up_again, g.nslot, sd, st, g, mode, sd));
+    else TRY(launch(h, k_aff_up, g.nslot, sa, st, g, mode, sa));
+  }
   int src = 0;
   // radix-4 levels: strides 1, 4, 16, ... until they cover every slot
   for (int d = 1; gh.levels > 0 && d < gh.maxnch + 1; d *= 4, src ^= 1)
     TRY(launch(h, k_aff_level, g.nslot, sa, st, g, src, d, fwd, sa));
-  const int sd = smem_aff_down(g.n);
   TRY(launch(h, k_aff_down, g.nslot, sd, st, g, mode, src, sd));
   return ECLQR_OK;
 }
@@ -1166,7 +1172,7 @@ int eclqr_time_kernel(eclqr_handle *h, const char *name) {
       {"k_param", (const void *)k_param}, {"k_elim", (const void *)k_elim},
       {"k_lqr_up", (const void *)k_lqr_up}, {"k_lqr_level", (const void *)k_lqr_level},
       {"k_riccati_down", (const void *)k_riccati_down}, {"k_riccati_finish", (const void *)k_riccati_finish},
-      {"k_aff_up", (const void *)k_aff_up},
+      {"k_aff_up", (const void *)k_aff_up}, {"k_aff_up_again", (const void *)k_aff_up_again},
       {"k_aff_level", (const void *)k_aff_level}, {"k_aff_down", (const void *)k_aff_down},
       {"k_aff_prep", (const void *)k_aff_prep},
       {"k_solve_init", (const void *)k_solve_init}, {"k_post_roll", (const void *)k_post_roll},

@@ -856,23 +856,16 @@ __global__ void k_aff_prep(Group g) {
   });
 }
 
-// chunk aggregates; also the boundary value slot (forward: slot 0 of the
-// problem holds y_0, backward: slot nch holds y_N).
-__global__ void k_aff_up(Group g, int mode, int per_task) {
-  const int t = team_task();
-  if (t >= g.nslot) return;
-  const ChunkInfo ci = g.chunk[t];
-  const ProbInfo &P = g.prob[ci.prob];
-  if (skipped_by_mask(g, ci.prob)) return;
+// What the chunk aggregates' kernels have to do besides aggregates: the boundary value's slot (forward:
+// slot 0 of the problem holds y_0, backward: slot nch holds y_N), and an empty map where one chunk
+// needs none.  Returns whether that was the task.
+static __device__ bool aff_up_ends(const Group &g, const ChunkInfo ci, const ProbInfo &P, int mode, bool fwd) {
   const int n = g.n, tid = team_rank();
-  const bool fwd = aff_forward(mode);
-  double *cs0 = g.CS[0];
   if (ci.c == P.nch) {
-    // boundary value
     const int s = fwd ? P.st0 : P.st0 + P.N;
     const int slot = fwd ? P.ch0 : P.ch0 + P.nch;
     const int dim = aff_dim(g, s, mode);
-    double *gv = cs0 + (size_t)slot * g.cs_stride + n * n;
+    double *gv = g.CS[0] + (size_t)slot * g.cs_stride + n * n;
     const double *src = stage_ws(g, s);
     for (int i = tid; i < dim; i += TEAM) {
       double v;
@@ -886,18 +879,29 @@ __global__ void k_aff_up(Group g, int mode, int per_task) {
       int *cm = g.CI[0] + (size_t)slot * CI_STRIDE;
       cm[CI_ROWS] = 1; cm[CI_NA] = dim; cm[CI_NB] = 0;
     }
-    return;
+    return true;
   }
+  if (P.nch > 1) return false;
+  // one chunk: k_aff_down starts from the boundary value, so the chunk's map is not
+  // composed; an empty map (no rows, no dimensions) ends the level at once
+  if (tid == 0) {
+    int *cm = g.CI[0] + (size_t)(fwd ? P.ch0 + ci.c + 1 : P.ch0 + ci.c) * CI_STRIDE;
+    cm[CI_ROWS] = 0; cm[CI_NA] = 0; cm[CI_NB] = 0;
+  }
+  return true;
+}
+
+// chunk aggregates
+__global__ void k_aff_up(Group g, int mode, int per_task) {
+  const int t = team_task();
+  if (t >= g.nslot) return;
+  const ChunkInfo ci = g.chunk[t];
+  const ProbInfo &P = g.prob[ci.prob];
+  if (skipped_by_mask(g, ci.prob)) return;
+  const int n = g.n, tid = team_rank();
+  const bool fwd = aff_forward(mode);
+  if (aff_up_ends(g, ci, P, mode, fwd)) return;
   const int slot = fwd ? P.ch0 + ci.c + 1 : P.ch0 + ci.c;
-  if (P.nch == 1) {
-    // one chunk: k_aff_down starts from the boundary value, so the chunk's map is not
-    // composed; an empty map (no rows, no dimensions) ends the level at once
-    if (tid == 0) {
-      int *cm = g.CI[0] + (size_t)slot * CI_STRIDE;
-      cm[CI_ROWS] = 0; cm[CI_NA] = 0; cm[CI_NB] = 0;
-    }
-    return;
-  }
   const int a = ci.c * P.L, b = min(a + P.L, P.N);
   double *sm = team_smem(per_task);
   double *Gm = sm, *gm = Gm + n * n, *Gs = gm + n, *gs = Gs + n * n, *Tm = gs + n, *tmp = Tm + n * n;
@@ -930,8 +934,10 @@ __global__ void k_aff_up(Group g, int mode, int per_task) {
     tsync();
     dcur = dout;
   }
-  double *cs = cs0 + (size_t)slot * g.cs_stride;
+  double *cs = g.CS[0] + (size_t)slot * g.cs_stride;
   for (int idx = tid; idx < n * n; idx += TEAM) cs[idx] = Gm[idx];
+  if (mode == AFF_ROLL)
+    for (int idx = tid; idx < n * n; idx += TEAM) g.CR[(size_t)t * g.cr_stride + idx] = Gm[idx];
   for (int i = tid; i < n; i += TEAM) cs[n * n + i] = gm[i];
   if (tid == 0) {
     int *cm = g.CI[0] + (size_t)slot * CI_STRIDE;
@@ -1061,9 +1067,9 @@ static __device__ __forceinline__ void aff_rows(const double *ring, double *ya, 
   }
 }
 
-// the last warp of the CTA
+// The last warp of the CTA.  end: where the chain's last value goes, instead of the stages' values.
 static __device__ __forceinline__ void aff_helper(const Group &g, const ProbInfo &P, int mode, int a, int b, double *ring,
-                                                  double *ya, double *yb, int *sdim) {
+                                                  double *ya, double *yb, int *sdim, double *end) {
   const int n = g.n, lane = threadIdx.x & 31, blk = n * (n + 1), steps = b - a;
   const bool fwd = aff_forward(mode);
   const int first = P.st0 + (fwd ? a : b - 1), dir = fwd ? 1 : -1;
@@ -1095,7 +1101,7 @@ static __device__ __forceinline__ void aff_helper(const Group &g, const ProbInfo
   __syncthreads();
   int slot = 0;
   for (int k = 0; k < steps; k++) {
-    if (lane < n && (fwd || k > 0 || b == P.N)) *o = ya[lane];
+    if (!end && lane < n && (fwd || k > 0 || b == P.N)) *o = ya[lane];
     o += step;
     if (k > 0) {  // into the block of stage k - 1, whose entries went to registers before this barrier
       fetch(slot);
@@ -1111,35 +1117,24 @@ static __device__ __forceinline__ void aff_helper(const Group &g, const ProbInfo
     double *t = ya; ya = yb; yb = t;
     __syncthreads();
   }
-  if (lane < n && (!fwd || b == P.N)) *o = ya[lane];
+  if (end) o = end + lane;
+  if (lane < n && (end || !fwd || b == P.N)) *o = ya[lane];
 }
 
-__global__ void k_aff_down(Group g, int mode, int fin, int /*per_task*/) {
-  const int t = team_task();
-  if (t >= g.nslot) return;
-  const ChunkInfo ci = g.chunk[t];
-  const ProbInfo &P = g.prob[ci.prob];
-  if (skipped_by_mask(g, ci.prob)) return;
-  if (ci.c >= P.nch) return;
-  const int n = g.n, a = ci.c * P.L, b = min(a + P.L, P.N), steps = b - a;
-  const bool fwd = aff_forward(mode), tr = mode == AFF_PLIN;
+// The chain over the stages [a, b) from the value sv (null: zero) of dimension d0.
+static __device__ __forceinline__ void aff_sweep(const Group &g, const ProbInfo &P, int mode, int a, int b, int d0,
+                                                 const double *sv, double *end) {
+  const int n = g.n, steps = b - a, lanes = TEAM - 32;
+  const bool tr = mode == AFF_PLIN;
   double *ring = g_smem, *ya = ring + kAffRing * n * (n + 1), *yb = ya + kAffY;
   int *sdim = (int *)(yb + kAffY);
-  // boundary value: with one chunk the problem's own (z_0, 0, rq_N or nu_0); after the scan the
-  // forward slot (ch0 + c) = y_a, the backward slot (ch0 + c + 1) = y_b
-  const int slot = fwd ? P.ch0 + ci.c : P.ch0 + ci.c + 1;
-  const double *end = stage_ws(g, fwd ? P.st0 : P.st0 + P.N);
-  const double *sv = P.nch > 1 ? g.CS[fin] + (size_t)slot * g.cs_stride + n * n
-                               : mode == AFF_CROLL ? nullptr
-                                                   : end + (mode == AFF_ROLL ? g.ws.z : mode == AFF_PLIN ? g.ws.rq : g.ws.nu);
-  const int d0 = aff_dim(g, P.st0 + (fwd ? a : b), mode), lanes = TEAM - 32;
   if (threadIdx.x >= lanes) {
     const int lane = threadIdx.x & 31;
     // y_0, and zeros beyond the dimensions of either buffer
     ya[lane] = sv && lane < d0 ? sv[lane] : 0.0;
     yb[lane] = 0.0;
     __syncwarp();
-    aff_helper(g, P, mode, a, b, ring, ya, yb, sdim);
+    aff_helper(g, P, mode, a, b, ring, ya, yb, sdim, end);
     return;
   }
   // a row over four lanes (two below n = 5), over fewer where the team has not as many
@@ -1150,6 +1145,53 @@ __global__ void k_aff_down(Group g, int mode, int fin, int /*per_task*/) {
   else if (4 * n > lanes) aff_rows<1, 32>(ring, ya, yb, sdim, n, tr, steps, d0);
   else if (n <= 16) aff_rows<4, 4>(ring, ya, yb, sdim, n, tr, steps, d0);
   else aff_rows<4, 8>(ring, ya, yb, sdim, n, tr, steps, d0);
+}
+
+__global__ void k_aff_down(Group g, int mode, int fin, int /*per_task*/) {
+  const int t = team_task();
+  if (t >= g.nslot) return;
+  const ChunkInfo ci = g.chunk[t];
+  const ProbInfo &P = g.prob[ci.prob];
+  if (skipped_by_mask(g, ci.prob)) return;
+  if (ci.c >= P.nch) return;
+  const int n = g.n, a = ci.c * P.L, b = min(a + P.L, P.N);
+  const bool fwd = aff_forward(mode);
+  // boundary value: with one chunk the problem's own (z_0, 0, rq_N or nu_0); after the scan the
+  // forward slot (ch0 + c) = y_a, the backward slot (ch0 + c + 1) = y_b
+  const int slot = fwd ? P.ch0 + ci.c : P.ch0 + ci.c + 1;
+  const double *end = stage_ws(g, fwd ? P.st0 : P.st0 + P.N);
+  const double *sv = P.nch > 1 ? g.CS[fin] + (size_t)slot * g.cs_stride + n * n
+                               : mode == AFF_CROLL ? nullptr
+                                                   : end + (mode == AFF_ROLL ? g.ws.z : mode == AFF_PLIN ? g.ws.rq : g.ws.nu);
+  aff_sweep(g, P, mode, a, b, aff_dim(g, P.st0 + (fwd ? a : b), mode), sv, nullptr);
+}
+
+// The chunk aggregates of the refinement's chains (CROLL, PLIN), in the place of k_aff_up: their
+// matrices are the rollout's product of the same Phi's (CROLL) and its transpose (PLIN), which the
+// solve's k_aff_up kept in CR, so that a chunk is one chain of its offsets from zero, n^2 a stage
+// instead of n^3 (16384 stages at n = 16: 191 us a launch with the products).
+__global__ void k_aff_up_again(Group g, int mode, int /*per_task*/) {
+  const int t = team_task();
+  if (t >= g.nslot) return;
+  const ChunkInfo ci = g.chunk[t];
+  const ProbInfo &P = g.prob[ci.prob];
+  if (skipped_by_mask(g, ci.prob)) return;
+  const bool fwd = aff_forward(mode);
+  if (aff_up_ends(g, ci, P, mode, fwd)) return;
+  const int n = g.n, a = ci.c * P.L, b = min(a + P.L, P.N);
+  const int slot = fwd ? P.ch0 + ci.c + 1 : P.ch0 + ci.c;
+  const int da = aff_dim(g, P.st0 + a, mode), db = aff_dim(g, P.st0 + b, mode);
+  double *cs = g.CS[0] + (size_t)slot * g.cs_stride;
+  const double *F = g.CR + (size_t)t * g.cr_stride;
+  for (int idx = team_rank(); idx < n * n; idx += TEAM) {
+    const int i = idx / n, j = idx - i * n;
+    cs[idx] = fwd ? F[idx] : F[j * n + i];
+  }
+  if (team_rank() == 0) {
+    int *cm = g.CI[0] + (size_t)slot * CI_STRIDE;
+    cm[CI_ROWS] = 0; cm[CI_NA] = fwd ? da : db; cm[CI_NB] = fwd ? db : da;
+  }
+  aff_sweep(g, P, mode, a, b, 0, nullptr, cs + n * n);
 }
 
 // ----------------------------------------------------------- stage-parallel helpers of the solve

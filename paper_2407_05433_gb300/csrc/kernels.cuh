@@ -41,6 +41,7 @@ __global__ void k_riccati_down(Group g, int fin, int per_task, int *queue);
 __global__ void k_riccati_finish(Group g, int per_task);
 __global__ void k_riccati_down_f32(Group g, int fin, int per_task);  // k_mixed.cu
 __global__ void k_aff_up(Group g, int mode, int per_task);
+__global__ void k_aff_up_again(Group g, int mode, int per_task);
 __global__ void k_aff_level(Group g, int src, int d, int fwd, int per_task);
 __global__ void k_aff_down(Group g, int mode, int fin, int per_task);
 __global__ void k_aff_prep(Group g);

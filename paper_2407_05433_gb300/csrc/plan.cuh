@@ -127,7 +127,7 @@ struct Group {
   double *CS[2];  // nslot * cs_stride
   int *CI[2];     // nslot * CI_STRIDE
   int cs_stride;
-  double *CR;     // nslot * cr_stride: per-slot scan results kept across kernels
+  double *CR;     // nslot * cr_stride: the rollout's chunk products, kept for the solve's other chains
   int cr_stride;
   int *status;    // batch-global, indexed by ProbInfo::id
   int *need_scan; // per problem: 1 once a stage leaves rows on x_i (set by k_scan_check)
