@@ -513,13 +513,14 @@ int eclqr_create(const eclqr_desc *d, const eclqr_options *opt, eclqr_handle **o
       if (L <= 0 && one_chunk) {
         L = std::max(1, pi.N);
       } else if (L <= 0) {
-        // about three chunks per SM (16384 stages at n = 16: 17.5 ms with 40-stage chunks, 20.3 with
-        // two chunks of 54 per SM, 22.1 with nine of 12), but never shorter than 7 stages: shorter
+        // three chunks per SM, and none more, which a few SMs would take as a fourth (16384 stages at
+        // n = 16: 14.3 ms with 456 chunks of 36 stages, 15.2 with 469 of 35, 14.8 with four of 27 per SM,
+        // 17.1 with two of 54), but never shorter than 7 stages: shorter
         // chunks place more boundaries, and where a boundary meets an ill-conditioned
         // stage the refinement needs more than its default passes (on the degenerate
         // n = 12 instance 6-stage chunks miss the 1e-9 gate after two).  A 1024-stage
         // problem then runs as 147 chunks, one CTA each, on a 152-SM GB300.
-        long long target = std::max<long long>(1, total_stages / (3LL * sms));
+        long long target = (total_stages + 3LL * sms - 1) / (3LL * sms);
         L = (int)std::min<long long>(64, std::max<long long>(7, target));
         L = std::max(1, std::min(L, pi.N));
       }
