@@ -168,10 +168,10 @@ __device__ __forceinline__ double seg_sum(double acc, int sg, int S) {
 
 // Reflector of a column x with squared norm d = ||x||^2 and pivot entry x_k:
 // nrm = sqrt(d), shift = sign(x_k) nrm (sign(0) = +1, also for -0),
-// v_k = x_k + shift and beta = 2 / ||v||^2 = 1 / (nrm (nrm + |x_k|)), all in integers (fx.cuh): with
-// m = d 2^(-2 h) in [1, 4), N = sqrt(m) and X = |x_k| 2^-h as integers of 60 fractional bits,
-// V = N + X is |v_k| and 1 / (N V) is beta, each within 2^-55 of its value before the rounding to
-// FP64.  In FP64, from single-precision seeds and one third-order step each, the same scalars are
+// v_k = x_k + shift and beta = 2 / ||v||^2, all in integers (fx.cuh): with m = d 2^(-2 h) in [1, 4),
+// N = sqrt(m) and X = |x_k| 2^-h as integers of 60 fractional bits, V = N + X is |v_k| and N V half
+// of ||v||^2, corrected for v_k's rounding to FP64, so that H = I - beta v v' is orthogonal to rounding
+// for the v that is used; each is within 2^-55 of its value before its own rounding.  In FP64, from single-precision seeds and one third-order step each, the same scalars are
 // eleven dependent instructions in every warp of the team, most of a short step (n = 12, 147 chunks:
 // k_dual_down 787 us).  Branch-free; false, with the outputs unset, when d is zero, subnormal, above
 // 2^1000 or not finite.
@@ -191,7 +191,10 @@ __device__ __forceinline__ bool hh_reflector(double d, double xk, double &nrm, d
   nrm = fx_to((long long)N, h - 60);
   shift = neg ? -nrm : nrm;
   vk = fx_to(neg ? -(long long)V : (long long)V, h - 60);
-  const unsigned long long q = __umul64hi(N << 2, V << 1);  // N V 2^-61
+  // ||v||^2 / 2 of the v formed: with v_k = V + dv after its rounding, N V + V dv
+  const int zs = 11 - __clzll((long long)V);
+  const unsigned long long dv = (((V >> (zs - 1)) + 1) >> 1 << zs) - V;
+  const unsigned long long q = __umul64hi((N + dv) << 2, V << 1);  // N V 2^-61
   const int z = __clzll((long long)q);
   beta = fx_to(fx_rcp(q << z), z - 2 * h - 60);  // N V 2^(2 h - 120) = (q 2^z 2^-64) 2^(2 h + 5 - z)
   return ok;

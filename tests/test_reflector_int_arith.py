@@ -61,8 +61,10 @@ def _reflector(d, xk, e1, e2):
     sig, expo = ((b & 0xfffffffffffff) | 1 << 52, ex - 1022) if ex else (0, -100000)
     sh = min(expo - 53 - h + 60, 9)
     V = N + (sig << sh if sh >= 0 else (sig >> -sh if sh > -63 else 0))
-    q = _hi(N << 2, V << 1)
-    assert max(N << 2, V << 1) <= M64 and q > 0
+    zs = 11 - (64 - V.bit_length())
+    dv = (((V >> (zs - 1)) + 1) >> 1 << zs) - V
+    q = _hi((N + dv) << 2, V << 1)
+    assert max((N + dv) << 2, V << 1) <= M64 and q > 0 and 2 <= zs <= 10
     z = 64 - q.bit_length()
     neg = math.copysign(1.0, xk) < 0 and xk != 0
     nrm = _to(N, h - 60)
@@ -97,8 +99,10 @@ def test_scalars_are_rounded_values(sign):
         assert shift == (-nrm if xk < 0 else nrm)
         v = root + abs(Decimal(xk))
         assert abs(abs(Decimal(vk)) / v - 1) <= half * 2 and (vk < 0) == (xk < 0)
-        # 2^-54 of the reciprocal's last bit and the truncated product, and the rounding
-        assert abs(Decimal(beta) * root * v - 1) <= half * 2 + Decimal(2) ** -54, (d, xk)
+        # beta ||v||^2 = 2 for the v formed: 2^-54 of the reciprocal's last bit and the truncated product,
+        # and the rounding
+        v2 = Decimal(d) - Decimal(xk) ** 2 + Decimal(vk) ** 2
+        assert abs(Decimal(beta) * v2 / 2 - 1) <= half * 2 + Decimal(2) ** -54, (d, xk)
         s, h, _ = _even(d)
         assert abs(Decimal(_to(_rsqrt(s, e1), -62 - h)) * root - 1) <= half * 2
 
