@@ -132,7 +132,7 @@ int team_for(const eclqr_handle *h, const void *kern, int ntasks, int n) {
       {(const void *)k_dual_down, 1},            {(const void *)k_primal_stage, 1, 0, 24, 2},
       {(const void *)k_dual_leaf, 1},
       {(const void *)k_aff_prep, 1},             {(const void *)k_stage_lists, 1},
-      {(const void *)k_dual_stage, 2},           {(const void *)k_param, 1},
+      {(const void *)k_dual_stage, 1, 0, 24, 2},         {(const void *)k_param, 1},
       {(const void *)k_resid, 1},                {(const void *)k_pcorr, 1},
       {(const void *)k_kkt, 1},                  {(const void *)k_post_roll, 1},
       {(const void *)k_recover, 1},              {(const void *)k_check_inputs, 1},
@@ -473,7 +473,7 @@ int eclqr_create(const eclqr_desc *d, const eclqr_options *opt, eclqr_handle **o
           {(const void *)k_lqr_up, smem_lqr_up(n, m)}, {(const void *)k_lqr_level, smem_lqr_level(n)},
           {(const void *)k_riccati_down, smem_riccati(n, m)},
           {(const void *)k_riccati_finish, smem_riccati_finish(n, m)}, {(const void *)k_aff_up, sa},
-          {(const void *)k_aff_level, sa}, {(const void *)k_aff_down, smem_aff_down(n)}, {(const void *)k_aff_up_again, smem_aff_down(n)}, {(const void *)k_resid, 4 * n + 2 * m},
+          {(const void *)k_aff_level, sa}, {(const void *)k_aff_down, smem_aff_down(n)}, {(const void *)k_aff_up_again, smem_aff_down(n)}, {(const void *)k_resid, 5 * n + 3 * m},
           {(const void *)k_pcorr, n + m + m * m}, {(const void *)k_dual_stage, smem_dual_stage(n, m)},
           {(const void *)k_dual_terminal, sdw}, {(const void *)k_dual_up, sdw}, {(const void *)k_dual_down, sdw + kHeldScratch},
           {(const void *)k_dual_root, sdw + kHeldScratch}, {(const void *)k_dual_leaf, smem_dual_leaf(n, m, wmax) + kHeldScratch}};
@@ -733,7 +733,7 @@ int run_solve(eclqr_handle *h, const GroupHost &gh, const Group &g, cudaStream_t
   TRY(aff_scan(h, gh, g, AFF_ROLL_, gst));
   TRY(launch(h, k_post_roll, g.nstage, 0, gst, g, 0));
   for (int r = 0; r < refine_passes; r++) {
-    const int sres = 4 * g.n + 2 * g.m;
+    const int sres = 5 * g.n + 3 * g.m;
     TRY(launch(h, k_resid, g.nstage, sres, gst, g, sres));
     TRY(aff_scan(h, gh, g, AFF_PLIN_, gst));
     const int sc = g.n + g.m + g.m * g.m;

@@ -84,40 +84,38 @@ __global__ void __launch_bounds__(256, 3) k_dual_stage(Group g, const double *x,
     }
     const double *A = g.A + P.oA + (size_t)i * n * n, *B = g.B + P.oB + (size_t)i * n * m;
     const double *Mm = g.M + P.oM + (size_t)i * n * m, *R = g.R + P.oR + (size_t)i * m * m;
-    const double *r = g.rv + P.orv + (size_t)i * m, *ui = u + P.ou + (size_t)i * m;
+    const double *rv = g.rv + P.orv + (size_t)i * m, *ui = u + P.ou + (size_t)i * m;
     const double *wn = stage_ws(g, s + 1);
     const int *win = stage_wi(g, s + 1);
     const int r1 = win[SI_UR], nb1 = n - r1;
     const double *U1 = wn + g.ws.UT, *T1 = wn + g.ws.UT + r1, *pi1 = wn + g.ws.pi;
     // objective gradients (eq. objective-gradients) and T_{i+1} pi_{i+1}
     const bool tne = win[SI_TEYE] != 0;  // T_{i+1} = I: T_{i+1} pi_{i+1} = pi_{i+1}
-    for (int a = tid; a < n; a += TEAM) {
-      double v = q[a];
-      for (int j = 0; j < n; j++) v = fma(Q[a * n + j], xi[j], v);
-      for (int j = 0; j < m; j++) v = fma(Mm[a * m + j], ui[j], v);
-      gx[a] = v;
-      double t = 0.0;
-      if (tne) t = pi1[a];
-      else
-        for (int j = 0; j < nb1; j++) t = fma(T1[a * n + j], pi1[j], t);
-      tp[a] = t;
-    }
-    for (int a = tid; a < m; a += TEAM) {
-      double v = r[a];
-      for (int j = 0; j < n; j++) v = fma(Mm[j * m + a], xi[j], v);
-      for (int j = 0; j < m; j++) v = fma(R[a * m + j], ui[j], v);
-      gu[a] = v;
+    // rows of x (n) and of u (m) side by side, on the same loops with their own pointers
+    for (int r = tid; r < n + m; r += TEAM) {
+      const bool ra = r < n;
+      const int a = ra ? r : r - n;
+      const double *p1 = ra ? Q + a * n : Mm + a, *p2 = (ra ? Mm : R) + a * m;
+      const int st = ra ? 1 : m;
+      double v = ra ? q[a] : rv[a];
+      for (int j = 0; j < n; j++) v = fma(p1[j * st], xi[j], v);
+      for (int j = 0; j < m; j++) v = fma(p2[j], ui[j], v);
+      (ra ? gx : gu)[a] = v;
+      if (ra) {
+        double t = tne ? pi1[a] : 0.0;
+        if (!tne)
+          for (int j = 0; j < nb1; j++) t = fma(T1[a * n + j], pi1[j], t);
+        tp[a] = t;
+      }
     }
     tsync();
-    for (int a = tid; a < n; a += TEAM) {
-      double v = gx[a];
-      for (int l = 0; l < n; l++) v = fma(A[l * n + a], tp[l], v);
-      rx[a] = v;
-    }
-    for (int a = tid; a < m; a += TEAM) {
-      double v = gu[a];
-      for (int l = 0; l < n; l++) v = fma(B[l * m + a], tp[l], v);
-      ws[g.ws.ru + a] = v;
+    for (int r = tid; r < n + m; r += TEAM) {
+      const bool ra = r < n;
+      const int a = ra ? r : r - n, st = ra ? n : m;
+      const double *p = ra ? A + a : B + a;
+      double v = (ra ? gx : gu)[a];
+      for (int l = 0; l < n; l++) v = fma(p[l * st], tp[l], v);
+      (ra ? rx : ws + g.ws.ru)[a] = v;
     }
     // X = A' U_{i+1} (n x r1)
     for (int idx = tid; idx < n * r1; idx += TEAM) {

@@ -1275,7 +1275,7 @@ __global__ void k_post_roll(Group g, int corr) {
 // ill-conditioned |Y| is large, and that cancellation would set the accuracy
 // of the costates and so of the multipliers.  The offsets that the next pass's chain (PLIN) adds to
 // its maps, rq + K' rr + Phi' P_{i+1} rc (ws.gv), follow from the stage's residual at once, while it
-// is in shared memory.  Per task: 4n + 2m doubles.
+// is in shared memory.  Per task: 5n + 3m doubles.
 __global__ void k_resid(Group g, int per_task) {
   for_stages(g, [&](const int s) {
     const StageInfo S = g.st[s];
@@ -1292,69 +1292,81 @@ __global__ void k_resid(Group g, int per_task) {
     const double *T = ws + g.ws.UT + ur, *Tn = wn + g.ws.UT + ur1;
     const double *Y = ws + g.ws.Y, *Z = ws + g.ws.Z, *Ab = ws + g.ws.Ab, *Bb = ws + g.ws.Bb;
     double *sm = team_smem(per_task);
-    double *xs = sm, *us = xs + n, *lh = us + m, *ga = lh + n, *gb = ga + n, *rcs = gb + m;
+    double *xs = sm, *us = xs + n, *lh = us + m, *ga = lh + n, *gb = ga + n, *g2 = gb + m, *rcs = g2 + n + m;
     // T_i = I, t_i = 0 (te) or T_{i+1} = I (tne): the products with them are their other factor
     const bool te = wi[SI_TEYE] != 0, tne = !last && stage_wi(g, s + 1)[SI_TEYE] != 0;
-    // One lane per row, rows of different blocks side by side: an FP64 instruction costs its warp
-    // the same whatever its active lanes, so rows of three blocks in one instruction take the
-    // time of the longest.  p[j sp] x[j] summed onto v in order of j.
+    // An FP64 instruction costs its warp the same whatever its active lanes, so what counts is how
+    // many follow one another: rows of different blocks lie side by side and run the same loop on
+    // their own pointers (a branch per block would run one block after the other), long rows are two
+    // items, and a few rows are split over several lanes.  p[j sp] x[j] summed onto v in order of j.
     auto dot = [](double v, const double *p, int sp, const double *x, int len) {
 #pragma unroll 4
       for (int j = 0; j < len; j++) v = fma(p[(size_t)j * sp], x[j], v);
       return v;
     };
-    // u_i (m rows), x_i (n), T_{i+1} pi_{i+1} (n)
-    const int mm = last ? 0 : m;
-    for (int r = tid; r < (last ? n : mm + 2 * n); r += TEAM) {
-      if (r < mm) {
-        us[r] = dot(dot(ws[g.ws.y + r], Y + r * n, 1, z, nx), Z + r * m, 1, v, mu);
-      } else if (r < mm + n) {
-        const int a = r - mm;
-        xs[a] = te ? z[a] : dot(ws[g.ws.t + a], T + a * n, 1, z, nx);
-      } else {
-        const int l = r - mm - n;
-        lh[l] = tne ? pin[l] : dot(0.0, Tn + l * n, 1, pin, ny);
-      }
+    // u_i = Y z + Z v + y
+    if (!last) {
+      const int parts = m <= 8 ? 4 : 2;
+      split_rows(m, parts, [&](int r, int k) {
+        double v0 = k == 0 ? ws[g.ws.y + r] : 0.0;
+        for (int j = k; j < nx; j += parts) v0 = fma(Y[r * n + j], z[j], v0);
+        for (int j = k; j < mu; j += parts) v0 = fma(Z[r * m + j], v[j], v0);
+        return v0;
+      }, [&](int r, double v0) { us[r] = v0; });
+    }
+    // x_i and T_{i+1} pi_{i+1}
+    for (int r = tid; r < (last ? n : 2 * n); r += TEAM) {
+      const bool rx = r < n;
+      const int a = rx ? r : r - n;
+      double v0 = rx ? (te ? z[a] : ws[g.ws.t + a]) : (tne ? pin[a] : 0.0);
+      if (rx ? !te : !tne) v0 = dot(v0, (rx ? T : Tn) + a * n, 1, rx ? z : pin, rx ? nx : ny);
+      (rx ? xs : lh)[a] = v0;
     }
     tsync();
     const double *Q = g.Q + P.oQ + (size_t)i * n * n, *q = g.qv + P.oqv + (size_t)i * n;
     const double *A = g.A + P.oA + (size_t)i * n * n, *B = g.B + P.oB + (size_t)i * n * m;
     const double *Mm = g.M + P.oM + (size_t)i * n * m, *R = g.R + P.oR + (size_t)i * m * m;
     const double *rv = g.rv + P.orv + (size_t)i * m;
-    // a = g^x + A'lh (n rows), b = g^u + B'lh (m), the dynamics' residual (ny)
-    for (int r = tid; r < (last ? n : n + m + ny); r += TEAM) {
-      const bool ra = r < n, rb = !ra && r < n + m;
-      const int a = ra ? r : (rb ? r - n : r - n - m);
-      double s0 = ra ? q[a] : (rb ? rv[a] : ws[g.ws.cb + a] - zn[a]);
-      s0 = dot(s0, ra ? Q + a * n : (rb ? Mm + a : Ab + a * n), rb ? m : 1, ra || rb ? xs : z, ra || rb ? n : nx);
-      if (!last) {
-        s0 = dot(s0, ra ? Mm + a * m : (rb ? R + a * m : Bb + a * m), 1, ra || rb ? us : v, ra || rb ? m : mu);
-        if (ra || rb) s0 = dot(s0, ra ? A + a : B + a, ra ? n : m, lh, n);
-      }
-      if (ra) ga[a] = s0;
-      else if (rb) gb[a] = s0;
-      else ws[g.ws.rc + a] = rcs[a] = s0;
+    // g^x (n rows) and g^u (m); A'lh and B'lh (the same rows, into g2); the dynamics' residual (ny)
+    const int rows = n + m;
+    for (int r = tid; r < (last ? n : 2 * rows + ny); r += TEAM) {
+      const int h = r < rows ? 0 : (r < 2 * rows ? 1 : 2), a = r - h * rows;
+      const bool ra = h < 2 && a < n, rb = h < 2 && !ra;  // rows of x, of u
+      const int b = rb ? a - n : a;
+      const double *p1 = h == 0 ? (ra ? Q + a * n : Mm + b) : h == 1 ? (ra ? A + a : B + b) : Ab + a * n;
+      const double *p2 = h == 0 ? (ra ? Mm + a * m : R + b * m) : Bb + a * m;
+      double s0 = h == 0 ? (ra ? q[a] : rv[b]) : h == 1 ? 0.0 : ws[g.ws.cb + a] - zn[a];
+      s0 = dot(s0, p1, h == 0 ? (ra ? 1 : m) : h == 1 ? (ra ? n : m) : 1, h == 0 ? xs : h == 1 ? lh : z, h == 2 ? nx : n);
+      s0 = dot(s0, p2, 1, h == 0 ? us : v, last || h == 1 ? 0 : h == 0 ? m : mu);
+      (h == 0 ? ga : h == 1 ? g2 : rcs)[a] = s0;
+      if (h == 2) ws[g.ws.rc + a] = s0;
     }
     tsync();
-    // rq (nx rows, kept in xs), rr (mu, in us), P_{i+1} rc (ny, in lh)
+    if (!last) {  // a = g^x + A'lh, b = g^u + B'lh
+      for (int r = tid; r < rows; r += TEAM) ga[r] += g2[r];
+      tsync();
+    }
+    // P_{i+1} rc (ny rows, into lh), rq (nx, kept in xs), rr (mu, in us)
     const double *Pn = wn + g.ws.P;
-    for (int r = tid; r < nx + mu + ny; r += TEAM) {
-      double s0;
-      if (r < nx) {
-        s0 = te ? ga[r] - pi[r] : dot(-pi[r], T + r, n, ga, n);
-        if (!last) s0 = dot(s0, Y + r, n, gb, m);
-        ws[g.ws.rq + r] = xs[r] = s0;
-      } else if (r < nx + mu) {
-        s0 = dot(0.0, Z + r - nx, m, gb, m);
-        ws[g.ws.rr + r - nx] = us[r - nx] = s0;
-      } else {
-        lh[r - nx - mu] = dot(0.0, Pn + (r - nx - mu) * n, 1, rcs, ny);
-      }
+    for (int r = tid; r < ny + nx + mu; r += TEAM) {
+      const int h = r < ny ? 0 : (r < ny + nx ? 1 : 2), a = h == 0 ? r : (h == 1 ? r - ny : r - ny - nx);
+      double s0 = h == 1 ? (te ? ga[a] : 0.0) - pi[a] : 0.0;
+      if (h == 1 && !te) s0 = dot(s0, T + a, n, ga, n);
+      s0 = dot(s0, h == 0 ? Pn + a * n : (h == 1 ? Y + a : Z + a), h == 0 ? 1 : (h == 1 ? n : m), h == 0 ? rcs : gb,
+               last ? 0 : (h == 0 ? ny : m));
+      (h == 0 ? lh : (h == 1 ? xs : us))[a] = s0;
+      if (h > 0) ws[(h == 1 ? g.ws.rq : g.ws.rr) + a] = s0;
     }
     if (last) return;
     tsync();
     const double *K = ws + g.ws.K, *Phi = ws + g.ws.Phi;
-    for (int r = tid; r < nx; r += TEAM) ws[g.ws.gv + r] = dot(dot(xs[r], K + r, n, us, mu), Phi + r, n, lh, ny);
+    const int parts = n <= 8 ? 4 : n <= 16 ? 2 : 1;
+    split_rows(nx, parts, [&](int r, int k) {
+      double v0 = k == 0 ? xs[r] : 0.0;
+      for (int j = k; j < mu; j += parts) v0 = fma(K[j * n + r], us[j], v0);
+      for (int j = k; j < ny; j += parts) v0 = fma(Phi[j * n + r], lh[j], v0);
+      return v0;
+    }, [&](int r, double v0) { ws[g.ws.gv + r] = v0; });
   });
 }
 
@@ -1378,17 +1390,18 @@ __global__ void k_pcorr(Group g, int per_task) {
       const int a = idx / mu, l = idx - a * mu;
       Ls[a * m + l] = ws[g.ws.Lh + a * m + l];
     }
-    for (int b = tid; b < ny; b += TEAM) {
-      double s0 = ppn[b];
-      for (int l = 0; l < ny; l++) s0 = fma(Pn[b * n + l], rc[l], s0);
-      w[b] = s0;
-    }
+    const int pw = n <= 8 ? 4 : n <= 16 ? 2 : 1, ph = m <= 8 ? 4 : 2;
+    split_rows(ny, pw, [&](int r, int k) {
+      double s0 = k == 0 ? ppn[r] : 0.0;
+      for (int l = k; l < ny; l += pw) s0 = fma(Pn[r * n + l], rc[l], s0);
+      return s0;
+    }, [&](int r, double s0) { w[r] = s0; });
     tsync();
-    for (int a = tid; a < mu; a += TEAM) {
-      double s0 = ws[g.ws.rr + a];
-      for (int b = 0; b < ny; b++) s0 = fma(Bb[b * m + a], w[b], s0);
-      hu[a] = s0;
-    }
+    split_rows(mu, ph, [&](int r, int k) {
+      double s0 = k == 0 ? ws[g.ws.rr + r] : 0.0;
+      for (int l = k; l < ny; l += ph) s0 = fma(Bb[l * m + r], w[l], s0);
+      return s0;
+    }, [&](int r, double s0) { hu[r] = s0; });
     tsync();
     // dv = -H_uu^{-1} hu with H_uu = L L' (L = Ls, lower): forward then backward
     // substitution by the first warp, lane a holding row a (mu <= 16), column by column; the
@@ -1430,10 +1443,12 @@ __global__ void k_recover(Group g, double *x, double *u) {
     const int *wi = stage_wi(g, s);
     const int ur = wi[SI_UR], nb = n - ur;
     const double *T = ws + g.ws.UT + ur, *z = ws + g.ws.z;
+    const bool te = wi[SI_TEYE] != 0;  // T = I, t = 0
     bool bad = false;
     for (int a = tid; a < n; a += TEAM) {
-      double v = ws[g.ws.t + a];
-      for (int j = 0; j < nb; j++) v = fma(T[a * n + j], z[j], v);
+      double v = te ? z[a] : ws[g.ws.t + a];
+      if (!te)
+        for (int j = 0; j < nb; j++) v = fma(T[a * n + j], z[j], v);
       x[P.ox + (size_t)S.i * n + a] = v;
       bad = bad || !isfinite(v);
     }

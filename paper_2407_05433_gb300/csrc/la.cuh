@@ -70,6 +70,19 @@ __device__ __forceinline__ double team_max_key(unsigned long long key) {
 }
 __device__ __forceinline__ double team_max(double v) { return team_max_key(abs_key(v)); }  // v >= 0
 
+// put(r, the sum of f(r, part) over the parts) for the rows r < rows, the parts of a row on neighbouring
+// lanes (parts a power of two).
+template <typename F, typename Put>
+__device__ __forceinline__ void split_rows(int rows, int parts, F f, Put put) {
+  const int tid = team_rank(), part = tid & (parts - 1), sh = __ffs(parts) - 1;
+  for (int i0 = 0; i0 < rows * parts; i0 += TEAM) {
+    const int r = (i0 + tid) >> sh;
+    double v = r < rows ? f(r, part) : 0.0;
+    for (int o = parts >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    if (part == 0 && r < rows) put(r, v);
+  }
+}
+
 // C (m x n) = op(A) op(B) (beta = 0) or C + op(A) op(B) (beta = 1); op(A) is m x k, op(B) is
 // k x n.  C must not alias A or B.  One accumulator per element: FP64 instructions of one
 // sub-partition do not overlap, so a second one would only add an addition.
