@@ -104,16 +104,18 @@ namespace {
 // kernel and state dimension on the 4096-problem uneven batch (each (n, m) group
 // alone, about seven problems per SM) or on 1280 problems of 48 stages.  For example, the
 // chunk up-sweeps of the long horizon (65536 stages in 1024 chunks) take 27 ms with two
-// warps per chunk against 37 with one; the affine chains of 1280 problems take 0.37 / 0.82
-// ms with 1 / 2 warps at n = 8, 0.72 / 0.72 / 0.86 with 1 / 2 / 4 at n = 16 and 1.26 /
-// 0.85 / 1.61 with 2 / 4 / 8 at n = 24 (160 problems at n = 32 0.68 / 0.55 with 4 / 8; of 320 problems 0.22 / 0.29 at n = 8, so they
-// keep the entry there); the stage elimination takes 2.2 / 3.8 ms with 1 / 2 at n = 8, 8.0
-// / 7.3 / 8.6 with 1 / 2 / 4 at n = 16 and 14.6 / 15.1 / 14.2 at n = 24.  The Riccati
-// sweep's products have thousands of independent integer multiply-adds per stage from
+// warps per chunk against 37 with one; the stage elimination takes 2.81 / 3.00 / 4.20 ms with
+// 1 / 2 / 4 at n = 16 and four rows a stage (65536 stages), but 3.43 / 3.25 with 1 / 2 at up to seven
+// rows (640 problems), and 5.36 / 3.36 / 2.84 / 3.25 with 1 / 2 / 4 / 8 at n = 32 (160 problems).
+// The affine chains (row warps beside the one that moves the data): 256 problems of 256 stages at
+// n = 16 133 / 102 / 154 us with 1 / 2 / 4, 160 problems at n = 32 110 / 91 / 124 with 2 / 4 / 8.  The
+// Riccati sweep's products have thousands of independent integer multiply-adds per stage from
 // n = 16 on: 1.44 / 1.48 / 1.65 ms with 1 / 2 / 4 warps at n = 8, 2.56 / 2.09 / 2.23 at
-// n = 12, 3.85 / 3.40 / 3.09 at n = 16 and 8.49 / 6.00 / 5.86 at n = 24; with 320 problems
+// n = 12, 3.85 / 3.40 / 3.09 at n = 16 and 8.49 / 6.00 / 5.86 at n = 24 (1280 problems); with 320
 // four warps are best at every n (0.60 against 0.71 ms with one at n = 8, 2.6 against 4.7
-// at n = 24).
+// at n = 24); with two sweeps per SM 8.1 / 7.0 / 6.4 / 4.8 ms with 1 / 2 / 4 / 8 at n = 16 (256
+// problems), with one 6.2 / 5.1 / 3.3 with 4 / 8 / 16 at n = 32, but 1.67 / 2.45 with 4 / 8 where
+// three share an SM (457 chunks at n = 16).
 int team_for(const eclqr_handle *h, const void *kern, int ntasks, int n) {
   if (h->opt.team_warps != 0) return h->opt.team_warps;
   // four lanes a row of an affine chain (two below n = 5), and never more than a row's latency pays for
@@ -123,16 +125,16 @@ int team_for(const eclqr_handle *h, const void *kern, int ntasks, int n) {
     return ntasks > 2 * h->sms || n < 12 ? kTeamWarps : n < 24 ? 8 : 16;
   }
   if (ntasks < h->sms) return kTeamWarps;
-  // warps below n1, from n1, n2 and n3 up; few: warps with one to four tasks per SM (-1: the
-  // entry, 0: the entry, at least two -- 256 problems of 256 stages, n = 16: 37 ms with two, 42 with one, 49 with four)
-  static const struct { const void *fn; int warps, few, n1, warps1, n2, warps2, n3, warps3; } table[] = {
-      {(const void *)k_riccati_down, 1, 0, 12, 2, 16, 4},
+  // warps below n1, from n1 and n2 up; with one to four tasks per SM at least two (256 problems of
+  // 256 stages, n = 16: 37 ms with two, 42 with one, 49 with four)
+  static const struct { const void *fn; int warps, n1, warps1, n2, warps2; } table[] = {
+      {(const void *)k_riccati_down, 1, 12, 2, 16, 4},
       {(const void *)k_riccati_down_f32, 1},     {(const void *)k_riccati_finish, 1},
-      {(const void *)k_elim, 1, 0, 16, 2, 24, 4}, {(const void *)k_primal_down, 1, 0, 24, 2},
-      {(const void *)k_dual_down, 1},            {(const void *)k_primal_stage, 1, 0, 24, 2},
+      {(const void *)k_elim, 1, 16, 2, 24, 4},    {(const void *)k_primal_down, 1, 24, 2},
+      {(const void *)k_dual_down, 1},            {(const void *)k_primal_stage, 1, 24, 2},
       {(const void *)k_dual_leaf, 1},
       {(const void *)k_aff_prep, 1},             {(const void *)k_stage_lists, 1},
-      {(const void *)k_dual_stage, 1, 0, 24, 2},         {(const void *)k_param, 1},
+      {(const void *)k_dual_stage, 1, 24, 2},    {(const void *)k_param, 1},
       {(const void *)k_resid, 1},                {(const void *)k_pcorr, 1},
       {(const void *)k_kkt, 1},                  {(const void *)k_post_roll, 1},
       {(const void *)k_recover, 1},              {(const void *)k_check_inputs, 1},
@@ -147,11 +149,8 @@ int team_for(const eclqr_handle *h, const void *kern, int ntasks, int n) {
   const bool many = ntasks >= kManyTasksPerSm * h->sms;
   for (const auto &e : table)
     if (e.fn == kern) {
-      const int w = e.n3 && n >= e.n3   ? e.warps3
-                    : e.n2 && n >= e.n2 ? e.warps2
-                    : e.n1 && n >= e.n1 ? e.warps1
-                                        : e.warps;
-      return many || e.few < 0 ? w : (e.few ? e.few : std::max(w, 2));
+      const int w = e.n2 && n >= e.n2 ? e.warps2 : e.n1 && n >= e.n1 ? e.warps1 : e.warps;
+      return many ? w : std::max(w, 2);
     }
   return kTeamWarps;
 }

@@ -91,7 +91,8 @@ __global__ void __launch_bounds__(256, 3) k_dual_stage(Group g, const double *x,
     const double *U1 = wn + g.ws.UT, *T1 = wn + g.ws.UT + r1, *pi1 = wn + g.ws.pi;
     // objective gradients (eq. objective-gradients) and T_{i+1} pi_{i+1}
     const bool tne = win[SI_TEYE] != 0;  // T_{i+1} = I: T_{i+1} pi_{i+1} = pi_{i+1}
-    // rows of x (n) and of u (m) side by side, on the same loops with their own pointers
+    // rows of x (n) and of u (m) side by side, on the same loops with their own pointers (51200 stages at
+    // n = 12 127 us, 266 with a loop for each)
     for (int r = tid; r < n + m; r += TEAM) {
       const bool ra = r < n;
       const int a = ra ? r : r - n;

@@ -221,12 +221,16 @@ __global__ void k_lqr_level(Group g, int src, int d, int per_task) {
 // exponents come from the diagonal, so entries are at most 1 in magnitude by Cauchy-Schwarz and
 // the scaling of states and controls does not matter.
 //
-// What bounds it: the integer multiply-adds (7 per 114 x 57 bit product, 4.1 cycles each per SM
-// sub-partition) where many problems share an SM, the latency of one stage's phases where few do.
+// What bounds it: where many problems share an SM, the fixed latency of its integer chains and the
+// barriers between a stage's phases (n = 24, 14 warps an SM: 40% of the issue slots, of 46k warp
+// instructions a stage 7k limb products); where few do, the latency of one stage's phases.
 // Loops are kept rolled: with them unrolled the code outgrew the instruction cache and 1280
 // problems of 64 stages at n = 24 took 12.8 ms instead of 8.0.  Against the FP64 QR, 64 stages of
 // 1280 problems: n = 24 20.3 -> 7.8 ms, n = 16 10.2 -> 4.1, n = 8 3.38 -> 1.93; of 160 problems at
 // n = 24 7.5 -> 2.9 ms (k_riccati_finish, which no longer forms P = R'R, 2.24 -> 1.0 at 1280, n = 24).
+// Then pivots by one warp, the minimiser's rows in one pass, H a stage ahead, single-entry tiles and
+// wider teams for few sweeps: 256 problems of 256 stages at n = 16 6.36 -> 3.57 ms, 160 problems at
+// n = 32 6.15 -> 3.38, one sweep of 64 stages at n = 4 0.42 -> 0.35.
 // The blocks are offsets into the task's shared memory (in elements of their type), so that every
 // access compiles to a shared-memory instruction with a 32-bit address.
 struct RiccatiFx {
@@ -1024,8 +1028,9 @@ __global__ void k_aff_level(Group g, int src, int d, int fwd, int per_task) {
 // does it: it copies the blocks [G | gv] asynchronously kAffRing stages ahead into shared memory,
 // stores y and looks up the dimensions.  The others hold a row over SEG lanes, read the coming
 // stage's entries into registers while the FP64 instructions run, and meet it at one barrier per
-// stage.  Per stage, 256 problems of 256 stages at n = 16 and 64 stages at n = 4: 0.70 and 0.72 us with the
-// next stage's entries read one stage ahead by the same warps, 0.63 and 0.57 with the ring alone.
+// stage.  Per stage, 256 problems of 256 stages at n = 16 and 64 stages at n = 4: 0.40 and 0.32 us; 0.70
+// and 0.72 with the next stage's entries read one stage ahead by the same warps, 0.63 and 0.57 with
+// the ring alone.
 template <int SEG, int KP>
 static __device__ __forceinline__ void aff_rows(const double *ring, double *ya, double *yb, const int *sdim, int n, bool tr,
                                                 int steps, int dcur) {
@@ -1275,7 +1280,8 @@ __global__ void k_post_roll(Group g, int corr) {
 // ill-conditioned |Y| is large, and that cancellation would set the accuracy
 // of the costates and so of the multipliers.  The offsets that the next pass's chain (PLIN) adds to
 // its maps, rq + K' rr + Phi' P_{i+1} rc (ws.gv), follow from the stage's residual at once, while it
-// is in shared memory.  Per task: 5n + 3m doubles.
+// is in shared memory.  640 problems of 32 to 128 stages: 353 us at n = 16, 150 at n = 8 (445 and 187 with
+// one lane per row and a branch per block).  Per task: 5n + 3m doubles.
 __global__ void k_resid(Group g, int per_task) {
   for_stages(g, [&](const int s) {
     const StageInfo S = g.st[s];
@@ -1372,7 +1378,8 @@ __global__ void k_resid(Group g, int per_task) {
 
 // Correction controls of a refinement pass: with w = P_{i+1} rc_i + p'_{i+1},
 // k'_i = -H_uu^{-1} (rr_i + Bbar' w) through the Cholesky factor of H_uu (-> dv), and the offsets
-// rc + Bbar k' of the chain that follows (CROLL, ws.gv).
+// rc + Bbar k' of the chain that follows (CROLL, ws.gv).  Short products are split over two or four
+// lanes a row: 640 problems at n = 16 180 -> 137 us, at n = 8 106 -> 94.
 __global__ void k_pcorr(Group g, int per_task) {
   for_stages(g, [&](const int s) {
     const StageInfo S = g.st[s];
