@@ -229,8 +229,8 @@ __global__ void k_lqr_level(Group g, int src, int d, int per_task) {
 // 1280 problems: n = 24 20.3 -> 7.8 ms, n = 16 10.2 -> 4.1, n = 8 3.38 -> 1.93; of 160 problems at
 // n = 24 7.5 -> 2.9 ms (k_riccati_finish, which no longer forms P = R'R, 2.24 -> 1.0 at 1280, n = 24).
 // Then pivots by one warp, the minimiser's rows in one pass, H a stage ahead, single-entry tiles and
-// wider teams for few sweeps: 256 problems of 256 stages at n = 16 6.36 -> 3.57 ms, 160 problems at
-// n = 32 6.15 -> 3.38, one sweep of 64 stages at n = 4 0.42 -> 0.35.
+// wider teams for few sweeps: 256 problems of 256 stages at n = 16 6.36 -> 3.45 ms, 160 problems at
+// n = 32 6.15 -> 3.31, one sweep of 64 stages at n = 4 0.42 -> 0.32.
 // The blocks are offsets into the task's shared memory (in elements of their type), so that every
 // access compiles to a shared-memory instruction with a 32-bit address.
 struct RiccatiFx {
@@ -320,25 +320,38 @@ static __device__ __noinline__ void riccati_value(const RiccatiFx w, int nz, int
   }
   team_sync();
   const bool bad = w.bad() != 0;
+  const int items = nz * (nz + 1) / 2 + nz;
+  auto store = [&](int a, int b, i128 v) {
+    int s;
+    const long long top = fx_lead(v, s);
+    const double x = bad ? __longlong_as_double(0x7ff8000000000000ll) : fx_to(top, s + w.e(z0 + a) + w.e(z0 + b) - kFxP);
+    if (b < nz) {
+      Po[a * ldo + b] = x;
+      Po[b * ldo + a] = x;
+    } else {
+      po[a] = x;
+    }
+  };
+  // the FP64 values, which the sweep itself does not wait for, from the team's other end where its
+  // last warps have no entry of their own
+  const bool apart = 2 * items <= TEAM;
   int a = 0, row = 0;  // row: linear index of (a, a); nz + 1 - a entries per row
 #pragma unroll 1
-  for (int idx = tid; idx < nz * (nz + 1) / 2 + nz; idx += TEAM) {
+  for (int idx = tid; idx < items; idx += TEAM) {
     while (idx - row > nz - a) row += nz + 1 - a++;
     const int b = a + idx - row;
     const i128 v = w.Gi(raw(a, b));
     const int4 l = fx_split4(fx_shift(v, w.e(z0 + a) + w.e(z0 + b) - w.eP(a) - w.eP(b)));
     w.P(a * w.ldp + b) = l;
     if (b < nz) w.P(b * w.ldp + a) = l;
-    if (Po) {
-      int s;
-      const long long top = fx_lead(v, s);
-      const double x = bad ? __longlong_as_double(0x7ff8000000000000ll) : fx_to(top, s + w.e(z0 + a) + w.e(z0 + b) - kFxP);
-      if (b < nz) {
-        Po[a * ldo + b] = x;
-        Po[b * ldo + a] = x;
-      } else {
-        po[a] = x;
-      }
+    if (Po && !apart) store(a, b, v);
+  }
+  if (Po && apart) {
+    const int idx = TEAM - 1 - tid;
+    if (idx < items) {
+      a = row = 0;
+      while (idx - row > nz - a) row += nz + 1 - a++;
+      store(a, a + idx - row, w.Gi(raw(a, a + idx - row)));
     }
   }
   team_sync();
@@ -488,23 +501,20 @@ static __device__ __forceinline__ void riccati_stage(const Group &g, const Ricca
   team_sync();
   fetch();
   // exponents of the columns of G + H from its diagonal, of the offsets from their largest entry
-#pragma unroll 1
-  for (int j = tid; j < kh; j += TEAM) {
-    const i128 d = w.Gi(packed(j, j));
-    const int t = max(d != 0 ? fx_bits(d) - kFxP + 2 * w.al(j) : kFxNone, fx_expo(w.H(packed(j, j))));
-    w.e(j) = t > kFxNone / 2 ? (t + 2) >> 1 : 0;
-  }
-  team_sync();
   if (tid < 32) {
-    int t = kFxNone;
+    int to = kFxNone;
 #pragma unroll 1
     for (int j = tid; j < kh; j += 32) {
-      const i128 d = w.Gi(packed(j, kh));
-      t = max(t, (d != 0 ? fx_bits(d) - kFxP + w.al(j) + w.al(kh) : kFxNone) - w.e(j));
-      t = max(t, fx_expo(w.H(packed(j, kh))) - w.e(j));
+      const int jj = packed(j, j), jo = packed(j, kh);
+      const i128 d = w.Gi(jj), o = w.Gi(jo);
+      const int t = max(d != 0 ? fx_bits(d) - kFxP + 2 * w.al(j) : kFxNone, fx_expo(w.H(jj)));
+      const int e = t > kFxNone / 2 ? (t + 2) >> 1 : 0;
+      w.e(j) = e;
+      to = max(to, (o != 0 ? fx_bits(o) - kFxP + w.al(j) + w.al(kh) : kFxNone) - e);
+      to = max(to, fx_expo(w.H(jo)) - e);
     }
-    t = __reduce_max_sync(kFull, t);
-    if (tid == 0) w.e(kh) = t > kFxNone / 2 ? t + 1 : 0;
+    to = __reduce_max_sync(kFull, to);
+    if (tid == 0) w.e(kh) = to > kFxNone / 2 ? to + 1 : 0;
   }
   team_sync();
   {
@@ -607,10 +617,11 @@ static __device__ __forceinline__ void riccati_stage(const Group &g, const Ricca
   // the minimiser's rows y_j / sqrt(d 2^(2h))
   const bool bad = w.bad() != 0;
   if (Rv) {
-    // every row at once, from the packed rows 0 .. mu - 1
+    // every row at once, from the packed rows 0 .. mu - 1, from the team's other end: its last warps
+    // have fewer entries of the Schur complement, or none
     int k = 0, row = 0;
 #pragma unroll 1
-    for (int idx = tid; idx < packed(mu, mu); idx += TEAM) {
+    for (int idx = TEAM - 1 - tid; idx < packed(mu, mu); idx += TEAM) {
       while (idx - row >= ld - k) row += ld - k++;
       const int j = k + idx - row;
       const unsigned long long rs = fx_rsqrt((unsigned long long)((fx_join4(w.G(row)) << w.hp(k)) >> 50));
