@@ -173,7 +173,10 @@ int eclqr_create(const eclqr_desc *desc, const eclqr_options *opt, eclqr_handle 
 
 /* Feasible-domain scan and stagewise elimination of Algorithm 1 (Sec. 3-5)
  * plus the coefficient part of the reduced Riccati solve (Sec. 6): everything
- * that does not depend on s_0.  status: device int32[P], overwritten. */
+ * that does not depend on s_0.  status: device int32[P], overwritten.
+ * The Riccati sweep (FP64 mode) resolves a value function's curvature down to
+ * about 2^-106 of |P| |A|^2; directions below that (a long stretch without control that
+ * grows) count as that small.  Subnormal entries of the reduced problem count as zero in it. */
 int eclqr_build(eclqr_handle *h, const eclqr_data *data, int32_t *status, void *stream);
 
 /* After eclqr_build: flags (device int32[P]) receives 1 for every problem whose

@@ -221,6 +221,16 @@ __global__ void k_lqr_level(Group g, int src, int d, int per_task) {
 // exponents come from the diagonal, so entries are at most 1 in magnitude by Cauchy-Schwarz and
 // the scaling of states and controls does not matter.
 //
+// Both hold only while the matrices stay positive semidefinite, and curvature below about 2^-106 of
+// |P| |A|^2 in a direction that is no coordinate axis is rounding noise: without more, a direction
+// of negative curvature gets gains of any size and the recursion grows without bound (a stretch of
+// 25 stages without control that grow by 4 each: gains of 1e18 and values past the limbs' 118 bits).
+// So every diagonal entry is raised by riccati_margin, more than the rounding that can make it
+// indefinite, after each product and each Schur complement, and a pivot below it counts as
+// noise.  Directions beyond the resolution then keep a small positive curvature, as the square
+// root's rows do by their form, and the recursion forgets them as it should.  n^2 2^-106 of |P| |A|^2 is
+// also the size of a square root's own rounding.
+//
 // What bounds it: where many problems share an SM, the fixed latency of its integer chains and the
 // barriers between a stage's phases (n = 24, 14 warps an SM: 40% of the issue slots, of 46k warp
 // instructions a stage 7k limb products); where few do, the latency of one stage's phases.
@@ -292,6 +302,13 @@ __device__ __forceinline__ void team_sync() {
   if (blockDim.x == 32) __syncwarp();
   else __syncthreads();
 }
+
+// What a diagonal entry is raised by, in units of 2^-114 of its scale: the rounding of W (up to four units
+// an entry after its scaling by 8) and of P's limbs (at most one) through n1 terms, as the norm of a matrix of kh
+// rows.  Of 615 recursions at n = 2 to 16 through stretches near and beyond the resolution 355 grew without
+// bound with no margin, 28 with a quarter of this one, none with half of it or all; where a square-root
+// QR in FP64 still has digits of the gains, the error here is half to two thirds of its error.
+__device__ __forceinline__ int riccati_margin(int n1, int kh) { return (n1 * kh >> 1) + 32; }
 
 // (j, k), j <= k < ld, of packed upper rows
 __device__ __forceinline__ int riccati_packed(int ld, int j, int k) { return j * ld - j * (j + 1) / 2 + k; }
@@ -453,7 +470,7 @@ static __device__ __forceinline__ void riccati_g(const RiccatiFx w, int n1, int 
 #pragma unroll
     for (int q = 0; q < T * T; q++) {
       const int jj = q < T ? j : j1, kk = T == 2 && (q & 1) ? k1 : k;
-      if (jj <= kk) w.Gi(riccati_packed(ld, jj, kk)) = acc[q].template value<54>();
+      if (jj <= kk) w.Gi(riccati_packed(ld, jj, kk)) = acc[q].template value<54>() + (jj == kk ? riccati_margin(n1, kh) : 0);
     }
   }
 }
@@ -541,7 +558,7 @@ static __device__ __forceinline__ void riccati_stage(const Group &g, const Ricca
     const int gk = packed(k, 0);
     if (tid < 32) {  // one long chain of scalars: the other warps wait for it instead of repeating it
       i128 d = fx_join4(w.G(gk + k));
-      const bool noise = d <= 0;
+      const bool noise = d <= riccati_margin(n1, kh);
       if (noise) d = (i128)1 << (kFxP - 53);  // rounding noise of a singular pivot
       const int h = (kFxP - fx_bits(d)) >> 1;
       const i128 dp = d << (2 * h);
@@ -611,7 +628,7 @@ static __device__ __forceinline__ void riccati_stage(const Group &g, const Ricca
       acc.zero();
 #pragma unroll 1
       for (int k = 0; k < mu; k++) acc.mad(w.W(k * ldx + mu + a), w.G(packed(k, mu + b)));
-      w.Gi(packed(mu + a, mu + b)) -= acc.value();
+      w.Gi(packed(mu + a, mu + b)) -= acc.value() - (a == b ? riccati_margin(n1, kh) : 0);
     }
   }
   // the minimiser's rows y_j / sqrt(d 2^(2h))
@@ -713,7 +730,7 @@ static __device__ void riccati_task(const Group &g, int fin, int t, int per_task
     for (int idx = tid; idx < nz * (nz + 1); idx += TEAM) {
       const int j = idx / (nz + 1), k = idx - j * (nz + 1);
       if (k < j) continue;
-      i128 s = 0;
+      i128 s = j == k ? rv * nz : 0;  // the rounding of rv shifted terms, as a matrix norm
 #pragma unroll 1
       for (int r = 0; r < rv; r++) {
         const int2 x = w.A(r * w.ldx + j), y = w.A(r * w.ldx + k);
