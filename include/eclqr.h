@@ -244,12 +244,21 @@ int eclqr_kkt_residual_parts(eclqr_handle *h, const double *s0, const double *x,
  *   ECLQR_ESTATE until the next eclqr_build or eclqr_set_costs.
  *   Outside a stream capture the call waits, once per pass, for 12 bytes of
  *   flags telling whether any problem takes part, and returns when none does
- *   (so it is host-synchronous); on a capturing stream it records one pass as
- *   the body of a conditional node that a replay runs while some problem takes
- *   part (where the graph takes no such node, all opt.kkt_refine passes, whose
- *   kernels return at once for the problems that take no part). */
+ *   (so it is host-synchronous); on a capturing stream it records all
+ *   opt.kkt_refine passes, whose kernels return at once for the problems
+ *   that take no part, or a loop (eclqr_capture_loop). */
 int eclqr_refine(eclqr_handle *h, const double *s0, double *x, double *u, double *lam, double *mu,
                  double *eta, double *alpha, double *resid, int32_t *status, void *stream);
+
+/* How eclqr_refine records itself on a capturing stream.  on = 0 (the state of a
+ * new handle): every pass, as plain nodes.  on = 1: one pass, as the body of a
+ * conditional node that a replay runs while some problem takes part, so that
+ * passes nobody needs cost nothing.  CUDA refuses to clone a graph that holds
+ * a conditional node or to put it into another graph as a child, so this is for
+ * captures whose graph the caller instantiates as it is.  Where the capturing
+ * graph takes no conditional handle, every pass is recorded all the same.  Results
+ * are the same either way.  Host only. */
+int eclqr_capture_loop(eclqr_handle *h, int32_t on);
 
 /* Mixed precision (opt.riccati_fp32 = 1): flags (device int32[P]) receives 1 for
  * every problem whose Riccati sweep eclqr_refine redid in FP64 since the last

@@ -79,7 +79,8 @@ struct eclqr_handle {
   double *zeros = nullptr;  // offsets of the corrections with homogeneous constraints
   int *any = nullptr;       // device: some problem takes part in the pass, rebuilds, takes the cheap
                             // correction; passes of a captured refinement so far
-  cudaStream_t loop_s = nullptr;  // the capturing stream of a captured refinement's loop
+  bool capture_loop = false;      // eclqr_capture_loop: a captured refinement may be a conditional loop
+  cudaStream_t loop_s = nullptr;  // the capturing stream of that loop
   bool in_loop = false;           // the launches being recorded are that loop's
   int *fp64 = nullptr;      // mixed precision: per-problem flags of the Riccati sweep's precision
   int *any_host = nullptr;  // pinned host copy of it
@@ -872,12 +873,12 @@ int eclqr_refine(eclqr_handle *h, const double *s0, double *x, double *u, double
   const RefineMasks mk = h->mk;
   const int corr = h->opt.corr_refine < 0 ? h->opt.refine : h->opt.corr_refine;
   // Outside a stream capture the passes stop as soon as no problem takes part (one 12-byte read
-  // back per pass, which also tells whether a pass rebuilds).  On a capturing stream the pass is
-  // recorded once, as the body of a conditional WHILE node whose condition k_refine_loop sets, so
-  // that a replay ends the same way (a 64-stage n = 4 problem that needs no pass: 1.9 ms with the
-  // eight passes recorded one after the other, 1.0 ms in the loop); where the stream's graph takes
-  // no conditional node, every pass is recorded, and its kernels return at once for problems that
-  // take no part.
+  // back per pass, which also tells whether a pass rebuilds).  On a capturing stream every pass is
+  // recorded, and its kernels return at once for problems that take no part; or, where the owner of
+  // the graph allows it (eclqr_capture_loop: such a graph cannot be cloned or put into another one), the
+  // pass is recorded once, as the body of a conditional WHILE node whose condition k_refine_loop
+  // sets, so that a replay ends as the eager call does (a 64-stage n = 4 problem that needs no pass: 1.9 ms
+  // with the eight passes recorded one after the other, 1.0 ms in the loop).
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) return ECLQR_ECUDA;
   const bool eager = cap == cudaStreamCaptureStatusNone;
@@ -956,6 +957,7 @@ int eclqr_refine(eclqr_handle *h, const double *s0, double *x, double *u, double
   // the passes as the body of a WHILE node; false where the capturing graph takes none (nothing is
   // recorded then)
   auto loop = [&](int first, int &rc) -> bool {
+    if (!h->capture_loop) return false;
     cudaGraph_t graph = nullptr;
     cudaGraphConditionalHandle cond;
     if (cudaStreamGetCaptureInfo(st, &cap, nullptr, &graph, nullptr, nullptr, nullptr) != cudaSuccess ||
@@ -1060,6 +1062,12 @@ int eclqr_refine(eclqr_handle *h, const double *s0, double *x, double *u, double
     h->stale = true;
     h->solved = false;
   }
+  return ECLQR_OK;
+}
+
+int eclqr_capture_loop(eclqr_handle *h, int32_t on) {
+  if (!h || on < 0 || on > 1) return ECLQR_EINVAL;
+  h->capture_loop = on != 0;
   return ECLQR_OK;
 }
 

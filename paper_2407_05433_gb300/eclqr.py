@@ -81,6 +81,8 @@ def load():
     lib.eclqr_kkt_residual_parts.restype = i32
     lib.eclqr_refine.argtypes = [vp] * 11
     lib.eclqr_refine.restype = i32
+    lib.eclqr_capture_loop.argtypes = [vp, ct.c_int32]
+    lib.eclqr_capture_loop.restype = i32
     lib.eclqr_riccati_fp64_flags.argtypes = [vp, vp, vp]
     lib.eclqr_riccati_fp64_flags.restype = i32
     lib.eclqr_reduced_dims.argtypes = [vp, vp, vp, vp]
@@ -155,6 +157,10 @@ def eclqr_kkt_residual_parts(h, s0, x, u, lam, mu, eta, alpha, resid, parts, str
 
 def eclqr_refine(h, s0, x, u, lam, mu, eta, alpha, resid, status, stream):
     return load().eclqr_refine(h, s0, x, u, lam, mu, eta, alpha, resid, status, stream)
+
+
+def eclqr_capture_loop(h, on):
+    return load().eclqr_capture_loop(h, on)
 
 
 def eclqr_kkt_residual_noalloc(desc, data, s0, x, u, lam, mu, eta, alpha, resid, stream):
@@ -342,8 +348,10 @@ class Batch:
 
         The graph keeps the current device pointers: refresh the inputs in place (self.d)
         and call replay().  A first eager pass on a side stream sets every kernel's
-        shared-memory attribute before capture.  Returns the number of kernel launches
-        recorded; those of the refinement's loop run once per pass that a replay needs."""
+        shared-memory attribute before capture.  The graph stays this Batch's own, so the
+        refinement is recorded as a loop (eclqr_capture_loop); a capture of run() by the caller
+        records every pass.  Returns the number of kernel launches recorded; those of the
+        loop run once per pass that a replay needs."""
         torch = self.torch
         side = torch.cuda.Stream(self.device)
         side.wait_stream(torch.cuda.current_stream(self.device))
@@ -353,8 +361,12 @@ class Batch:
         torch.cuda.synchronize(self.device)
         before = self.launches()
         graph = torch.cuda.CUDAGraph()
-        with torch.cuda.graph(graph, capture_error_mode="relaxed"):
-            self.run()
+        _check(eclqr_capture_loop(self.h, 1), "eclqr_capture_loop")
+        try:
+            with torch.cuda.graph(graph, capture_error_mode="relaxed"):
+                self.run()
+        finally:
+            eclqr_capture_loop(self.h, 0)
         self.graph = graph
         self.graph_launches = self.launches() - before
         return self.graph_launches
