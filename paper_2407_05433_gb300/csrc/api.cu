@@ -968,6 +968,7 @@ int eclqr_refine(eclqr_handle *h, const double *s0, double *x, double *u, double
     rc = [&]() -> int {
       TRY(prepare(st, first));
       k_refine_loop<<<1, 1, 0, st>>>(cond, h->any, h->opt.kkt_refine, 1);
+      if (cudaPeekAtLastError() != cudaSuccess) return ECLQR_ECUDA;
       const cudaGraphNode_t *deps = nullptr;
       const cudaGraphEdgeData *edges = nullptr;
       size_t ndeps = 0;
@@ -988,7 +989,11 @@ int eclqr_refine(eclqr_handle *h, const double *s0, double *x, double *u, double
       h->in_loop = true;
       int r = pass(h->loop_s, true, true);
       if (r == ECLQR_OK) r = prepare(h->loop_s, 0);
-      if (r == ECLQR_OK) k_refine_loop<<<1, 1, 0, h->loop_s>>>(cond, h->any, h->opt.kkt_refine, 0);
+      if (r == ECLQR_OK) {
+        // without this launch the loop would never end: an unrecorded one fails the capture
+        k_refine_loop<<<1, 1, 0, h->loop_s>>>(cond, h->any, h->opt.kkt_refine, 0);
+        if (cudaPeekAtLastError() != cudaSuccess) r = ECLQR_ECUDA;
+      }
       h->in_loop = false;
       if (cudaStreamEndCapture(h->loop_s, &body) != cudaSuccess) return ECLQR_ECUDA;
       h->launches += 2;
