@@ -315,7 +315,6 @@ __device__ __forceinline__ int riccati_packed(int ld, int j, int k) { return j *
 
 // P and p from raw sums: the block of G from row z0 on, nz states and the offset column, with
 // entry exponents e(z0 + a) + e(z0 + b) (p: e(z0 + a) + e(z0 + nz)).  Brings every diagonal entry to [2^112, 2^114),
-//
 // sets w.P and w.eP, and writes P and p in FP64 where they are given.
 static __device__ __noinline__ void riccati_value(const RiccatiFx w, int nz, int z0, double *Po, int ldo, double *po) {
   const int ld = z0 + nz + 1;
@@ -599,7 +598,8 @@ static __device__ __forceinline__ void riccati_stage(const Group &g, const Ricca
       acc.zero();
       acc.mad(y4, g2);
       const i128 t = acc.value<57>();
-      w.W(k * ldx + j) = fx_split4(t + __mul64hi((long long)(t >> 57) << 6, r << 1));
+      // the offsets (j = kh) may pass the columns' 2^114, so theirs can wrap: their multiplier has no reader
+      w.W(k * ldx + j) = fx_split4(t + __mul64hi((long long)((unsigned long long)(t >> 57) << 6), r << 1));
     }
     team_sync();
     // rows k + 1 .. mu - 1
@@ -706,7 +706,7 @@ static __device__ void riccati_task(const Group &g, int fin, int t, int per_task
     const double *src = crel_cost(g.CS[fin] + (size_t)slot * g.cs_stride, n);
     const int nz = g.CI[fin][(size_t)slot * CI_STRIDE + CI_NA], rv = g.CI[fin][(size_t)slot * CI_STRIDE + CI_ROWS2];
 #pragma unroll 1
-      for (int j = tid; j <= nz; j += TEAM) {
+    for (int j = tid; j <= nz; j += TEAM) {
       int mx = kFxNone;
 #pragma unroll 1
       for (int r = 0; r < rv; r++) mx = max(mx, fx_expo(src[r * ldr + j]));
