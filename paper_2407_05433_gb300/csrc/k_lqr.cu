@@ -564,9 +564,11 @@ static __device__ __forceinline__ void riccati_stage(const Group &g, const Ricca
       const unsigned long long g0 = (unsigned long long)fx_rcp((unsigned long long)(dp >> 50));
       // 2^114 - (dp g0 >> 55), below 2^63: the low 64 bits are all of it
       const unsigned long long lo = (unsigned long long)dp, t = (__umul64hi(lo, g0) << 9) | ((lo * g0) >> 55);
-      // the offsets' column has no bound by the diagonal: where the shift would pass 2^116, its
-      // exponent is raised first
-      const int over = fx_bits(fx_join4(w.G(gk + kh))) + h - 116;
+      // the offsets' column has no bound by the diagonal: where the shift would pass 2^114, its
+      // exponent is raised first.  Then y / sqrt(d 2^(2h)) of the offsets is at most 2^58 for each pivot,
+      // and a later row, whose y / sqrt(d 2^(2h)) over the pivots have squares that sum to its diagonal,
+      // at most 2^114, collects at most sqrt(15) 2^115: below the limbs' 2^118.  (From 2^116 it could pass them.)
+      const int over = fx_bits(fx_join4(w.G(gk + kh))) + h - kFxP;
       if (tid == 0) {
         if (noise) w.G(gk + k) = fx_split4(d);
         w.hp(k) = h;
@@ -598,7 +600,7 @@ static __device__ __forceinline__ void riccati_stage(const Group &g, const Ricca
       acc.zero();
       acc.mad(y4, g2);
       const i128 t = acc.value<57>();
-      // the offsets (j = kh) may pass the columns' 2^114, so theirs can wrap: their multiplier has no reader
+      // the offsets' (j = kh) can wrap: their multiplier has no reader
       w.W(k * ldx + j) = fx_split4(t + __mul64hi((long long)((unsigned long long)(t >> 57) << 6), r << 1));
     }
     team_sync();

@@ -1,6 +1,6 @@
 """The integer Riccati sweep by itself, without the refinement that would hide its errors, and at the ends of its
-range: values whose condition is far beyond FP64's 2^53, curvature below the sweep's resolution, offsets that a
-small pivot carries past the columns' scale.  Against the KKT solution of extended precision."""
+range: values whose condition is far beyond FP64's 2^53, curvature below the sweep's resolution, offsets that
+small pivots carry past the columns' scale.  Against the KKT solution of extended precision."""
 import numpy as np
 import pytest
 
@@ -90,3 +90,20 @@ def test_offsets_that_a_small_pivot_lifts(seed):
     status, _, (ex, eu), e = _errors(_feasible(pb), **RAW)
     size = max(1.0, float(np.max(np.abs(e["u"])) / np.max(np.abs(e["x"]))))
     assert status == 0 and eu <= 1e-9 and ex <= 20 * (n + m) * EPS * size * 8, (ex, eu, size)
+
+
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+@pytest.mark.parametrize("m", [3, 8, 16])
+def test_a_row_that_collects_the_offsets_of_many_small_pivots(m, sign):
+    """R's first m - 1 rows are parallel to 2^-26, their linear costs just below a power of two, and the last row is
+    coupled to every pivot as strongly as a positive definite R allows: its offset grows with each.  u is -R^{-1} r."""
+    k, d = m - 2, 2.0 ** -26 * 1.001
+    R = np.ones((m, m))
+    R[1:-1, 1:-1] += d * np.eye(k)
+    R[-1, -1] = 7.99
+    R[-1, 1:-1] = R[1:-1, -1] = 1.0 + 0.97 * np.sqrt(6.99 * d / k)
+    pb = synth.make_problem(1, 3, 2, m, 0, 0)
+    pb.R[:], pb.B[:], pb.M[:], pb.rv[:] = R, 0.0, 0.0, 0.0
+    pb.rv[:, 1:-1] = 0.9999 * sign
+    status, _, (ex, eu), _ = _errors(_feasible(pb), **RAW)
+    assert status == 0 and ex <= 1e-12 and eu <= m * EPS * np.linalg.cond(R), (ex, eu)
