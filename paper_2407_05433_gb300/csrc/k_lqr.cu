@@ -386,7 +386,9 @@ static __device__ __forceinline__ void riccati_fetch(const Group &g, const Ricca
   }
 }
 
-// Starts the copy of a stage's H and h in the order (v, z, 1), packed rows, into w.H.
+// Starts the copy of a stage's H and h in the order (v, z, 1), packed rows, into w.H: the lower triangles
+// of Rbar and Qbar, those that k_elim's Cholesky found positive definite (the upper ones differ by rounding,
+// and where a Hessian is singular to rounding that is the sign of its smallest eigenvalue).
 static __device__ __forceinline__ void riccati_fetch_h(const Group &g, const RiccatiFx w, const double *ws, int nx, int mu) {
   const int n = g.n, m = g.m, kh = nx + mu, ld = kh + 1;
   const double *Qb = ws + g.ws.Qb, *Mb = ws + g.ws.Mb, *Rb = ws + g.ws.Rb, *qb = ws + g.ws.qb, *rb = ws + g.ws.rb;
@@ -397,8 +399,8 @@ static __device__ __forceinline__ void riccati_fetch_h(const Group &g, const Ric
     const int k = j + idx - row;
     const double *src;
     if (k == kh) src = j < mu ? rb + j : qb + (j - mu);
-    else if (k < mu) src = Rb + j * m + k;
-    else src = j < mu ? Mb + (k - mu) * m + j : Qb + (j - mu) * n + (k - mu);
+    else if (k < mu) src = Rb + k * m + j;
+    else src = j < mu ? Mb + (k - mu) * m + j : Qb + (k - mu) * n + (j - mu);
     copy_async(&w.H(idx), src);
   }
 }
@@ -696,7 +698,7 @@ static __device__ void riccati_task(const Group &g, int fin, int t, int per_task
     for (int idx = tid; idx < nz * (nz + 1); idx += TEAM) {
       const int j = idx / (nz + 1), k = idx - j * (nz + 1);
       if (k < j) continue;
-      const double x = k < nz ? Qb[j * n + k] : qb[j];
+      const double x = k < nz ? Qb[k * n + j] : qb[j];  // the triangle that the convexity test reads
       if (fx_nonfinite(x)) w.bad() = 1;
       w.Gi(riccati_packed(nz + 1, j, k)) = fx_from4(x, w.e(j) + w.e(k));
     }

@@ -1,6 +1,8 @@
 """The integer Riccati sweep by itself, without the refinement that would hide its errors, and at the ends of its
 range: values whose condition is far beyond FP64's 2^53, curvature below the sweep's resolution, offsets that
 small pivots carry past the columns' scale.  Against the KKT solution of extended precision."""
+import os
+
 import numpy as np
 import pytest
 
@@ -107,3 +109,22 @@ def test_a_row_that_collects_the_offsets_of_many_small_pivots(m, sign):
     pb.rv[:, 1:-1] = 0.9999 * sign
     status, _, (ex, eu), _ = _errors(_feasible(pb), **RAW)
     assert status == 0 and ex <= 1e-12 and eu <= m * EPS * np.linalg.cond(R), (ex, eu)
+
+
+@pytest.mark.parametrize("chunk", [50, 7])
+def test_the_sweep_reads_the_triangle_that_was_tested(chunk):
+    """A draw in units up to 2^48 apart (golden/near_singular_units.npz) whose reduced terminal Hessian is singular to
+    rounding: positive definite by the lower triangle, which the convexity test factors, indefinite by the upper
+    one.  Status OK, and the residual at the floor that FP64 sets (8 ulp of every row's |K||w| + |b|)."""
+    g = np.load(os.path.join(os.path.dirname(__file__), "golden", "near_singular_units.npz"))
+    N, n, m = (int(v) for v in g["dims"])
+    pb = synth.ECLQRProblem(N=N, n=n, m=m, **{k: g[k] for k in (
+        "p", "q", "A", "B", "c", "C", "D", "d", "E", "e", "Q", "M", "R", "qv", "rv", "s0")})
+    b = eclqr.Batch([pb], chunk=chunk)
+    try:
+        b.run()
+        (r,) = b.results()
+    finally:
+        b.close()
+    floor = EPS * float(np.max(exact.residual_scale(pb, exact.exact_kkt(pb))))
+    assert r["status"] == 0 and np.isfinite(r["x"]).all() and r["resid"] <= 8 * floor, (r["resid"], floor)
