@@ -23,24 +23,6 @@ __device__ __forceinline__ int team_rank() { return threadIdx.x; }
 #define TEAM ((int)blockDim.x)
 __device__ __forceinline__ void tsync() { __syncthreads(); }
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-  return v;
-}
-
-// arg-max over non-negative values; ties resolve to the lowest index.  The
-// bit pattern of a non-negative double orders like the value, so the
-// comparison runs on the integer pipe.
-__device__ __forceinline__ void warp_argmax(long long &key, int &idx) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    long long k2 = __shfl_xor_sync(kFull, key, o);
-    int i2 = __shfl_xor_sync(kFull, idx, o);
-    if (k2 > key || (k2 == key && i2 < idx)) { key = k2; idx = i2; }
-  }
-}
-
 // The bit pattern of |v| for the integer maximum reductions: non-negative doubles order like their
 // patterns, and a NaN counts as nothing, as in fmax.
 __device__ __forceinline__ unsigned long long abs_key(double v) {
@@ -102,20 +84,14 @@ static __device__ void wgemm(int m, int n, int k, const double *A, int lda, cons
 // ---------------------------------------------------------------------------
 // Householder core shared by the factorizations below.
 //
-// Per-CTA static scratch: one partial dot product per thread, and for column
-// pivoting the running squared norms of the candidate columns with their
-// values at the last exact evaluation and two lists of active columns.  Sized
-// for teams of up to kMaxTeam threads and matrices of up to kMaxCols columns
+// Per-CTA static scratch, for column pivoting: the running squared norms of the
+// candidate columns with their values at the last exact evaluation, the pivot's
+// row and two lists of active columns.  Sized for matrices of up to kMaxCols columns
 // (the header's dimension limits keep every factored matrix at or below
-// 3 * 32 + 64 + 1 = 161 columns).  The static total stays below 10 KB, which
+// 3 * 32 + 64 + 1 = 161 columns).  The static total stays below 8 KB, which
 // the largest dynamic request (219 KB) leaves room for.
 // ---------------------------------------------------------------------------
-constexpr int kMaxTeam = 256;
 constexpr int kMaxCols = 168;
-__device__ __forceinline__ double *hh_part() {
-  __shared__ double part[kMaxTeam];
-  return part;
-}
 __device__ __forceinline__ double *hh_norms() {
   __shared__ double norms[2 * kMaxCols];
   return norms;
