@@ -613,8 +613,8 @@ def run_gpu(args):
 
     # untimed setup: the fewest refinement passes on the KKT residual that leave as many problems
     # under their gate as the library default (8), for one or two reduced passes in the first
-    # solve; a captured step records every pass, so passes that no problem needs still cost their
-    # launches and the sweeps of slow-converging problems
+    # solve; the passes end when no problem takes part, but on this batch a few slow-converging
+    # problems take part in every pass that is allowed, each with the latency of their sweeps
     refine, kkt_refine, kr_trials = autotune_refine(pbs, dev, gates, flush, stream, team_warps=args.team_warps)
     batch = eclqr.Batch(pbs, device=dev, refine=refine, corr_refine=CORR_REFINE, kkt_refine=kkt_refine,
                         team_warps=args.team_warps)

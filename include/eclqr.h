@@ -111,15 +111,18 @@ typedef struct {
   int32_t refine;    /* refinement passes on the reduced LQR KKT residual; default 2          */
   int32_t chunk;     /* stages per scan chunk; 0 = chosen from the horizons, n and the SM count: one
                       * chunk per problem of a group unless its longest horizon exceeds
-                      * min(150, 40 + 8 n) stages by more than n / 2 times the batch's
-                      * stages per SM, else 7 to 64 stages.  A problem that fits one chunk is swept
+                      * min(150, 40 + 8 n) stages by more than max(3, n / 2) times the
+                      * batch's stages per SM, else 7 to 64 stages.  A problem that fits one chunk is swept
                       * once per scan, from its terminal element, with no chunk aggregate */
   int32_t team_warps; /* warps of the CTA that runs one task: 1, 2, 4 or 8 for every kernel;
                        * 0 (default) = per kernel: 4 when a launch has fewer tasks than
                        * SMs; with at least 4 tasks per SM the kernel's measured best for
-                       * the group's n (1 for the per-problem sweeps and the small
-                       * per-stage kernels, 1 or 4 for the stage elimination, 2 or 8 for
-                       * the affine-chain sweep); in between that but at least 2          */
+                       * the group's n (1 for most, 1, 2 or 4 for the stage elimination
+                       * and the Riccati sweep); in between that but at least 2.  The
+                       * Riccati sweep takes 4, or 8 (n >= 12) or 16 (n >= 24) with at
+                       * most two sweeps per SM, whenever it has fewer than 4; the affine
+                       * chains take 1, 2 or 4 by n alone, and in every case one warp
+                       * more, which moves their data                                     */
   int32_t scan_skip;  /* 1 (default): take the shortcut of Sec. 6 (complete algorithm and
                        * complexity) where it applies: a problem without state-only or
                        * terminal rows whose every stage's mixed rows leave no row on x_i
@@ -130,8 +133,8 @@ typedef struct {
                        * refinement workspace and eclqr_refine only computes the residual */
   double refine_tol;  /* eclqr_refine corrects a problem only while its residual exceeds
                        * this; default 5e-10                                              */
-  int32_t riccati_fp32; /* 1: mixed precision -- the square-root Riccati sweep of every
-                       * problem runs in FP32, everything else in FP64 (the domain scan,
+  int32_t riccati_fp32; /* 1: mixed precision -- the Riccati sweep of every problem
+                       * runs in FP32 (in square-root form), everything else in FP64 (the domain scan,
                        * null-space bases and rank decisions, the elimination, rollout,
                        * refinement and multipliers); eclqr_refine then refines in FP64
                        * and redoes in FP64 the problems it leaves above refine_tol.

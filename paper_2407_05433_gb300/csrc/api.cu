@@ -21,10 +21,10 @@ using namespace eclqr;
 namespace {
 
 // dynamic shared memory per task: the 227 KB opt-in limit less room for the
-// static scratch of the team reductions and the Householder core (< 8 KB)
+// static scratch of the team reductions and the Householder core (< 7 KB)
 constexpr int kMaxSmemBytes = 219 * 1024;
-// doubles of static scratch that the multiplier kernels once had: the documented limit on the row
-// counts includes them, so that it stays where it is
+// part of the documented limit on the row counts (eclqr.h), as doubles on top of the multiplier kernels'
+// shared memory: a batch that the limit rejects stays rejected, whatever these kernels use
 constexpr int kHeldScratch = 304;
 constexpr int kTeamWarps = 4;  // default team: one warp per SM sub-partition
 constexpr int kManyTasksPerSm = 4;  // a launch with at least this many tasks per SM takes the table's team
@@ -104,8 +104,8 @@ namespace {
 // them, and needs no CTA barrier.  The entries are the fastest team measured per
 // kernel and state dimension on the 4096-problem uneven batch (each (n, m) group
 // alone, about seven problems per SM) or on 1280 problems of 48 stages.  For example, the
-// chunk up-sweeps of the long horizon (65536 stages in 1024 chunks) take 27 ms with two
-// warps per chunk against 37 with one; the stage elimination takes 2.81 / 3.00 / 4.20 ms with
+// chunk up-sweeps of the long horizon (65536 stages in 1024 chunks) take 32.3 / 22.8 / 22.1 ms
+// with 1 / 2 / 4 warps per chunk at n = 16, 4.5 / 4.5 / 7.5 at n = 8; the stage elimination takes 2.81 / 3.00 / 4.20 ms with
 // 1 / 2 / 4 at n = 16 and four rows a stage (65536 stages), but 3.43 / 3.25 with 1 / 2 at up to seven
 // rows (640 problems), and 5.36 / 3.36 / 2.84 / 3.25 with 1 / 2 / 4 / 8 at n = 32 (160 problems).
 // The affine chains (row warps beside the one that moves the data): 256 problems of 256 stages at
@@ -126,8 +126,8 @@ int team_for(const eclqr_handle *h, const void *kern, int ntasks, int n) {
     return ntasks > 2 * h->sms || n < 12 ? kTeamWarps : n < 24 ? 8 : 16;
   }
   if (ntasks < h->sms) return kTeamWarps;
-  // warps below n1, from n1 and n2 up; with one to four tasks per SM at least two (256 problems of
-  // 256 stages, n = 16: 37 ms with two, 42 with one, 49 with four)
+  // warps below n1, from n1 and n2 up; with one to four tasks per SM at least two (256 problems of 256
+  // stages at n = 16, a whole pass: 12.4 ms with at least one, two or four alike, so the line has no cost)
   static const struct { const void *fn; int warps, n1, warps1, n2, warps2; } table[] = {
       {(const void *)k_riccati_down, 1, 12, 2, 16, 4},
       {(const void *)k_riccati_down_f32, 1},     {(const void *)k_riccati_finish, 1},

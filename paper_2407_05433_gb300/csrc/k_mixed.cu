@@ -1,8 +1,8 @@
 // k_mixed.cu -- the square-root Riccati sweep in FP32 (mixed-precision mode).
 //
-// Same recursion as k_riccati_down (Sec. 6, square-root cost rows; the stage
-// factor L' upper triangular in the QR's column order (v, z)), with every
-// product, reflector and triangular solve in FP32 and the stored factors (P, p,
+// The value function as square-root cost rows (Sec. 6; the stage factor L' upper
+// triangular in the QR's column order (v, z)), where the FP64 mode's k_riccati_down
+// carries P itself in 114-bit integers, with every product, reflector and triangular solve in FP32 and the stored factors (P, p,
 // K, k, chol(H_uu), Phi) widened to FP64.  The rank-revealing parts of the
 // method -- the domain scan, the null-space bases T, Z, the particular solutions
 // t, y and every rank decision -- stay FP64 in the other kernels.  The factors

@@ -43,7 +43,7 @@ struct WsLayout {
   int nu, NH, Pnu, pnu, UA, BU, UC, Ux, ru;
   int LT, lt;   // Cholesky factor L' of the reduced stage Hessian in the order (v, z), upper
                 // triangular (L L' = [Rbar Mbar'; Mbar Qbar]), and L^{-1} [rbar; qbar]
-  int Rv;       // the Riccati QR's rows of the minimiser, (R_vv | R_vz | o_v), ld n + m + 1
+  int Rv;       // the Riccati sweep's rows of the minimiser, (R_vv | R_vz | o_v), ld n + m + 1
   int gv;       // offset of the affine chain's stage map (k_aff_prep, k_resid, k_pcorr), n, right after Phi
   int Hpre;     // the stage's own rows projected onto x_i (k_primal_stage), n x (n + 1)
   int stride;
